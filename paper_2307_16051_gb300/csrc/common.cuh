@@ -80,54 +80,37 @@ constexpr long long kSpinLimit = 1LL << 24;
 
 __device__ __forceinline__ float round_h(float v) { return __half2float(__float2half_rn(v)); }
 
-// fl16(fl32(a / b)) for a binary16 value b != 0 (held in a float) and
-// rb = __frcp_rn(b), with no division and no branch.
-//   q = fl32(a rb) is within 2^-22.9 |a/b| of a/b, hence so is fl32(a/b).
-//   h = fl16(q).  Let m be the binary16 rounding boundary (the midpoint of
-//   two adjacent binary16 values lo < hi) next to q on the side of q away
-//   from h.  If |q - m| > 2^-21 |q|, no boundary separates q from fl32(a/b)
-//   and h is the answer.  Otherwise the answer is decided exactly:
-//   e = |a| - m |b| is exact (m |b| has at most 23 significant bits, and
-//   Sterbenz's lemma applies), and fl32(|a/b|) > m iff e > up |b| / 2,
-//   < m iff e < -dn |b| / 2 (up, dn: the single-precision spacings above and
-//   below m; m has a zero last bit, so single-precision ties go to m), and
-//   = m otherwise, when binary16 rounding of the tie picks the even one of
-//   lo and hi.  The sign is that of q.  NaN and infinity follow q.
-__device__ __forceinline__ float div_round_h(float a, float b, float rb)
+// The multipliers of the binary16 factorisations, l = fl16(fl32(a / u)) for a
+// binary16 pivot u != 0, with no division and no branch.  With y = -1/|u| from
+// the hardware's approximate reciprocal (relative error at most 2^-23) and a
+// given the sign of u (a'),
+//   q = fl(a' y),  e = fl(q |u| + a'),  q' = fl(e y + q)
+// is -fl32(a / u) exactly:
+//   * q is within a few units of -a'/|u|, so e is exact (a 24-bit times an
+//     11-bit significand, cancelled to a few units), and
+//     q + e y = -a'/|u| (1 + d) with |d| < 2^-44;
+//   * a quotient of a 24-bit by an 11-bit significand is never within 2^-36
+//     (relative) of a midpoint of two binary32 values without being one (a' - m |u|
+//     is a multiple of 2^-34 for a 25-bit m), and it is never a midpoint
+//     (that m |u| has more than 24 bits); so q' rounds as the quotient does.
+// Results below binary32's normal range round to a binary16 zero either way.
+// y negative makes the sign of a zero result right: e is then +0.
+__device__ __forceinline__ float rcp_neg_abs(float u)
 {
-    const float q = __fmul_rn(a, rb);
-    const __half h = __float2half_rn(q);
-    const float aq = fabsf(q);
-    const unsigned hb = __half_as_ushort(h) & 0x7fffu;
-    const float ah = __half2float(__ushort_as_half((unsigned short)hb));
-    const unsigned nb = (aq > ah) ? hb + 1u : (hb ? hb - 1u : 0u);
-    const float nf = __half2float(__ushort_as_half((unsigned short)nb));
-    const float m = 0.5f * (ah + nf);
-    const bool near = (aq != 0.0f) && (fabsf(aq - m) <= aq * 0x1p-21f);
-    const float ab = fabsf(b);
-    const float e = __fmaf_rn(-m, ab, fabsf(a));
-    const unsigned mu = __float_as_uint(m);
-    const float up = __fsub_rn(__uint_as_float(mu + 1u), m);
-    const float dn = __fsub_rn(m, __uint_as_float(mu - 1u));
-    const float sup = 0.5f * up * ab, sdn = 0.5f * dn * ab;
-    const unsigned lob = min(hb, nb);
-    const float lo = fminf(ah, nf), hi = fmaxf(ah, nf);
-    const float exact = (e > sup) ? hi : ((-e > sdn) ? lo : ((lob & 1u) ? hi : lo));
-    return copysignf(near ? exact : ah, q);
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(-fabsf(u)));
+    return y;
 }
-
-// The common case of div_round_h alone: fl16(fl32(a rb)), and in *unsure
-// whether a binary16 rounding boundary lies within 2^-20 |q| of q (then the
-// caller must use div_round_h; when *unsure is false the result is exact, by
-// the same argument).
-__device__ __forceinline__ float div_round_h_fast(float a, float rb, bool* unsure)
+// -fl32(a / u), u finite and not zero: us carries u's sign, y = rcp_neg_abs(u), den = |u|
+__device__ __forceinline__ float div_neg(float a, float us, float y, float den)
 {
-    const float q = __fmul_rn(a, rb);
-    const __half h = __float2half_rn(q);
-    const __half lo = __float2half_rn(__fmul_rn(q, 1.0f - 0x1p-20f));
-    const __half hi = __float2half_rn(__fmul_rn(q, 1.0f + 0x1p-20f));
-    *unsure = !(__half_as_ushort(lo) == __half_as_ushort(hi) && __half_as_ushort(h) == __half_as_ushort(lo));
-    return __half2float(h);
+    const float as = __uint_as_float(__float_as_uint(a) ^ (__float_as_uint(us) & 0x80000000u));
+    const float q = __fmul_rn(as, y);
+    return __fmaf_rn(__fmaf_rn(q, den, as), y, q);
+}
+__device__ __forceinline__ float div_round_h(float a, float u)
+{
+    return -round_h(div_neg(a, u, rcp_neg_abs(u), fabsf(u)));
 }
 
 // The sum of part[0 .. n) in index order, by every thread of the block (the

@@ -815,44 +815,59 @@ __global__ void __launch_bounds__(kOffThreads) k_offdiag(S* __restrict__ A, int6
 // padded) and the unrounded pivots a_tt (kStagePivOff floats in).
 constexpr int kStagePivOff = 2 * 128 * 128;
 
-// k_diag_lu16: the diagonal block [K, K+w)^2 (w <= 128), one CTA of 512
-// threads, as a column pipeline.  Warp v owns columns 8v..8v+7 and lane l rows
-// 4l..4l+3, so every thread keeps a 4 x 8 tile in registers.  Warp v first
-// applies, in order k = 0, 1, ..., 8v-1, the updates of the earlier warps'
-// columns as each column's multipliers appear in shared memory (a ready flag
-// per column), then factors its own eight columns: for column t the lanes
-// check |a_it| <= |a_tt| for their rows below t (partial pivoting keeps the
-// diagonal; ties go to the diagonal, which comes first), form
-// l_it = fl16(a_it / fl16(a_tt)), publish them, and update the warp's later
-// columns.  Row k's entries of a warp's columns are rounded to binary16 (U)
-// by that warp when it applies update k.  Every entry takes its updates in
-// increasing k, one binary32 fused multiply-add each, exactly as in
-// right-looking elimination; only the warps' schedule is pipelined, so the
-// critical path is one division and one hand-off per column instead of a
-// block-wide barrier per step.  Finished entries stay in the registers (U on
-// and above the diagonal, L below).  Every wait is bounded: a wait that gives
-// up marks the fast path failed, so the host refactors with interchanges.
-// (The hand-offs use CTA-scope release/acquire on the flags; a fence per
-// column and a clock-based wait cost 1.7x in time.)
+// k_diag_lu16: the diagonal block [K, K+w)^2 (w <= 128) in one CTA, right-looking
+// over blocks of eight columns.  It is bound by its dependent chain (128
+// columns), so the chain runs in one warp and everything else beside it.
+// Step q (C0 = 8 q), between two CTA barriers:
+//   warp 0: the multipliers of the next 32 rows (a row per lane; the diagonal
+//     block's U and pivots are in registers), block q applied to the next
+//     diagonal block, and that block factored in registers (lane r holds
+//     row r; the pivot row by shuffles, about 90 cycles a column);
+//   the others: U's next columns (warp 4, for warp 0's next block) and those
+//     further right, the multipliers of the rows further below, step q-1
+//     published; then (the warps off warp 0's scheduler) block q applied to the
+//     rest of the trailing matrix, four columns of every few rows per thread.
+// The working copy S is binary32 in shared memory; final entries go to Hs as
+// binary16, the multipliers negated (so updates are fused multiply-adds
+// without a sign).  Products use fma.rn.f32.f16 (binary16 x binary16 +
+// binary32, one rounding), which equals the binary32 fused multiply-add of the
+// promoted values and saves the promotions.  Multipliers: div_neg
+// (common.cuh).  Every entry takes its updates in increasing k, one fused
+// multiply-add each, exactly as in right-looking elimination; partial pivoting
+// keeps the diagonal iff |a_it| <= |a_tt| for all rows below (ties go to the
+// diagonal, which comes first), checked on every pre-division value; a pivot
+// that is zero or not finite in binary16 is left to the interchanging path
+// too.  There are no spin waits.
+// Measured (GB300, w = 128, one launch alone): 30.7 us, of which about 20 are the
+// steps and 5 the stage; the former column pipeline (a hand-off between warps
+// per column, 16 warps competing for the issue slots of the chain) took 57 us.
+// NT threads; WMAX = 64 or 128, the largest w.
 constexpr int kD16Threads = 512;
-constexpr size_t kDiag16Smem = 128 * 128 * sizeof(float);
-constexpr int kDiagSpinLimit = 1 << 22;  // polls of a ready flag before a wait gives up
+template <int WMAX>
+struct Diag16 {
+    static constexpr int LD = WMAX + 4;   // floats; LDS.128 of one row per lane is conflict-free
+    static constexpr int HLD = WMAX + 8;  // binary16
+    static constexpr size_t smem = (size_t)WMAX * LD * 4 + (size_t)WMAX * HLD * 2;
+};
+constexpr size_t kDiag16Smem = Diag16<128>::smem;
 
-// Column hand-off inside the CTA: the producer's lane 0 publishes a column
-// with a CTA-scope release store of its ready flag (shared memory); a
-// consumer's lane 0 polls it with CTA-scope acquire loads, at most
-// kDiagSpinLimit times.  (This exact loop shape matters: an equivalent
-// for-loop with the bound test first compiled to a 2.6x slower kernel.)
-__device__ __forceinline__ bool diag_wait(const int* f, int* failp)
+// fl32(a b + c), a and b binary16 (bits)
+__device__ __forceinline__ float fma_h(unsigned short a, unsigned short b, float c)
 {
-    int it = 0;
-    while (true) {
-        int v;
-        asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"((unsigned)__cvta_generic_to_shared(f)) : "memory");
-        if (v) return true;
-        if (*(volatile const int*)failp) return false;
-        if (++it > kDiagSpinLimit) { *(volatile int*)failp = 1; return false; }
-    }
+    float d;
+    asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(d) : "h"(a), "h"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned short h_lo(unsigned v) { return (unsigned short)(v & 0xffffu); }
+__device__ __forceinline__ unsigned short h_hi(unsigned v) { return (unsigned short)(v >> 16); }
+__device__ __forceinline__ unsigned short h_bits(float v) { return __half_as_ushort(__float2half_rn(v)); }
+__device__ __forceinline__ float h_val(unsigned short v) { return __half2float(__ushort_as_half(v)); }
+__device__ __forceinline__ unsigned h_pack(unsigned short lo, unsigned short hi) { return (unsigned)lo | ((unsigned)hi << 16); }
+// entry e (0..7, a constant after unrolling) of eight packed binary16 values
+__device__ __forceinline__ unsigned short h_at(const uint4& v, int e)
+{
+    const unsigned w = (e < 2) ? v.x : (e < 4) ? v.y : (e < 6) ? v.z : v.w;
+    return (e & 1) ? h_hi(w) : h_lo(w);
 }
 
 // Eight consecutive entries (16-byte aligned) as binary32, and back: binary16
@@ -883,195 +898,290 @@ __device__ __forceinline__ void store8(float* p, const float* v)
     reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-// PUB: also publish each finished column t to pub[t * 128 + i] as the 64-bit
-// word {epoch, value} (U above the diagonal, the unrounded pivot on it, the
-// multipliers below), for the streaming off-diagonal solves of k_panel16.
-template <bool PUB = false, typename S = __half>
-__device__ __forceinline__ void diag_lu16_body(S* __restrict__ A, int64_t lda, int K, int w,
+// The published copy of a factored diagonal block (k_panel16): 64-bit words
+// {epoch, two binary16 values}; a word is its own ready flag.
+//   word k * 64 + e / 2, e > k even:           u_ke, u_k(e+1)
+//   word kPubL + k * 64 + e / 2, e > k even:   -l_ek, -l_(e+1)k
+//   word kPubP + t:                            the unrounded pivot a_tt (binary32)
+// Step s publishes U's rows 8(s-1)..8(s-1)+7 right of block column s-1, the
+// diagonal 8 x 8 block s, its pivots, and the multipliers of block column s:
+// what the streaming rows and columns need for their own step s.
+constexpr int kPubL = 128 * 64;
+constexpr int kPubP = 2 * 128 * 64;
+constexpr size_t kPubWords = (size_t)kPubP + 128;
+
+__device__ __forceinline__ void pub_store2(unsigned long long* dst, unsigned epoch, unsigned v0, unsigned v1)
+{
+    const unsigned long long t = (unsigned long long)epoch << 32;
+    asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(dst), "l"(t | v0), "l"(t | v1) : "memory");
+}
+
+// One warp per k (k = 0..7, warp v of 8): Hs and rc hold block columns <= s and U's rows < 8 s.
+template <int HLD>
+__device__ __forceinline__ void diag16_publish(int s, int w8, const unsigned short* Hs, const float4* rc,
+                                               unsigned long long* pub, unsigned epoch, int v, int lane)
+{
+    const int C = 8 * s, k = C + v, e = C + 4 * lane;
+    if (e < w8) {
+        const unsigned short* h = Hs + e * HLD + k;
+        pub_store2(pub + kPubL + k * 64 + (e >> 1), epoch, h_pack(h[0], h[HLD]), h_pack(h[2 * HLD], h[3 * HLD]));
+        if (s > 0) {
+            const uint2 u = *reinterpret_cast<const uint2*>(Hs + (k - 8) * HLD + e);
+            pub_store2(pub + (k - 8) * 64 + (e >> 1), epoch, u.x, u.y);
+        }
+    }
+    if (lane < 2) {
+        const uint2 u = *reinterpret_cast<const uint2*>(Hs + k * HLD + e);
+        pub_store2(pub + k * 64 + (e >> 1), epoch, u.x, u.y);
+    } else if (lane == 2 && v < 4) {
+        pub_store2(pub + kPubP + C + 2 * v, epoch, __float_as_uint(rc[C + 2 * v].z), __float_as_uint(rc[C + 2 * v + 1].z));
+    }
+}
+
+// PUB: also publish the block as it is factored, for the streaming solves of
+// k_panel16.  stage (may be null): U11, L11^T and the pivots for k_offdiag16.
+template <bool PUB = false, typename S_ = __half, int WMAX = 128, int NT = kD16Threads>
+__device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, int K, int w,
                                                int* __restrict__ ipiv, int* __restrict__ flag,
                                                float* __restrict__ stage,
                                                unsigned long long* __restrict__ pub = nullptr, unsigned epoch = 0)
 {
     if (*(volatile int*)flag) return;
-    extern __shared__ __align__(16) float lsh[];  // lsh[t * 128 + i] = l_it (0 for i <= t)
-    __shared__ int rdy[128];
-    __shared__ int fail;
-    __shared__ float pvs[128];  // unrounded pivots, copied to the stage at the end
-    const int tid = threadIdx.x, lane = tid & 31, v = tid >> 5;
-    const int r0 = 4 * lane, C0 = 8 * v;
-    const int wp = (w + 31) & ~31;
+    using G = Diag16<WMAX>;
+    constexpr int LD = G::LD, HLD = G::HLD, NW = NT / 32, NU = 24 * NW;  // NU: threads of the warps off scheduler 0
+    constexpr int RW = WMAX / 32;  // warps 0..RW-1 take the rows below a block, warps 4..RW+3 the columns right of it
+    static_assert(!PUB || NW == 16, "eight publishing warps");
+    extern __shared__ __align__(16) float lsh[];
+    float* S = lsh;                                                            // S[i * LD + j]: the working copy
+    unsigned short* Hs = reinterpret_cast<unsigned short*>(S + WMAX * LD);     // U, and L negated
+    __shared__ float4 rc[WMAX];  // per pivot: rcp_neg_abs, |u|, the unrounded value
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int w8 = (w + 7) & ~7, nq = w8 >> 3;
     const bool vec = (w % 8 == 0) && ((((uintptr_t)(A + (int64_t)K * lda + K)) & 15) == 0) && (lda % 8 == 0);
-    if (tid < 128) rdy[tid] = 0;
-    if (tid == 0) fail = 0;
-    float a[4][8];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int i = r0 + r;
-        const S* src = A + (int64_t)(K + min(i, w - 1)) * lda + K + C0;
-        if (vec && i < w && C0 + 8 <= w) {
-            load8(src, a[r]);
+    // load, eight columns per thread, padded with the identity to w8
+    for (int p = tid; p < w8 * nq; p += NT) {
+        const int i = p / nq, C = 8 * (p - i * nq);
+        const S_* src = A + (int64_t)(K + min(i, w - 1)) * lda + K + C;
+        float v[8];
+        if (vec) {
+            load8(src, v);
         } else {
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                const int j = C0 + c;
-                a[r][c] = (i < w && j < w) ? ld_elem(src + c) : ((i == j) ? 1.0f : 0.0f);
+                const int j = C + c;
+                v[c] = (i < w && j < w) ? ld_elem(src + c) : ((i == j) ? 1.0f : 0.0f);
             }
         }
+        store8(S + i * LD + C, v);
     }
     __syncthreads();
-    float* PV = stage + kStagePivOff;
-    bool bad = false, alive = true;
-    if (C0 < w) {
-        // the earlier warps' columns, in order
-        for (int k0 = 0; k0 < C0 && alive; k0 += 4) {
+    bool bad = false;
+    const int r = lane & 7;
+    const int pubv = wid - 8;  // warps 8..15 publish
+    const bool pubw = wid >= 8;
+    float d[8];  // warp 0, lane r < 8: row r of the diagonal block (the other lanes' values are not used)
+    if (wid == 0) {
+        *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(S + r * LD);
+        *reinterpret_cast<float4*>(d + 4) = *reinterpret_cast<const float4*>(S + r * LD + 4);
+    }
+    for (int q = 0; q < nq; ++q) {
+        const int C0 = 8 * q, C1 = C0 + 8;
+        unsigned um[8][4];            // warp 0: U's rows of the diagonal block, packed from the diagonal on
+        float cp[8], cy[8], cu[8];    // and its pivots, rcp_neg_abs, |u|
+        if (wid == 0) {
+            unsigned hw[4];  // row r's multipliers, packed
+            unsigned viol = 0;
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const int k = k0 + kk;  // row k is register row kk of lane k / 4
-                int ok = 1;
-                if (lane == 0) ok = diag_wait(&rdy[k], &fail);
-                __syncwarp();
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) {
-                    alive = false;
-                    break;
+            for (int k = 0; k < 8; ++k) {
+                // the pivot row's shuffles run beside the division
+                const float p = __shfl_sync(0xffffffffu, d[k], k);
+                float us[8];
+                us[k] = p;
+#pragma unroll
+                for (int e = k + 1; e < 8; ++e) us[e] = __shfl_sync(0xffffffffu, d[e], k);
+                const float ut = round_h(p), y = rcp_neg_abs(ut);
+#pragma unroll
+                for (int e = k & ~1; e < 8; e += 2) {
+                    const __half2 v = __floats2half2_rn(e < k ? 0.0f : us[e], us[e + 1]);
+                    um[k][e / 2] = *reinterpret_cast<const unsigned*>(&v);
                 }
-                const float4 l4 = *reinterpret_cast<const float4*>(&lsh[k * 128 + r0]);
-                const float lk[4] = {l4.x, l4.y, l4.z, l4.w};
-                float u[8];
+                cp[k] = p;
+                cy[k] = y;
+                cu[k] = fabsf(ut);
+                const unsigned short l = h_bits(div_neg(d[k], p, y, cu[k]));
+                if (!(fabsf(d[k]) <= fabsf(p))) viol |= 1u << k;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) u[c] = round_h(__shfl_sync(0xffffffffu, a[kk][c], k >> 2));
-                if (lane == (k >> 2)) {
+                for (int e = k + 1; e < 8; ++e)
+                    d[e] = fma_h(l, (e & 1) ? h_hi(um[k][e / 2]) : h_lo(um[k][e / 2]), d[e]);
+                rc[C0 + k] = make_float4(y, cu[k], p, 0.0f);
+                unsigned row[4];  // row k is final in lane k: its multipliers, then U
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) a[kk][c] = u[c];
+                for (int e = 0; e < 4; ++e) row[e] = 2 * e < k ? hw[e] : um[k][e];
+                if (k & 1) {
+                    hw[k / 2] |= (unsigned)l << 16;
+                    row[k / 2] = (um[k][k / 2] & 0xffff0000u) | (hw[k / 2] & 0xffffu);
+                } else {
+                    hw[k / 2] = l;
                 }
+                if (lane == k)
+                    *reinterpret_cast<uint4*>(Hs + (C0 + k) * HLD + C0) = make_uint4(row[0], row[1], row[2], row[3]);
+            }
+            // rows below row k (lane r > k)
+            if (lane < 8 && (viol & ((1u << r) - 1u))) bad = true;
+        } else if ((wid & 3) && q > 0) {
+            // block q-1 applied right of and below itself, but for the diagonal block (warp 0's)
+            const int B0 = C0 - 8, n4 = (w8 - C0) >> 2, t = ((wid >> 2) * 3 + (wid & 3) - 1) * 32 + lane;
+            float rn4;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rn4) : "f"((float)n4));
+            const int sl = (int)(((float)t + 0.5f) * rn4), ns = (int)(((float)NU + 0.5f) * rn4);
+            const int J = C0 + 4 * (t - sl * n4);
+            if (sl < ns) {
+                unsigned short u[8][4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    if (r0 + r > k) {
+                for (int k = 0; k < 8; ++k) {
+                    const uint2 v = *reinterpret_cast<const uint2*>(Hs + (B0 + k) * HLD + J);
+                    u[k][0] = h_lo(v.x); u[k][1] = h_hi(v.x); u[k][2] = h_lo(v.y); u[k][3] = h_hi(v.y);
+                }
+#pragma unroll 2
+                for (int i = C0 + sl; i < w8; i += ns) {
+                    if (i < C1 && J < C1) continue;
+                    float* Si = S + i * LD + J;
+                    float4 v = *reinterpret_cast<const float4*>(Si);
+                    const uint4 L = *reinterpret_cast<const uint4*>(Hs + i * HLD + B0);
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) a[r][c] = fmaf(-lk[r], u[c], a[r][c]);
+                    for (int k = 0; k < 8; ++k) {
+                        const unsigned short l = h_at(L, k);
+                        v.x = fma_h(l, u[k][0], v.x);
+                        v.y = fma_h(l, u[k][1], v.y);
+                        v.z = fma_h(l, u[k][2], v.z);
+                        v.w = fma_h(l, u[k][3], v.w);
                     }
+                    *reinterpret_cast<float4*>(Si) = v;
+                }
             }
         }
-        // this warp's own columns
+        __syncthreads();
+        if (PUB && pubw && q > 0) diag16_publish<HLD>(q - 1, w8, Hs, rc, pub, epoch, pubv, lane);
+        if (C1 >= w8) break;
+        if (wid == 0) {
+            // row C1 + lane, with the diagonal block's U and pivots in registers
+            const int i = min(C1 + lane, w8 - 1);
+            const float* Si = S + i * LD + C0;
+            float x[8];
+            *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(Si);
+            *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(Si + 4);
+            unsigned short h[8];
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-            const int t = C0 + kk;
-            if (alive && t < w) {
-                const int src = t >> 2;  // row t is register row kk & 3 of lane t / 4
-                const float p = __shfl_sync(0xffffffffu, a[kk & 3][kk], src);
-                const float ut = round_h(p);
-                const float rut = __frcp_rn(ut);
-                float lv[4];
-                bool unsure = false;
+            for (int k = 0; k < 8; ++k) {
+                h[k] = h_bits(div_neg(x[k], cp[k], cy[k], cu[k]));
+                bad |= !(fabsf(x[k]) <= fabsf(cp[k]));
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    bool u = false;
-                    lv[r] = div_round_h_fast(a[r][kk], rut, &u);
-                    unsure |= u && (r0 + r > t);
-                }
-                if (__any_sync(0xffffffffu, unsure)) {  // rare: decide the boundary cases exactly
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) lv[r] = div_round_h(a[r][kk], ut, rut);
-                }
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    if (r0 + r > t) {
-                        if (!(fabsf(a[r][kk]) <= fabsf(p))) bad = true;
-                        a[r][kk] = lv[r];
-                    } else {
-                        lv[r] = 0.0f;
-                    }
-                }
-                if (lane == src) {
-                    a[kk & 3][kk] = ut;
-                    pvs[t] = p;
-                    if (!(ut != 0.0f)) bad = true;  // zero pivot: info is the interchanging path's
-                }
-                *reinterpret_cast<float4*>(&lsh[t * 128 + r0]) = make_float4(lv[0], lv[1], lv[2], lv[3]);
-                __syncwarp();
-                if (lane == 0) asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" :: "r"((unsigned)__cvta_generic_to_shared(&rdy[t])), "r"(1) : "memory");
-                if constexpr (PUB) {
-                    // column t is final: U entries (rounded) above the diagonal, p on it, l below
-                    unsigned long long wv[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const int i = r0 + r;
-                        const float v = (i < t) ? a[r][kk] : ((i == t) ? p : lv[r]);
-                        wv[r] = ((unsigned long long)epoch << 32) | __float_as_uint(v);
-                    }
-                    unsigned long long* dst = pub + t * 128 + r0;
-                    asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(dst), "l"(wv[0]), "l"(wv[1]) : "memory");
-                    asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(dst + 2), "l"(wv[2]), "l"(wv[3]) : "memory");
-                }
-                float u[8];
-#pragma unroll
-                for (int c = kk + 1; c < 8; ++c) u[c] = round_h(__shfl_sync(0xffffffffu, a[kk & 3][c], src));
-                if (lane == src) {
-#pragma unroll
-                    for (int c = kk + 1; c < 8; ++c) a[kk & 3][c] = u[c];
-                }
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    if (r0 + r > t) {
-#pragma unroll
-                        for (int c = kk + 1; c < 8; ++c) a[r][c] = fmaf(-lv[r], u[c], a[r][c]);
-                    }
+                for (int e = k + 1; e < 8; ++e)
+                    x[e] = fma_h(h[k], (e & 1) ? h_hi(um[k][e / 2]) : h_lo(um[k][e / 2]), x[e]);
             }
+            if (C1 + lane < w8)
+                *reinterpret_cast<uint4*>(Hs + i * HLD + C0) =
+                    make_uint4(h_pack(h[0], h[1]), h_pack(h[2], h[3]), h_pack(h[4], h[5]), h_pack(h[6], h[7]));
+            __syncwarp();
+            asm volatile("bar.arrive 2, %0;" ::"n"(NT) : "memory");
+            asm volatile("bar.sync 3, 64;" ::: "memory");  // U's next columns (warp 4)
+            const float* Sd = S + (C1 + r) * LD + C1;
+            *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(Sd);
+            *reinterpret_cast<float4*>(d + 4) = *reinterpret_cast<const float4*>(Sd + 4);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint4 U = *reinterpret_cast<const uint4*>(Hs + (C0 + k) * HLD + C1);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) d[e] = fma_h(h[k], h_at(U, e), d[e]);
+            }
+        } else {
+            const int F0 = C1 + 32;  // first row below and column right that are not warp 0's and warp 4's
+            if (wid >= 1 && wid < RW) {
+                const int i = F0 + (wid - 1) * 32 + lane;
+                if (i < w8) {
+                    float x[8];
+                    const float* Si = S + i * LD + C0;
+                    *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(Si);
+                    *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(Si + 4);
+                    unsigned short h[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const uint4 U = *reinterpret_cast<const uint4*>(Hs + (C0 + k) * HLD + C0);
+                        const float4 c = rc[C0 + k];
+                        bad |= !(fabsf(x[k]) <= fabsf(c.z));
+                        h[k] = h_bits(div_neg(x[k], c.z, c.x, c.y));
+#pragma unroll
+                        for (int e = k + 1; e < 8; ++e) x[e] = fma_h(h[k], h_at(U, e), x[e]);
+                    }
+                    *reinterpret_cast<uint4*>(Hs + i * HLD + C0) =
+                        make_uint4(h_pack(h[0], h[1]), h_pack(h[2], h[3]), h_pack(h[4], h[5]), h_pack(h[6], h[7]));
+                }
+            } else if (wid >= 4 && wid < 4 + RW) {
+                const int j = (wid == 4 ? C1 : F0 + (wid - 5) * 32) + lane;  // a column right
+                if (j < w8) {
+                    float x[8];
+                    uint4 L[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        x[k] = S[(C0 + k) * LD + j];
+                        L[k] = *reinterpret_cast<const uint4*>(Hs + (C0 + k) * HLD + C0);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const unsigned short u = h_bits(x[k]);
+                        Hs[(C0 + k) * HLD + j] = u;
+#pragma unroll
+                        for (int e = k + 1; e < 8; ++e) x[e] = fma_h(h_at(L[e], k), u, x[e]);
+                    }
+                }
+                __syncwarp();
+                if (wid == 4) asm volatile("bar.arrive 3, 64;" ::: "memory");
+            }
+            __syncwarp();
+            asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
         }
     }
-    if (!alive) bad = true;
+    if (PUB && pubw) diag16_publish<HLD>(nq - 1, w8, Hs, rc, pub, epoch, pubv, lane);
+    if (tid < w8) bad |= !(rc[tid].y > 0.0f && rc[tid].y <= 65504.0f);
     if (__syncthreads_or(bad)) {
         if (tid == 0) atomicOr(flag, 1);
         return;
     }
-    // the factors (binary16) to A, U11 and L11^T (binary32, identity / zero padded to wp) to the stage
+    // the factors to A (the sign of L's entries restored)
+    for (int p = tid; p < w * nq; p += NT) {
+        const int i = p / nq, C = 8 * (p - i * nq);
+        const uint4 h = *reinterpret_cast<const uint4*>(Hs + i * HLD + C);
+        unsigned hw[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int i = r0 + r;
-        if (i < w && C0 < w) {
-            S* dst = A + (int64_t)(K + i) * lda + K + C0;
-            if (vec && C0 + 8 <= w) {
-                store8(dst, a[r]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (C0 + c < w) st_elem(dst + c, a[r][c]);
+        for (int c = 0; c < 8; c += 2) {
+            if (C + c < i) hw[c / 2] ^= 0x8000u;
+            if (C + c + 1 < i) hw[c / 2] ^= 0x80000000u;
+        }
+        S_* dst = A + (int64_t)(K + i) * lda + K + C;
+        if constexpr (std::is_same<S_, __half>::value) {
+            if (vec) {
+                *reinterpret_cast<uint4*>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                continue;
             }
         }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (C + c < w) st_elem(dst + c, h_val((c & 1) ? h_hi(hw[c / 2]) : h_lo(hw[c / 2])));
     }
-    float* SU = stage;
-    float* SL = stage + wp * wp;
-    if (C0 < wp) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int i = r0 + r;
-            if (i >= wp) continue;
-            float uu[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int j = C0 + c;
-                uu[c] = (i < w && j < w) ? ((j >= i) ? a[r][c] : 0.0f) : ((i == j) ? 1.0f : 0.0f);
-            }
-            *reinterpret_cast<float4*>(&SU[i * wp + C0]) = make_float4(uu[0], uu[1], uu[2], uu[3]);
-            *reinterpret_cast<float4*>(&SU[i * wp + C0 + 4]) = make_float4(uu[4], uu[5], uu[6], uu[7]);
+    if (stage) {
+        // U11 and L11^T (binary32, identity / zero padded to wp) and the pivots
+        const int wp = (w + 31) & ~31;
+        float* SU = stage;
+        float* SL = stage + wp * wp;
+        for (int p = tid; p < wp * wp; p += NT) {
+            const int i = p / wp, j = p - i * wp;
+            SU[p] = (i < w && j < w) ? (j >= i ? h_val(Hs[i * HLD + j]) : 0.0f) : (i == j ? 1.0f : 0.0f);
+            SL[p] = (i < w && j < w && j > i) ? h_val(Hs[j * HLD + i] ^ 0x8000u) : 0.0f;
         }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int j = C0 + c;
-            float ll[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int i = r0 + r;
-                ll[r] = (i < w && j < w && i > j) ? a[r][c] : 0.0f;
-            }
-            if (r0 < wp) *reinterpret_cast<float4*>(&SL[j * wp + r0]) = make_float4(ll[0], ll[1], ll[2], ll[3]);
-        }
+        if (tid < w) stage[kStagePivOff + tid] = rc[tid].z;
     }
-    if (tid < w) { ipiv[K + tid] = K + tid; PV[tid] = pvs[tid]; }
+    if (tid < w) ipiv[K + tid] = K + tid;
 }
-
-
-
 
 template <typename S>
 __global__ void __launch_bounds__(kD16Threads, 1) k_diag_lu16(S* __restrict__ A, int64_t lda, int K, int w,
@@ -1082,137 +1192,81 @@ __global__ void __launch_bounds__(kD16Threads, 1) k_diag_lu16(S* __restrict__ A,
 }
 
 // k_panel16: the diagonal block and the off-diagonal solves of one panel in
-// one launch.  One CTA factors the diagonal block (the column pipeline above)
-// and publishes every finished column t as {epoch, value} words; the other
-// CTAs stream behind it, one step per published column:
-//   row CTAs (256 rows of L21 each): row i at step t forms
-//     x_it - sum_{k<t} l_ik u_kt (the sum in increasing k, one fused
-//     multiply-add per term) from its own multipliers and U's column t, checks
-//     it against the unrounded pivot and forms l_it = fl16(x / u_tt);
-//   column CTAs (256 columns of U12 each): column j at step t forms
-//     u_tj = fl16(a_tj - sum_{k<t} l_tk u_kj) from its own U entries and row t
-//     of L11 (entry t of the published columns 0..t-1).
-// Every entry takes the same fused multiply-adds in the same order as in the
-// right-looking solves of k_offdiag16, so the results are bitwise those of
-// k_diag_lu16 followed by k_offdiag16; only the schedule differs (the
-// off-diagonal chains run one column behind the diagonal block instead of
-// after it).  A published word is its own ready flag (the epoch is unique per
-// launch and the buffer is cleared before each factorisation), so the
-// producer needs no fence.  Each CTA keeps its rows' (columns') 128 values in
-// shared memory; every wait is bounded and also gives up when the fast path
-// has been abandoned.  The CTAs' roles follow the order they start in (see
-// k_panel16), so no co-residency is needed.
+// one launch.  One CTA factors the diagonal block (above) and publishes each
+// block column of eight as it is finished; the other CTAs stream behind it,
+// one step per block column: a CTA owns up to 256 rows of L21 or columns of
+// U12 ("lines"), their not-yet-solved entries X in binary32 in shared memory.
+// At step q
+//   * a solver thread per line applies block q-1 to its block q (64 fused
+//     multiply-adds), and solves it: for a row, l_it = fl16(x_it / u_tt) with
+//     the pivot check; for a column, u_tj = fl16(x_tj);
+//   * the helper warps apply block q-1 to the lines' blocks q+1, q+2, ...;
+//   * two warps fetch the published words of later steps into M (binary16,
+//     M[k][e] = u_ke for rows, -l_ek for columns), an mbarrier per step;
+// and one barrier of the solvers and helpers joins them.  So what is left
+// after the last published block is one block solve: a step of the stream
+// (about 500 cycles) is shorter than a step of the diagonal block, and the
+// launch takes the diagonal block's time plus a tail of one step (N = 4096:
+// 36.6 us a panel on average, 67.9 us with the column pipeline and left-looking
+// streams).  Eight
+// lines' multipliers of a solved block overwrite the first half of its place
+// in X.  Every entry takes its fused multiply-adds in increasing k, so the
+// results are bitwise those of k_diag_lu16 followed by k_offdiag16.  Every
+// wait is bounded and also ends when the fast path has been abandoned: the
+// warps then run their steps without waiting, so no barrier is missed.
 constexpr int kPnlThreads = 512;
-constexpr int kPnlRows = 256;   // at most this many rows (columns) per streaming CTA: one thread each
-constexpr int kPnlFetchW = 14;  // warps 14 and 15 fetch the published columns (even / odd t)
-constexpr int kPnlLd = 132;     // padded stride of the per-thread histories and the column cache (floats)
-constexpr size_t kPnlSmem = (size_t)kPnlRows * kPnlLd * 4 + (size_t)128 * kPnlLd * 4 + 128 * 8;
+constexpr int kPnlRows = 256;   // at most this many lines per streaming CTA
+constexpr int kPnlFetchW = 14;  // warps 14 and 15 fetch the published words
+constexpr int kPnlXld = 132;    // floats
+constexpr int kPnlMld = 136;    // binary16
+constexpr size_t kPnlSmem = (size_t)kPnlRows * kPnlXld * 4 + (size_t)128 * kPnlMld * 2 + 128 * 4 + 16 * 8;
+static_assert(kPnlSmem >= kDiag16Smem, "the diagonal block's CTA uses the same launch");
 constexpr long long kPnlSpin = 1LL << 22;
 
-// Fetch warp: copy published column t (all 128 entries, lane l: entries 4l..4l+3)
-// into the CTA's cache once its words carry this launch's epoch.  row_major:
-// cache[e * kPnlLd + t] (row e of the panel, column t), else cache[t * kPnlLd + e].
-__device__ __forceinline__ bool pnl_fetch(const unsigned long long* pub, int t, unsigned epoch, const int* flag,
-                                          float* cache, bool row_major, const int* gave_up)
+// Fetch lane: one pair of published words (16 bytes) once both carry this launch's epoch.
+__device__ __forceinline__ bool pnl_fetch2(const unsigned long long* q, unsigned epoch, const int* flag,
+                                           const int* gave_up, unsigned& v0, unsigned& v1)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long* q = pub + t * 128 + 4 * lane;
     for (long long it = 0; it < kPnlSpin; ++it) {
-        unsigned long long v0, v1, v2, v3;
-        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(v0), "=l"(v1) : "l"(q) : "memory");
-        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(v2), "=l"(v3) : "l"(q + 2) : "memory");
-        const bool ok = (unsigned)(v0 >> 32) == epoch && (unsigned)(v1 >> 32) == epoch &&
-                        (unsigned)(v2 >> 32) == epoch && (unsigned)(v3 >> 32) == epoch;
-        if (__all_sync(0xffffffffu, ok)) {
-            const float f[4] = {__uint_as_float((unsigned)v0), __uint_as_float((unsigned)v1),
-                                __uint_as_float((unsigned)v2), __uint_as_float((unsigned)v3)};
-            if (row_major) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) cache[(4 * lane + r) * kPnlLd + t] = f[r];
-            } else {
-                *reinterpret_cast<float4*>(cache + t * kPnlLd + 4 * lane) = make_float4(f[0], f[1], f[2], f[3]);
-            }
+        unsigned long long a, b;
+        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(q) : "memory");
+        if ((unsigned)(a >> 32) == epoch && (unsigned)(b >> 32) == epoch) {
+            v0 = (unsigned)a;
+            v1 = (unsigned)b;
             return true;
         }
         if ((it & 63) == 63 && (*(volatile const int*)flag || *(volatile const int*)gave_up)) return false;
-        __nanosleep(32);
     }
     return false;
 }
 
-__device__ __forceinline__ bool pnl_wait_ready(uint32_t bar, const int* gave_up)
+__device__ __forceinline__ void pnl_wait_ready(uint32_t bar, int* gave_up)
 {
+    if (*(volatile int*)gave_up) return;
     for (long long it = 0; it < kPnlSpin; ++it) {
         uint32_t done;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done)
                      : "r"(bar)
                      : "memory");
-        if (done) return true;
-        if (*(volatile const int*)gave_up) return false;
+        if (done || *(volatile int*)gave_up) return;
     }
-    return false;
+    *(volatile int*)gave_up = 1;
 }
 
-// Steps t .. t+NB-1 of one streaming row (column) at once: each history
-// value h[k], k < t, is loaded once for the NB dot products (shared-memory
-// traffic / NB), then the NB x NB tail in order.  Every entry still takes its
-// fused multiply-adds in increasing k.  c: the cache rows (ROWS: U's columns,
-// else L11's rows), c + j * kPnlLd the one for step t + j.
-template <bool ROWS, int NB>
-__device__ __forceinline__ void pnl_steps(float* __restrict__ h, const float* __restrict__ c, int t, bool* bad)
+// x[e] += h_k M[k][e], k = 0..7 in order: block b's finished eight (hist) applied to eight later entries
+__device__ __forceinline__ void pnl_apply(const uint4& hist, const unsigned short* __restrict__ M, float (&x)[8])
 {
-    float acc[NB];
 #pragma unroll
-    for (int j = 0; j < NB; ++j) acc[j] = h[t + j];
-    int k = 0;
-#pragma unroll 4
-    for (; k + 4 <= t; k += 4) {
-        const float4 l4 = *reinterpret_cast<const float4*>(h + k);
+    for (int k = 0; k < 8; ++k) {
+        const uint4 m = *reinterpret_cast<const uint4*>(M + k * kPnlMld);
+        const unsigned short h = h_at(hist, k);
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            const float4 c4 = *reinterpret_cast<const float4*>(c + j * kPnlLd + k);
-            acc[j] = fmaf(-l4.x, c4.x, acc[j]);
-            acc[j] = fmaf(-l4.y, c4.y, acc[j]);
-            acc[j] = fmaf(-l4.z, c4.z, acc[j]);
-            acc[j] = fmaf(-l4.w, c4.w, acc[j]);
-        }
-    }
-    for (; k < t; ++k) {
-        const float lk = h[k];
-#pragma unroll
-        for (int j = 0; j < NB; ++j) acc[j] = fmaf(-lk, c[j * kPnlLd + k], acc[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-#pragma unroll
-        for (int jj = 0; jj < j; ++jj) acc[j] = fmaf(-h[t + jj], c[j * kPnlLd + t + jj], acc[j]);
-        if (ROWS) {
-            const float p = c[j * kPnlLd + t + j];
-            const float ut = round_h(p);
-            if (!(fabsf(acc[j]) <= fabsf(p))) *bad = true;
-            h[t + j] = div_round_h(acc[j], ut, __frcp_rn(ut));
-        } else {
-            h[t + j] = round_h(acc[j]);
-        }
+        for (int e = 0; e < 8; ++e) x[e] = fma_h(h, h_at(m, e), x[e]);
     }
 }
 
-__device__ __forceinline__ bool pnl_test_ready(uint32_t bar)
-{
-    uint32_t done;
-    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(done)
-                 : "r"(bar)
-                 : "memory");
-    return done != 0;
-}
-
-// One streaming CTA: ROWS = rows of L21 (cache = U's columns, cache[t][k] = u_kt,
-// entry t = the unrounded pivot), else columns of U12 (cache = L11 by rows,
-// cache[t][k] = l_tk).  Threads 0..255 each own one row (column) and its
-// 128-value history; warps 14 and 15 fetch the published columns; column t
-// is signalled through ready[t] (an mbarrier per column, used once).
+// One streaming CTA: ROWS = rows of L21, else columns of U12; rpc lines (a multiple of 32).
 template <bool ROWS, typename S = __half>
 __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, int K, int w, int N, int blk,
                                                int rpc, __half* __restrict__ Ut, int ldut, int ut_col0, int ut_k0,
@@ -1220,72 +1274,114 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
                                                unsigned epoch, unsigned* __restrict__ err)
 {
     extern __shared__ __align__(16) float psm[];
-    float* H = psm;                          // H[r * kPnlLd + t]: a, replaced by l (rows) / u (columns) at step t
-    float* Cc = psm + kPnlRows * kPnlLd;     // the published columns
-    uint64_t* ready = reinterpret_cast<uint64_t*>(Cc + 128 * kPnlLd);
+    float* X = psm;                                                                   // X[line * kPnlXld + t]
+    unsigned short* M = reinterpret_cast<unsigned short*>(X + kPnlRows * kPnlXld);    // M[k * kPnlMld + e]
+    float* pv = reinterpret_cast<float*>(M + 128 * kPnlMld);                          // unrounded pivots (rows)
+    uint64_t* ready = reinterpret_cast<uint64_t*>(pv + 128);
     __shared__ int gave_up;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int idx = K + w + blk * rpc + tid;  // row (ROWS) or column of this thread
-    const bool mine = tid < rpc, live = mine && idx < N;
-    float* h = H + (mine ? tid : 0) * kPnlLd;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int w8 = (w + 7) & ~7, nq = w8 >> 3;
+    const int line0 = K + w + blk * rpc, nlive = min(rpc, N - line0);
     if (tid == 0) gave_up = 0;
-    if (tid < 128) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&ready[tid])));
+    if (tid < 16) asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"((unsigned)__cvta_generic_to_shared(&ready[tid])));
     const bool vec = (w % 8 == 0) && (lda % 8 == 0) && ((((uintptr_t)(A + K)) & 15) == 0);
-    if (live) {
-        if (ROWS) {
-            const S* R = A + (int64_t)idx * lda + K;
+    if (ROWS) {
+        for (int p = tid; p < rpc * nq; p += kPnlThreads) {
+            const int r = p / nq, C = 8 * (p - r * nq);
+            float v[8];
+            const S* src = A + (int64_t)(line0 + min(r, nlive - 1)) * lda + K + C;
             if (vec) {
-                for (int t = 0; t < w; t += 8) load8(R + t, h + t);
+                load8(src, v);
             } else {
-                for (int t = 0; t < w; ++t) h[t] = ld_elem(R + t);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[c] = (C + c < w) ? ld_elem(src + c) : 0.0f;
             }
-        } else {
-            for (int t = 0; t < w; ++t) h[t] = ld_elem(A + (int64_t)(K + t) * lda + idx);
+            store8(X + r * kPnlXld + C, v);
+        }
+    } else {
+        for (int p = tid; p < rpc * w8; p += kPnlThreads) {
+            const int t = p / rpc, c = p - t * rpc;
+            X[c * kPnlXld + t] = (t < w) ? ld_elem(A + (int64_t)(K + t) * lda + line0 + min(c, nlive - 1)) : 0.0f;
         }
     }
     __syncthreads();
     bool bad = false;
     if (warp >= kPnlFetchW) {
-        // fetchers: warp 14 the even columns, warp 15 the odd ones
-        const int f = warp - kPnlFetchW;
-        const int tmax = ROWS ? w : w - 1;  // the column CTAs never need the last column
-        for (int t = f; t < tmax; t += 2) {
-            if (!pnl_fetch(pub, t, epoch, flag, Cc, !ROWS, &gave_up)) {
-                *(volatile int*)&gave_up = 1;
-                break;
-            }
-            __syncwarp();
-            if ((tid & 31) == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(&ready[t]))
-                             : "memory");
-        }
-    } else if (mine) {
-        // rows need columns t..t+nb-1; columns need L11's rows t..t+nb-1, i.e. columns up to t+nb-2
-        const int lag = ROWS ? 0 : 1;
-        auto bar_of = [&](int col) { return (unsigned)__cvta_generic_to_shared(&ready[col]); };
-        for (int t = 0; t < w;) {
-            const int need = t - lag;
-            if (need >= 0 && !pnl_wait_ready(bar_of(need), &gave_up)) {
-                *(volatile int*)&gave_up = 1;
-                break;
-            }
-            // take up to four steps when their columns are already in (decided once per warp)
-            int nb = 1;
-            if ((threadIdx.x & 31) == 0)
-                while (nb < 4 && t + nb < w && (need + nb < 0 || pnl_test_ready(bar_of(need + nb)))) ++nb;
-            nb = __shfl_sync(0xffffffffu, nb, 0);
-            __syncwarp();  // lane 0's acquire of the extra columns orders the whole warp's reads
-            if (live) {
-                const float* c = Cc + t * kPnlLd;
-                switch (nb) {
-                case 4: pnl_steps<ROWS, 4>(h, c, t, &bad); break;
-                case 3: pnl_steps<ROWS, 3>(h, c, t, &bad); break;
-                case 2: pnl_steps<ROWS, 2>(h, c, t, &bad); break;
-                default: pnl_steps<ROWS, 1>(h, c, t, &bad); break;
+        const int f = tid - 32 * kPnlFetchW;  // 0..63
+        bool ok = true;
+        for (int q = 0; q < nq; ++q) {
+            // rows: U's rows 8(q-1).. right of block q-1, the diagonal block q, its pivots; columns: L's block column q
+            const int C = 8 * q, n4 = (w8 - C) >> 2;
+            const int n0 = ROWS ? (q > 0 ? 8 * n4 : 0) : 8 * n4, n = ROWS ? n0 + 16 + 4 : n0;
+            for (int p = f; ok && p < n; p += 64) {
+                unsigned v0, v1;
+                if (p < n0 || p < n0 + 16) {
+                    int k, e;
+                    if (p < n0) {
+                        k = (ROWS ? C - 8 : C) + p / n4;
+                        e = C + 4 * (p % n4);
+                    } else {
+                        k = C + ((p - n0) >> 1);
+                        e = C + 4 * ((p - n0) & 1);
+                    }
+                    ok = pnl_fetch2(pub + (ROWS ? 0 : kPubL) + k * 64 + (e >> 1), epoch, flag, &gave_up, v0, v1);
+                    if (ok) *reinterpret_cast<uint2*>(M + k * kPnlMld + e) = make_uint2(v0, v1);
+                } else {
+                    const int k = C + 2 * (p - n0 - 16);
+                    ok = pnl_fetch2(pub + kPubP + k, epoch, flag, &gave_up, v0, v1);
+                    if (ok) *reinterpret_cast<float2*>(pv + k) = make_float2(__uint_as_float(v0), __uint_as_float(v1));
                 }
             }
-            t += nb;
+            if (!ok) *(volatile int*)&gave_up = 1;
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(&ready[q]))
+                             : "memory");
         }
+    } else {
+        const int nsol = rpc >> 5;  // solver warps; the rest help
+        for (int q = 0; q < nq; ++q) {
+            const int C0 = 8 * q, B0 = C0 - 8;
+            pnl_wait_ready((unsigned)__cvta_generic_to_shared(&ready[q]), &gave_up);
+            __syncwarp();
+            if (warp < nsol) {
+                float* xl = X + tid * kPnlXld + C0;
+                float x[8];
+                *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xl);
+                *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(xl + 4);
+                if (q > 0) pnl_apply(*reinterpret_cast<const uint4*>(xl - 8), M + B0 * kPnlMld + C0, x);
+                unsigned short h[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint4 m = *reinterpret_cast<const uint4*>(M + (C0 + k) * kPnlMld + C0);
+                    if (ROWS) {
+                        const float p = pv[C0 + k], ut = h_val(h_at(m, k));
+                        if (!(fabsf(x[k]) <= fabsf(p))) bad = true;
+                        h[k] = h_bits(div_neg(x[k], p, rcp_neg_abs(ut), fabsf(ut)));
+                    } else {
+                        h[k] = h_bits(x[k]);
+                    }
+#pragma unroll
+                    for (int e = k + 1; e < 8; ++e) x[e] = fma_h(h[k], h_at(m, e), x[e]);
+                }
+                *reinterpret_cast<uint4*>(xl) =
+                    make_uint4(h_pack(h[0], h[1]), h_pack(h[2], h[3]), h_pack(h[4], h[5]), h_pack(h[6], h[7]));
+            } else if (q > 0) {
+                const int nitem = nsol * (nq - q - 1);
+                for (int it = warp - nsol; it < nitem; it += kPnlFetchW - nsol) {
+                    const int b = it / nsol, ln = 32 * (it - b * nsol) + lane, C = C0 + 8 + 8 * b;
+                    float* xl = X + ln * kPnlXld;
+                    float x[8];
+                    *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xl + C);
+                    *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(xl + C + 4);
+                    pnl_apply(*reinterpret_cast<const uint4*>(xl + B0), M + B0 * kPnlMld + C, x);
+                    *reinterpret_cast<float4*>(xl + C) = make_float4(x[0], x[1], x[2], x[3]);
+                    *reinterpret_cast<float4*>(xl + C + 4) = make_float4(x[4], x[5], x[6], x[7]);
+                }
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kPnlFetchW) : "memory");
+        }
+        if (tid >= nlive) bad = false;
     }
     if (__syncthreads_or(bad) && tid == 0) atomicOr(flag, 1);
     if (gave_up) {
@@ -1297,29 +1393,54 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
         }
         return;
     }
-    if (!live) return;
+    // the solved blocks: eight binary16 values (multipliers negated) at X[line][8 q]
     if (ROWS) {
-        S* R = A + (int64_t)idx * lda + K;
-        if (vec) {
-            for (int t = 0; t < w; t += 8) store8(R + t, h + t);
-        } else {
-            for (int t = 0; t < w; ++t) st_elem(R + t, h[t]);
+        for (int p = tid; p < nlive * nq; p += kPnlThreads) {
+            const int r = p / nq, C = 8 * (p - r * nq);
+            uint4 h = *reinterpret_cast<const uint4*>(X + r * kPnlXld + C);
+            h.x ^= 0x80008000u; h.y ^= 0x80008000u; h.z ^= 0x80008000u; h.w ^= 0x80008000u;
+            S* dst = A + (int64_t)(line0 + r) * lda + K + C;
+            if constexpr (std::is_same<S, __half>::value) {
+                if (vec) {
+                    *reinterpret_cast<uint4*>(dst) = h;
+                    continue;
+                }
+            }
+            if (vec) {
+                float v[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) v[c] = h_val(h_at(h, c));
+                store8(dst, v);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (C + c < w) st_elem(dst + c, h_val(h_at(h, c)));
+            }
         }
     } else {
-        for (int t = 0; t < w; ++t) st_elem(A + (int64_t)(K + t) * lda + idx, h[t]);
-        // U12^T for the tensor-core update: row idx - ut_col0, columns ut_k0 .. ut_k0 + w - 1
-        // (columns left of ut_col0 are not part of that update)
-        if (Ut && idx >= ut_col0) {
-            __half* u0 = Ut + (int64_t)(idx - ut_col0) * ldut + ut_k0;
-            if ((w % 8 == 0) && (ldut % 8 == 0) && (ut_k0 % 8 == 0) && ((((uintptr_t)Ut) & 15) == 0)) {
-                for (int t = 0; t < w; t += 8) {
-                    __align__(16) __half e[8];
+        // U12 by rows, then U12^T for the tensor-core update: row idx - ut_col0, columns
+        // ut_k0 .. ut_k0 + w - 1 (columns left of ut_col0 are not part of that update)
+        const unsigned short* Xh = reinterpret_cast<const unsigned short*>(X);
+        for (int p = tid; p < rpc * w; p += kPnlThreads) {
+            const int t = p / rpc, c = p - t * rpc;
+            if (c < nlive)
+                st_elem(A + (int64_t)(K + t) * lda + line0 + c,
+                        h_val(Xh[2 * (c * kPnlXld + (t & ~7)) + (t & 7)]));
+        }
+        if (Ut) {
+            const bool uvec = (w % 8 == 0) && (ldut % 8 == 0) && (ut_k0 % 8 == 0) && ((((uintptr_t)Ut) & 15) == 0);
+            for (int p = tid; p < nlive * nq; p += kPnlThreads) {
+                const int c = p / nq, C = 8 * (p - c * nq), idx = line0 + c;
+                if (idx < ut_col0) continue;
+                const uint4 h = *reinterpret_cast<const uint4*>(X + c * kPnlXld + C);
+                __half* u0 = Ut + (int64_t)(idx - ut_col0) * ldut + ut_k0 + C;
+                if (uvec) {
+                    *reinterpret_cast<uint4*>(u0) = h;
+                } else {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) e[q] = __float2half_rn(h[t + q]);
-                    *reinterpret_cast<uint4*>(u0 + t) = *reinterpret_cast<const uint4*>(e);
+                    for (int e = 0; e < 8; ++e)
+                        if (C + e < w) u0[e] = __ushort_as_half(h_at(h, e));
                 }
-            } else {
-                for (int t = 0; t < w; ++t) u0[t] = __float2half_rn(h[t]);
             }
         }
     }
@@ -1338,7 +1459,7 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
 template <typename S>
 __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16(S* __restrict__ A, int64_t lda, int K, int w, int N,
                                                            int nrb, int rpc, int* __restrict__ ipiv, int* __restrict__ flag,
-                                                           float* __restrict__ stage, __half* __restrict__ Ut,
+                                                           __half* __restrict__ Ut,
                                                            int ldut, int ut_col0, int ut_k0,
                                                            unsigned long long* __restrict__ pub, unsigned epoch,
                                                            unsigned* __restrict__ err, int* __restrict__ tickets,
@@ -1354,7 +1475,7 @@ __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16(S* __restrict__ A, i
     __syncthreads();
     const int r = role;
     if (r == 0)
-        diag_lu16_body<true, S>(A, lda, K, w, ipiv, flag, stage, pub, epoch);
+        diag_lu16_body<true, S>(A, lda, K, w, ipiv, flag, nullptr, pub, epoch);
     else if (r <= nrb)
         panel16_stream<true, S>(A, lda, K, w, N, r - 1, rpc, Ut, ldut, ut_col0, ut_k0, flag, pub, epoch, err);
     else
@@ -1390,7 +1511,7 @@ __device__ __forceinline__ void offdiag16_body(S* __restrict__ A, int64_t lda, i
                                                int nrow_blocks, __half* __restrict__ Ut, int ldut,
                                                int* __restrict__ flag, const float* stage, int bid,
                                                int ut_col0 = -1, int ut_k0 = 0, int tid_in = -1,
-                                               float* smem = nullptr, int off0 = 0)
+                                               float* smem = nullptr)
 {
     if (ut_col0 < 0) ut_col0 = K + w;
     if (tid_in < 0 && *(volatile int*)flag) return;  // (a group of a larger CTA: its caller checked)
@@ -1401,7 +1522,7 @@ __device__ __forceinline__ void offdiag16_body(S* __restrict__ A, int64_t lda, i
     float* D = smem ? smem : osm;    // U11 (row role) or L11^T (column role), wp x wp
     float* X = D + wp * wp;          // X[t * ROWS + tid]: this thread's multipliers / U entries
     float* pv = X + wp * ROWS;          // |a_tt|, unrounded
-    float* rinv = pv + wp;           // 1 / u_tt, correctly rounded
+    float* rinv = pv + wp;           // rcp_neg_abs(u_tt)
     const int tid = tid_in >= 0 ? tid_in : (int)threadIdx.x;
     const bool row_role = bid < nrow_blocks;
     {
@@ -1413,10 +1534,9 @@ __device__ __forceinline__ void offdiag16_body(S* __restrict__ A, int64_t lda, i
         if (tid < wp) pv[tid] = fabsf(stage[kStagePivOff + tid]);
     }
     __syncthreads();
-    if (row_role && tid < wp) rinv[tid] = __frcp_rn(D[tid * wp + tid]);
+    if (row_role && tid < wp) rinv[tid] = rcp_neg_abs(D[tid * wp + tid]);
     __syncthreads();
-    // off0: the first off0 rows (columns) below (right of) the block are someone else's
-    const int idx = K + w + off0 + (row_role ? bid : bid - nrow_blocks) * ROWS + tid;
+    const int idx = K + w + (row_role ? bid : bid - nrow_blocks) * ROWS + tid;
     const bool live = idx < N;
     float* Xt = X + tid;
     if (row_role) {
@@ -1451,7 +1571,7 @@ __device__ __forceinline__ void offdiag16_body(S* __restrict__ A, int64_t lda, i
                 const int t = j0 + tt;
                 const float* Dt = D + t * wp + j0;
                 if (live && t < w && !(fabsf(x[tt]) <= pv[t])) bad = true;
-                const float l = div_round_h(x[tt], Dt[tt], rinv[t]);
+                const float u = Dt[tt], l = -round_h(div_neg(x[tt], u, rinv[t], fabsf(u)));
                 x[tt] = l;
 #pragma unroll
                 for (int k = tt + 1; k < 32; ++k) x[k] = fmaf(-l, Dt[k], x[k]);
@@ -1534,10 +1654,9 @@ template <typename S, int ROWS = kO16Rows>
 __global__ void __launch_bounds__(ROWS) k_offdiag16(S* __restrict__ A, int64_t lda, int K, int w, int N,
                                                  int nrow_blocks, __half* __restrict__ Ut, int ldut,
                                                  int* __restrict__ flag, const float* __restrict__ stage,
-                                                 int ut_col0, int ut_k0, int off0)
+                                                 int ut_col0, int ut_k0)
 {
-    offdiag16_body<S, ROWS>(A, lda, K, w, N, nrow_blocks, Ut, ldut, flag, stage, (int)blockIdx.x, ut_col0, ut_k0, -1,
-                            nullptr, off0);
+    offdiag16_body<S, ROWS>(A, lda, K, w, N, nrow_blocks, Ut, ldut, flag, stage, (int)blockIdx.x, ut_col0, ut_k0);
 }
 
 // The off-diagonal solves of one panel: 128 rows (columns) per CTA, or 256 for a
@@ -1546,19 +1665,19 @@ __global__ void __launch_bounds__(ROWS) k_offdiag16(S* __restrict__ A, int64_t l
 // results: every row (column) is solved by one thread in the same order.
 template <typename S>
 static nl_status launch_offdiag16(S* A, int64_t ld, int K, int wd, int N, __half* ut, int ldut, int* flag,
-                                  const float* stage, int ut_col0, int ut_k0, cudaStream_t st, int off0 = 0)
+                                  const float* stage, int ut_col0, int ut_k0, cudaStream_t st)
 {
-    const int rest = N - K - wd - off0, wp = (int)round_up(wd, 32);  // rows (columns) from K + wd + off0
+    const int rest = N - K - wd, wp = (int)round_up(wd, 32);
     const bool wide = wp > 64 && 2 * (int)cdiv(rest, kO16Rows) > num_sms();
     prof_begin("k_offdiag16", st);
     if (wide) {
         const int nrb = (int)cdiv(rest, 256);
         k_offdiag16<S, 256><<<2 * nrb, 256, offdiag16_smem(wp, 256), st>>>(A, ld, K, wd, N, nrb, ut, ldut, flag, stage,
-                                                                         ut_col0, ut_k0, off0);
+                                                                         ut_col0, ut_k0);
     } else {
         const int nrb = (int)cdiv(rest, kO16Rows);
         k_offdiag16<S><<<2 * nrb, kO16Threads, offdiag16_smem(wp), st>>>(A, ld, K, wd, N, nrb, ut, ldut, flag, stage,
-                                                                        ut_col0, ut_k0, off0);
+                                                                        ut_col0, ut_k0);
     }
     prof_end("k_offdiag16", st);
     NL_CUDA_OK(cudaGetLastError());
@@ -1642,7 +1761,7 @@ size_t lu_work_bytes(int N, int nb, bool fp64)
     size_t ut = fp64 ? 0 : (size_t)round_up(N, 128) * nb * 2;
     size_t shadow = fp64 ? 0 : (nb > 128 ? (size_t)N * round_up(N, 64) * 4 + 256 : round_up(ut, 256));
     return round_up(pnl, 256) + round_up(ut, 256) + 256 + (size_t)2 * 128 * 128 * 8 + 128 * 8 +
-           round_up((size_t)128 * 128 * 8, 256) + shadow;
+           round_up(kPubWords * 8, 256) + shadow;
 }
 
 void lu_work_carve(void* base, int N, int nb, bool fp64, LuWork* w)
@@ -1660,7 +1779,7 @@ void lu_work_carve(void* base, int N, int nb, bool fp64, LuWork* w)
     w->stage = p;
     p += (size_t)2 * 128 * 128 * 8 + 128 * 8;
     w->pub = (unsigned long long*)p;
-    p += round_up((size_t)128 * 128 * 8, 256);
+    p += round_up(kPubWords * 8, 256);
     w->ut2 = nullptr;
     if (!fp64 && nb > 128) {
         w->p32 = (float*)p;
@@ -1826,52 +1945,25 @@ static nl_status trailing_update(int N, S* A, int64_t ld, int K, int wd, int nb,
 }
 
 // The streaming panel (k_panel16): one CTA for the diagonal block plus
-// ceil(rest / rpc) CTAs for the rows of L21 and as many for the columns of
-// U12 (rpc = 128 while they all fit on the device at once, else 256), when
-// they fit in one wave; otherwise the two-launch path.
-static int panel16_max_ctas()
+// ceil(rest / rpc) CTAs for the rows of L21 and as many for the columns of U12.
+static nl_status panel16_setup()
 {
-    // computed once; concurrent first callers compute the same value (never a transient 0)
-    static std::atomic<int> cap{-1};
-    int c = cap.load(std::memory_order_acquire);
-    if (c < 0) {
-        c = 0;
-        int dev = 0, nsm = 0, per = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-            set_max_dynamic_smem((const void*)k_panel16<__half>) == NL_OK &&
-            set_max_dynamic_smem((const void*)k_panel16<float>) == NL_OK &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_panel16<__half>, kPnlThreads, kPnlSmem) == cudaSuccess)
-            c = per * nsm;
-        cudaGetLastError();
-        cap.store(c, std::memory_order_release);
-    }
-    return c;
+    static std::atomic<bool> done{false};
+    if (done.load(std::memory_order_acquire)) return NL_OK;
+    if (set_max_dynamic_smem((const void*)k_panel16<__half>) != NL_OK ||
+        set_max_dynamic_smem((const void*)k_panel16<float>) != NL_OK)
+        return NL_ECUDA;
+    done.store(true, std::memory_order_release);
+    return NL_OK;
 }
 
-// Rows (columns) per streaming CTA: 128 when the launch then fits on the GPU
-// (with 256 the full CTAs fall behind the diagonal block; 64 is no faster and
-// takes twice the SMs from concurrent solves), else 256; 0 when neither fits
-// (two launches instead).
+// Lines (rows, columns) per streaming CTA, one CTA per SM: 64 while all fit on
+// the GPU at once, else 128 (a launch of several waves keeps going: a CTA that
+// starts after the diagonal block is done finds every word published).
 static int panel16_rows_per_cta(int rest, int pref = 0)
 {
-    // 128 rows per CTA while every CTA fits at once (more CTAs in the chain's shadow), else
-    // 256; beyond what fits in one wave the two launches are as fast (measured on GB300 at
-    // N = 32768: the factorisation takes 65-66 ms either way)
-    const int cap = panel16_max_ctas();
-    for (int rpc : {pref == kPnlRows ? kPnlRows : 128, kPnlRows})
-        if (1 + 2 * (int)cdiv(rest, rpc) <= cap) return rpc;
-    return 0;
-}
-
-// Rows (and columns) of a panel the streaming launch takes: all of them when its
-// CTAs fit on the device at once, else as many as 256-row CTAs fitting at once
-// cover (the rest go to a following off-diagonal launch); 0 = none.
-static int panel16_fit_rows(int rest, int pref = 0)
-{
-    if (panel16_rows_per_cta(rest, pref) > 0) return rest;
-    const int nrb = (panel16_max_ctas() - 1) / 2;
-    return nrb >= 1 ? std::min(rest, nrb * kPnlRows) : 0;
+    if (pref == kPnlRows) return kPnlRows;
+    return 1 + 2 * (int)cdiv(rest, 64) <= num_sms() ? 64 : 128;
 }
 
 static std::atomic<unsigned> g_panel_epoch{0};
@@ -1887,13 +1979,13 @@ static nl_status launch_panel16(S* A, int64_t ld, int K, int wd, int N, int* ipi
     unsigned epoch = ++g_panel_epoch;
     if (epoch == 0) epoch = ++g_panel_epoch;  // 0 is the cleared buffer's tag
     int* flag = w.flag;
-    float* stage = (float*)w.stage;
     unsigned long long* pub = w.pub;
+    NL_TRY(panel16_setup());
     unsigned* err = tc_error_word();
     if (!err) err = (unsigned*)(w.info + 2);  // (a word of the info block nobody else uses)
     int* tickets = w.info + 8;  // two counters (+8, +9) of the info block; slot: the panel's index mod 2
     prof_begin("k_panel16", st);
-    k_panel16<S><<<1 + 2 * nrb, kPnlThreads, kPnlSmem, st>>>(A, ld, K, wd, N, nrb, rpc, ipiv, flag, stage, Ut, ldut,
+    k_panel16<S><<<1 + 2 * nrb, kPnlThreads, kPnlSmem, st>>>(A, ld, K, wd, N, nrb, rpc, ipiv, flag, Ut, ldut,
                                                             ut_col0, ut_k0, pub, epoch, err, tickets, slot);
     prof_end("k_panel16", st);
     NL_CUDA_OK(cudaGetLastError());
@@ -1993,20 +2085,13 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
         if (fast) {
             const int wp = (int)round_up(wd, 32);
             if constexpr (kHalf) {
-                const int R = (rest > 0 && w.stream >= 0) ? panel16_fit_rows(rest, w.stream) : 0;
-                if (R > 0) {
+                if (rest > 0 && w.stream >= 0) {
                     if (!pub_cleared) {
-                        NL_CUDA_OK(cudaMemsetAsync(w.pub, 0, (size_t)128 * 128 * 8, st));
+                        NL_CUDA_OK(cudaMemsetAsync(w.pub, 0, kPubWords * 8, st));
                         pub_cleared = true;
                     }
-                    // the streamed rows and columns, then (if any) the rest in one off-diagonal launch
                     __half* utp = tc ? ut_of(K) : nullptr;
-                    NL_TRY(launch_panel16(A, ld, K, wd, K + wd + R, ipiv, w, utp, nb, st, (K / nb) & 1));
-                    if (R < rest) {
-                        NL_TRY(launch_offdiag16<__half>(A, ld, K, wd, N, utp, nb, w.flag, (const float*)w.stage, -1,
-                                                        0, st, R));
-                        ++nl;
-                    }
+                    NL_TRY(launch_panel16(A, ld, K, wd, N, ipiv, w, utp, nb, st, (K / nb) & 1));
                     NL_TRY(update(K, wd, tc, utp));
                     nl += 2;
                     continue;
@@ -2148,7 +2233,7 @@ static nl_status lu16_factor_2lvl(int N, __half* A, int64_t ld, int* ipiv, int W
     }
     int nl = 0;
     NL_CUDA_OK(cudaMemsetAsync(w.info, 0, 10 * sizeof(int), st));  // info, flag, ..., the panel's role ticket
-    NL_CUDA_OK(cudaMemsetAsync(w.pub, 0, (size_t)128 * 128 * 8, st));
+    NL_CUDA_OK(cudaMemsetAsync(w.pub, 0, kPubWords * 8, st));
     static bool smem_set = false;
     if (!smem_set) {
         if (set_max_dynamic_smem((const void*)k_offdiag16<float>) != NL_OK ||
@@ -2166,14 +2251,9 @@ static nl_status lu16_factor_2lvl(int N, __half* A, int64_t ld, int* ipiv, int W
         for (int p0 = 0; p0 < Wd; p0 += 128) {
             const int K = K0 + p0, wd = std::min(128, Wd - p0), rest = N - K - wd;
             __half* ut = (tc && far > 0) ? w.ut : nullptr;
-            const int R = (rest > 0 && w.stream >= 0) ? panel16_fit_rows(rest, w.stream) : 0;
-            if (R > 0) {
-                NL_TRY(launch_panel16<float>(P, ldp, K, wd, K + wd + R, ipiv, w, ut, W, st, (K / 128) & 1, C1, p0));
+            if (rest > 0 && w.stream >= 0) {
+                NL_TRY(launch_panel16<float>(P, ldp, K, wd, N, ipiv, w, ut, W, st, (K / 128) & 1, C1, p0));
                 ++nl;
-                if (R < rest) {
-                    NL_TRY(launch_offdiag16<float>(P, ldp, K, wd, N, ut, W, w.flag, (const float*)w.stage, C1, p0, st, R));
-                    ++nl;
-                }
             } else {
                 prof_begin("k_diag_lu16", st);
                 k_diag_lu16<float><<<1, kD16Threads, kDiag16Smem, st>>>(P, ldp, K, wd, ipiv, w.flag, (float*)w.stage);
@@ -2485,12 +2565,14 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_lu_g(const GInst* __re
     diag_lu_body<T, S, RND>(reinterpret_cast<S*>(I.A), I.ld, K, min(nb, I.N - K), I.ipiv, I.flag, I.stage);
 }
 
-__global__ void __launch_bounds__(kD16Threads, 1) k_diag_lu16_g(const GInst* __restrict__ inst,
-                                                                const GTask* __restrict__ tasks, int K, int nb)
+// WMAX = 64 (panels of at most 64 columns): half the threads, so two blocks share an SM
+template <int WMAX>
+__global__ void __launch_bounds__(4 * WMAX, 128 / WMAX) k_diag_lu16_g(const GInst* __restrict__ inst,
+                                                                      const GTask* __restrict__ tasks, int K, int nb)
 {
     const GInst I = inst[tasks[blockIdx.x].inst];
-    diag_lu16_body(reinterpret_cast<__half*>(I.A), I.ld, K, min(nb, I.N - K), I.ipiv, I.flag,
-                   reinterpret_cast<float*>(I.stage));
+    diag_lu16_body<false, __half, WMAX, 4 * WMAX>(reinterpret_cast<__half*>(I.A), I.ld, K, min(nb, I.N - K), I.ipiv,
+                                                  I.flag, reinterpret_cast<float*>(I.stage));
 }
 
 template <typename T, typename S, bool RND>
@@ -3210,7 +3292,8 @@ nl_status lu_grouped_setup()
 {
     static bool smem_set = false;
     if (!smem_set) {
-        if (set_max_dynamic_smem((const void*)k_diag_lu16_g) != NL_OK ||
+        if (set_max_dynamic_smem((const void*)k_diag_lu16_g<64>) != NL_OK ||
+            set_max_dynamic_smem((const void*)k_diag_lu16_g<128>) != NL_OK ||
             set_max_dynamic_smem((const void*)k_offdiag16_g) != NL_OK ||
             set_max_dynamic_smem((const void*)k_diag_lu_g<double, double, false>) != NL_OK ||
             set_max_dynamic_smem((const void*)k_offdiag_g<double, double, false>) != NL_OK ||
@@ -3268,7 +3351,8 @@ nl_status lu_grouped_factor(const GroupPlan& plan, const GInst* dev_inst, cudaSt
         } else {
             if (nd) {
                 prof_begin("k_diag_lu16", st);
-                k_diag_lu16_g<<<nd, kD16Threads, kDiag16Smem, st>>>(dev_inst, td, K, nb);
+                if (nb <= 64) k_diag_lu16_g<64><<<nd, 256, Diag16<64>::smem, st>>>(dev_inst, td, K, nb);
+                else k_diag_lu16_g<128><<<nd, 512, Diag16<128>::smem, st>>>(dev_inst, td, K, nb);
                 prof_end("k_diag_lu16", st);
             }
             if (no) {
@@ -3297,7 +3381,7 @@ __global__ void k_div_round16(int64_t n, const float* __restrict__ a, const floa
                               float* __restrict__ out)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = div_round_h(a[i], b[i], __frcp_rn(b[i]));
+    if (i < n) out[i] = div_round_h(a[i], b[i]);
 }
 
 }  // namespace nl
