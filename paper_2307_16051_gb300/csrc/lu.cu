@@ -824,7 +824,7 @@ constexpr int kStagePivOff = 2 * 128 * 128;
 //     diagonal block, and that block factored in registers (lane r holds
 //     row r; the pivot row by shuffles, about 90 cycles a column);
 //   the others: U's next columns (warp 4, for warp 0's next block) and those
-//     further right, the multipliers of the rows further below, step q-1
+//     further right, the multipliers of the rows further below; step q
 //     published; then (the warps off warp 0's scheduler) block q applied to the
 //     rest of the trailing matrix, four columns of every few rows per thread.
 // The working copy S is binary32 in shared memory; final entries go to Hs as
@@ -838,7 +838,7 @@ constexpr int kStagePivOff = 2 * 128 * 128;
 // diagonal, which comes first), checked on every pre-division value; a pivot
 // that is zero or not finite in binary16 is left to the interchanging path
 // too.  There are no spin waits.
-// Measured (GB300, w = 128, one launch alone): 30.7 us, of which about 20 are the
+// Measured (GB300, w = 128, one launch alone): 28.7 us, of which about 19 are the
 // steps and 5 the stage; the former column pipeline (a hand-off between warps
 // per column, 16 warps competing for the issue slots of the chain) took 57 us.
 // NT threads; WMAX = 64 or 128, the largest w.
@@ -903,9 +903,7 @@ __device__ __forceinline__ void store8(float* p, const float* v)
 //   word k * 64 + e / 2, e > k even:           u_ke, u_k(e+1)
 //   word kPubL + k * 64 + e / 2, e > k even:   -l_ek, -l_(e+1)k
 //   word kPubP + t:                            the unrounded pivot a_tt (binary32)
-// Step s publishes U's rows 8(s-1)..8(s-1)+7 right of block column s-1, the
-// diagonal 8 x 8 block s, its pivots, and the multipliers of block column s:
-// what the streaming rows and columns need for their own step s.
+// Step s publishes U's rows and L's columns 8 s..8 s + 7 and their pivots.
 constexpr int kPubL = 128 * 64;
 constexpr int kPubP = 2 * 128 * 64;
 constexpr size_t kPubWords = (size_t)kPubP + 128;
@@ -916,7 +914,7 @@ __device__ __forceinline__ void pub_store2(unsigned long long* dst, unsigned epo
     asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(dst), "l"(t | v0), "l"(t | v1) : "memory");
 }
 
-// One warp per k (k = 0..7, warp v of 8): Hs and rc hold block columns <= s and U's rows < 8 s.
+// One warp per k (k = 0..7, warp v of 8).
 template <int HLD>
 __device__ __forceinline__ void diag16_publish(int s, int w8, const unsigned short* Hs, const float4* rc,
                                                unsigned long long* pub, unsigned epoch, int v, int lane)
@@ -924,18 +922,12 @@ __device__ __forceinline__ void diag16_publish(int s, int w8, const unsigned sho
     const int C = 8 * s, k = C + v, e = C + 4 * lane;
     if (e < w8) {
         const unsigned short* h = Hs + e * HLD + k;
-        pub_store2(pub + kPubL + k * 64 + (e >> 1), epoch, h_pack(h[0], h[HLD]), h_pack(h[2 * HLD], h[3 * HLD]));
-        if (s > 0) {
-            const uint2 u = *reinterpret_cast<const uint2*>(Hs + (k - 8) * HLD + e);
-            pub_store2(pub + (k - 8) * 64 + (e >> 1), epoch, u.x, u.y);
-        }
-    }
-    if (lane < 2) {
         const uint2 u = *reinterpret_cast<const uint2*>(Hs + k * HLD + e);
+        pub_store2(pub + kPubL + k * 64 + (e >> 1), epoch, h_pack(h[0], h[HLD]), h_pack(h[2 * HLD], h[3 * HLD]));
         pub_store2(pub + k * 64 + (e >> 1), epoch, u.x, u.y);
-    } else if (lane == 2 && v < 4) {
-        pub_store2(pub + kPubP + C + 2 * v, epoch, __float_as_uint(rc[C + 2 * v].z), __float_as_uint(rc[C + 2 * v + 1].z));
     }
+    if (lane == 0 && v < 4)
+        pub_store2(pub + kPubP + C + 2 * v, epoch, __float_as_uint(rc[C + 2 * v].z), __float_as_uint(rc[C + 2 * v + 1].z));
 }
 
 // PUB: also publish the block as it is factored, for the streaming solves of
@@ -1042,12 +1034,34 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
                     const uint2 v = *reinterpret_cast<const uint2*>(Hs + (B0 + k) * HLD + J);
                     u[k][0] = h_lo(v.x); u[k][1] = h_hi(v.x); u[k][2] = h_lo(v.y); u[k][3] = h_hi(v.y);
                 }
-#pragma unroll 2
-                for (int i = C0 + sl; i < w8; i += ns) {
-                    if (i < C1 && J < C1) continue;
-                    float* Si = S + i * LD + J;
+                // two rows at a time (a thread of the diagonal block's columns starts below it)
+                int i = C0 + sl;
+                if (J < C1)
+                    while (i < C1) i += ns;
+                const int step = ns * LD, hstep = ns * HLD;
+                float* Si = S + i * LD + J;
+                const unsigned short* Hi = Hs + i * HLD + B0;
+                for (; i + ns < w8; i += 2 * ns, Si += 2 * step, Hi += 2 * hstep) {
+                    float4 v = *reinterpret_cast<const float4*>(Si), z = *reinterpret_cast<const float4*>(Si + step);
+                    const uint4 L = *reinterpret_cast<const uint4*>(Hi), M = *reinterpret_cast<const uint4*>(Hi + hstep);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const unsigned short l = h_at(L, k), m = h_at(M, k);
+                        v.x = fma_h(l, u[k][0], v.x);
+                        v.y = fma_h(l, u[k][1], v.y);
+                        v.z = fma_h(l, u[k][2], v.z);
+                        v.w = fma_h(l, u[k][3], v.w);
+                        z.x = fma_h(m, u[k][0], z.x);
+                        z.y = fma_h(m, u[k][1], z.y);
+                        z.z = fma_h(m, u[k][2], z.z);
+                        z.w = fma_h(m, u[k][3], z.w);
+                    }
+                    *reinterpret_cast<float4*>(Si) = v;
+                    *reinterpret_cast<float4*>(Si + step) = z;
+                }
+                if (i < w8) {
                     float4 v = *reinterpret_cast<const float4*>(Si);
-                    const uint4 L = *reinterpret_cast<const uint4*>(Hs + i * HLD + B0);
+                    const uint4 L = *reinterpret_cast<const uint4*>(Hi);
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         const unsigned short l = h_at(L, k);
@@ -1061,7 +1075,6 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
             }
         }
         __syncthreads();
-        if (PUB && pubw && q > 0) diag16_publish<HLD>(q - 1, w8, Hs, rc, pub, epoch, pubv, lane);
         if (C1 >= w8) break;
         if (wid == 0) {
             // row C1 + lane, with the diagonal block's U and pivots in registers
@@ -1139,6 +1152,7 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
             }
             __syncwarp();
             asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
+            if (PUB && pubw) diag16_publish<HLD>(q, w8, Hs, rc, pub, epoch, pubv, lane);
         }
     }
     if (PUB && pubw) diag16_publish<HLD>(nq - 1, w8, Hs, rc, pub, epoch, pubv, lane);
@@ -1207,8 +1221,9 @@ __global__ void __launch_bounds__(kD16Threads, 1) k_diag_lu16(S* __restrict__ A,
 // after the last published block is one block solve: a step of the stream
 // (about 500 cycles) is shorter than a step of the diagonal block, and the
 // launch takes the diagonal block's time plus a tail of one step (N = 4096:
-// 36.6 us a panel on average, 67.9 us with the column pipeline and left-looking
-// streams).  Eight
+// 30.5 us a panel on average, 67.9 us with the column pipeline and left-looking
+// streams; one pair of words in flight per fetching lane and a step published
+// only in the next one: 36.6 us).  Eight
 // lines' multipliers of a solved block overwrite the first half of its place
 // in X.  Every entry takes its fused multiply-adds in increasing k, so the
 // results are bitwise those of k_diag_lu16 followed by k_offdiag16.  Every
@@ -1223,21 +1238,28 @@ constexpr size_t kPnlSmem = (size_t)kPnlRows * kPnlXld * 4 + (size_t)128 * kPnlM
 static_assert(kPnlSmem >= kDiag16Smem, "the diagonal block's CTA uses the same launch");
 constexpr long long kPnlSpin = 1LL << 22;
 
-// Fetch lane: one pair of published words (16 bytes) once both carry this launch's epoch.
-__device__ __forceinline__ bool pnl_fetch2(const unsigned long long* q, unsigned epoch, const int* flag,
-                                           const int* gave_up, unsigned& v0, unsigned& v1)
+// Fetch lane: up to five pairs of published words (16 bytes each; bit v of todo:
+// pair v), all loads in flight at once, until both words of every pair carry
+// this launch's epoch.
+template <typename Src, typename Dst>
+__device__ __forceinline__ bool pnl_fetch(unsigned todo, Src src, Dst dst, unsigned epoch, const int* flag,
+                                          const int* gave_up)
 {
-    for (long long it = 0; it < kPnlSpin; ++it) {
-        unsigned long long a, b;
-        asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(q) : "memory");
-        if ((unsigned)(a >> 32) == epoch && (unsigned)(b >> 32) == epoch) {
-            v0 = (unsigned)a;
-            v1 = (unsigned)b;
-            return true;
-        }
-        if ((it & 63) == 63 && (*(volatile const int*)flag || *(volatile const int*)gave_up)) return false;
+    for (long long it = 0; todo && it < kPnlSpin; ++it) {
+        unsigned long long a[5], b[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v)
+            if (todo >> v & 1u)
+                asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a[v]), "=l"(b[v]) : "l"(src(v)) : "memory");
+#pragma unroll
+        for (int v = 0; v < 5; ++v)
+            if ((todo >> v & 1u) && (unsigned)(a[v] >> 32) == epoch && (unsigned)(b[v] >> 32) == epoch) {
+                dst(v, (unsigned)a[v], (unsigned)b[v]);
+                todo &= ~(1u << v);
+            }
+        if (todo && (it & 63) == 63 && (*(volatile const int*)flag || *(volatile const int*)gave_up)) return false;
     }
-    return false;
+    return !todo;
 }
 
 __device__ __forceinline__ void pnl_wait_ready(uint32_t bar, int* gave_up)
@@ -1285,6 +1307,7 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
     if (tid == 0) gave_up = 0;
     if (tid < 16) asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"((unsigned)__cvta_generic_to_shared(&ready[tid])));
     const bool vec = (w % 8 == 0) && (lda % 8 == 0) && ((((uintptr_t)(A + K)) & 15) == 0);
+    const bool cvec = (lda % 8 == 0) && ((((uintptr_t)(A + line0)) & 15) == 0);  // eight columns at a time
     if (ROWS) {
         for (int p = tid; p < rpc * nq; p += kPnlThreads) {
             const int r = p / nq, C = 8 * (p - r * nq);
@@ -1298,6 +1321,21 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
             }
             store8(X + r * kPnlXld + C, v);
         }
+    } else if (cvec) {
+        const int g8 = rpc >> 3;
+        for (int p = tid; p < g8 * w8; p += kPnlThreads) {
+            const int t = p / g8, c = 8 * (p - t * g8);
+            float v[8];
+            if (t < w && c + 8 <= nlive) {
+                load8(A + (int64_t)(K + t) * lda + line0 + c, v);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    v[e] = (t < w) ? ld_elem(A + (int64_t)(K + t) * lda + line0 + min(c + e, nlive - 1)) : 0.0f;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) X[(c + e) * kPnlXld + t] = v[e];
+        }
     } else {
         for (int p = tid; p < rpc * w8; p += kPnlThreads) {
             const int t = p / rpc, c = p - t * rpc;
@@ -1307,31 +1345,21 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
     __syncthreads();
     bool bad = false;
     if (warp >= kPnlFetchW) {
-        const int f = tid - 32 * kPnlFetchW;  // 0..63
         bool ok = true;
         for (int q = 0; q < nq; ++q) {
-            // rows: U's rows 8(q-1).. right of block q-1, the diagonal block q, its pivots; columns: L's block column q
-            const int C = 8 * q, n4 = (w8 - C) >> 2;
-            const int n0 = ROWS ? (q > 0 ? 8 * n4 : 0) : 8 * n4, n = ROWS ? n0 + 16 + 4 : n0;
-            for (int p = f; ok && p < n; p += 64) {
-                unsigned v0, v1;
-                if (p < n0 || p < n0 + 16) {
-                    int k, e;
-                    if (p < n0) {
-                        k = (ROWS ? C - 8 : C) + p / n4;
-                        e = C + 4 * (p % n4);
-                    } else {
-                        k = C + ((p - n0) >> 1);
-                        e = C + 4 * ((p - n0) & 1);
-                    }
-                    ok = pnl_fetch2(pub + (ROWS ? 0 : kPubL) + k * 64 + (e >> 1), epoch, flag, &gave_up, v0, v1);
-                    if (ok) *reinterpret_cast<uint2*>(M + k * kPnlMld + e) = make_uint2(v0, v1);
-                } else {
-                    const int k = C + 2 * (p - n0 - 16);
-                    ok = pnl_fetch2(pub + kPubP + k, epoch, flag, &gave_up, v0, v1);
-                    if (ok) *reinterpret_cast<float2*>(pv + k) = make_float2(__uint_as_float(v0), __uint_as_float(v1));
-                }
-            }
+            // warp v: every second of the step's eight rows of M from the v-th, four entries per lane;
+            // lanes 0 and 1 of a row CTA also four pivots
+            const int C = 8 * q, f = warp - kPnlFetchW, e = C + 4 * lane, kp = C + 4 * f + 2 * lane;
+            const unsigned long long* src = pub + (ROWS ? 0 : kPubL) + (C + f) * 64 + (e >> 1);
+            unsigned short* dst = M + (C + f) * kPnlMld + e;
+            const unsigned todo = (e < w8 ? 15u : 0u) | (ROWS && lane < 2 ? 16u : 0u);
+            ok = ok && pnl_fetch(
+                           todo, [&](int v) { return v < 4 ? src + v * 128 : pub + kPubP + kp; },
+                           [&](int v, unsigned v0, unsigned v1) {
+                               if (v < 4) *reinterpret_cast<uint2*>(dst + 2 * v * kPnlMld) = make_uint2(v0, v1);
+                               else *reinterpret_cast<float2*>(pv + kp) = make_float2(__uint_as_float(v0), __uint_as_float(v1));
+                           },
+                           epoch, flag, &gave_up);
             if (!ok) *(volatile int*)&gave_up = 1;
             __syncwarp();
             if (lane == 0)
@@ -1421,8 +1449,25 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
         // U12 by rows, then U12^T for the tensor-core update: row idx - ut_col0, columns
         // ut_k0 .. ut_k0 + w - 1 (columns left of ut_col0 are not part of that update)
         const unsigned short* Xh = reinterpret_cast<const unsigned short*>(X);
-        for (int p = tid; p < rpc * w; p += kPnlThreads) {
-            const int t = p / rpc, c = p - t * rpc;
+        const int g8 = cvec ? nlive >> 3 : 0;  // whole groups of eight columns
+        for (int p = tid; p < g8 * w; p += kPnlThreads) {
+            const int t = p / g8, c = 8 * (p - t * g8);
+            unsigned short h[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) h[e] = Xh[2 * ((c + e) * kPnlXld + (t & ~7)) + (t & 7)];
+            S* dst = A + (int64_t)(K + t) * lda + line0 + c;
+            if constexpr (std::is_same<S, __half>::value) {
+                *reinterpret_cast<uint4*>(dst) =
+                    make_uint4(h_pack(h[0], h[1]), h_pack(h[2], h[3]), h_pack(h[4], h[5]), h_pack(h[6], h[7]));
+            } else {
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = h_val(h[e]);
+                store8(dst, v);
+            }
+        }
+        for (int p = tid; p < (rpc - 8 * g8) * w; p += kPnlThreads) {
+            const int t = p / (rpc - 8 * g8), c = 8 * g8 + p - t * (rpc - 8 * g8);
             if (c < nlive)
                 st_elem(A + (int64_t)(K + t) * lda + line0 + c,
                         h_val(Xh[2 * (c * kPnlXld + (t & ~7)) + (t & 7)]));
