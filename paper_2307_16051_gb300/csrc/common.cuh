@@ -113,27 +113,6 @@ __device__ __forceinline__ float div_round_h(float a, float u)
     return -round_h(div_neg(a, u, rcp_neg_abs(u), fabsf(u)));
 }
 
-// The sum of part[0 .. n) in index order, by every thread of the block (the
-// last block of a grid-wide reduction): the partials are staged through
-// shared memory a block's width at a time (parallel loads from L2) and thread
-// 0 adds them in order, so the result is that of one thread's sequential
-// loop; valid in thread 0.
-__device__ __forceinline__ double ordered_sum_staged(const double* part, int n, double* buf)
-{
-    double t = 0.0;
-    for (int base = 0; base < n; base += blockDim.x) {
-        const int q = base + threadIdx.x;
-        if (q < n) buf[threadIdx.x] = __ldcg(part + q);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int m = min((int)blockDim.x, n - base);
-            for (int e = 0; e < m; ++e) t += buf[e];
-        }
-        __syncthreads();
-    }
-    return t;
-}
-
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
 {
@@ -155,6 +134,19 @@ __device__ __forceinline__ T block_sum(T v, T* red)
     T s = T(0);
     for (int w = 0; w < nw; ++w) s += red[w];
     return s;
+}
+
+// The sum of part[0 .. n), by every thread of the last block of a grid-wide
+// reduction: each thread adds every blockDim.x-th partial in order, then the
+// fixed tree of block_sum (red: blockDim.x / 32 entries; valid in every
+// thread).  One thread adding all of them takes a dependent double addition
+// each, the whole of a small kernel's tail: 2048 partials took 75 us of the
+// residual's 263 us at N = 16384, and 512 about 10 of 29 us at N = 4096.
+__device__ __forceinline__ double partials_sum(const double* part, int n, double* red)
+{
+    double t = 0.0;
+    for (int q = threadIdx.x; q < n; q += blockDim.x) t += __ldcg(part + q);
+    return block_sum(t, red);
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int* p)

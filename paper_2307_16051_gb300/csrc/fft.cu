@@ -102,8 +102,7 @@ __global__ void __launch_bounds__(128) k_fft_pass_a(int N, int L, int L1, int L2
 // inverse transform).  MODE 2: the inverse transform's real part / L at the
 // indices N-1 .. 2N-2 gives y_i; then t_i, r_i = 1/(1 - t_i), F_i = v_i - r_i
 // (v = x + scale u, also written to xout when given), and ||F||_2 with a
-// deterministic reduction (per-block partials, the last block sums them in
-// block order).
+// deterministic reduction (per-block partials, the last block sums them).
 template <int MODE, typename TU>
 __global__ void __launch_bounds__(128) k_fft_pass_b(int N, int L, int L1, int L2, const double2* __restrict__ tw,
                                                     const double2* __restrict__ Y, const double2* __restrict__ Hh,
@@ -160,9 +159,8 @@ __global__ void __launch_bounds__(128) k_fft_pass_b(int N, int L, int L1, int L2
         }
         __syncthreads();
         if (last) {
-            __shared__ double buf[128];
             __threadfence();
-            const double sum = ordered_sum_staged(part, L1, buf);
+            const double sum = partials_sum(part, L1, red);
             if (threadIdx.x == 0) {
                 *fnorm = sqrt(sum);
                 *cnt = 0u;

@@ -4,14 +4,17 @@
 // Givens rotations for left-preconditioned GMRES.
 //
 // All reductions run in a fixed order (per-thread sequential sums, then a
-// fixed shuffle tree, then per-block partials summed in block order by the
-// last block), so every result is bitwise reproducible from run to run.
+// fixed shuffle tree, then the per-block partials summed in a fixed tree by
+// the last block), so every result is bitwise reproducible from run to run.
 #include "common.cuh"
 #include "internal.h"
 
 namespace nl {
 
+// Warps (rows) per block and iterations' loads in flight; 4 and 16 warps, eight in
+// flight and two rows per warp were no faster at N = 4096 and N >= 16384.
 constexpr int kGemvWarps = 8;
+constexpr int kGemvUnroll = 4;
 
 // r_i = b_i - sum_j A_ij u_j (b NULL: r = A u).  One warp per row, float4
 // loads along the row.  The dot product is accumulated in two-float
@@ -65,17 +68,17 @@ __device__ __forceinline__ double gemv_row(int N, const float* __restrict__ A, i
         const float4* u4 = reinterpret_cast<const float4*>(u);
         DF s = {0.0f, 0.0f};
         int k = lane;
-        // four iterations' loads in flight before their products (the same order of terms): at
+        // kGemvUnroll iterations' loads in flight before their products (the same order of terms): at
         // N = 4096 a warp per row has 32 iterations, too few warps to hide the latency one at a time
-        for (; k + 96 < n4; k += 128) {
-            float4 a[4], x[4];
+        for (; k + 32 * (kGemvUnroll - 1) < n4; k += 32 * kGemvUnroll) {
+            float4 a[kGemvUnroll], x[kGemvUnroll];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < kGemvUnroll; ++q) {
                 a[q] = __ldcs(A4 + k + 32 * q);
                 x[q] = __ldg(u4 + k + 32 * q);
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < kGemvUnroll; ++q) {
                 df_add_prod(s, a[q].x, x[q].x);
                 df_add_prod(s, a[q].y, x[q].y);
                 df_add_prod(s, a[q].z, x[q].z);
@@ -137,9 +140,8 @@ __global__ void __launch_bounds__(kGemvWarps * 32)
     }
     __syncthreads();
     if (last && rnorm) {
-        __shared__ double buf[kGemvWarps * 32];
         __threadfence();
-        const double t = ordered_sum_staged(partial, (int)gridDim.x, buf);
+        const double t = partials_sum(partial, (int)gridDim.x, red);
         if (threadIdx.x == 0) *rnorm = sqrt(t);
     }
     if (last && threadIdx.x == 0) *counter = 0u;
@@ -149,7 +151,7 @@ int gemv_partials(int N) { return (int)cdiv(N, kGemvWarps); }
 
 // Grouped residual r = b - J32 u: one block per task {instance, first row},
 // instances with an IR step in progress only; per-instance block partials
-// summed in block order by the instance's last block (into st.nr_new).
+// summed by the instance's last block (into st.nr_new).
 __global__ void __launch_bounds__(kGemvWarps * 32)
     k_gemv_residual_g(const BInst* __restrict__ inst, BState* __restrict__ st, const BTask* __restrict__ tasks)
 {
@@ -174,9 +176,8 @@ __global__ void __launch_bounds__(kGemvWarps * 32)
     }
     __syncthreads();
     if (last) {
-        __shared__ double buf[kGemvWarps * 32];
         __threadfence();
-        const double t = ordered_sum_staged(I.part, nblk, buf);
+        const double t = partials_sum(I.part, nblk, red);
         if (threadIdx.x == 0) {
             S.nr_new = sqrt(t);
             I.cnt[1] = 0u;
@@ -227,9 +228,8 @@ __global__ void __launch_bounds__(256) k_norm32(int N, const float* __restrict__
     }
     __syncthreads();
     if (last) {
-        __shared__ double buf[256];
         __threadfence();
-        const double t = ordered_sum_staged(partial, (int)gridDim.x, buf);
+        const double t = partials_sum(partial, (int)gridDim.x, red);
         if (threadIdx.x == 0) {
             *out = sqrt(t);
             *counter = 0u;

@@ -11,23 +11,29 @@
 namespace nl {
 
 // ---------------------------------------------------------------- K1: F(x) --
-// Block = kFRows rows x kFSlices j-slices; rows and j-chunks are staged in
-// shared memory (x + scale*u for the chunk, and the h window it needs).
-constexpr int kFRows = 32, kFSlices = 8, kFChunk = 256;
+// Block = ROWS rows x 256 / ROWS j-slices; rows and j-chunks are staged in
+// shared memory (x + scale*u for the chunk, and the h window it needs).  The
+// bound is the double-precision pipe (two fused multiply-adds per SM and
+// cycle): a block's time is ROWS N / 2 cycles, so a single evaluation takes the
+// rows per block (8, 16 or 32) that leave the busiest SM the fewest rows.
+// Measured with the partial sums' tree below: N = 1001 16.0 us (20.5 with 32 rows),
+// N = 2048 24.8 (32.9), N = 256 12.0 either way (latency).
+constexpr int kFRows = 32, kFThreads = 256, kFChunk = 256;
 
-// Rows [i0, i0 + kFRows) of F at x + scale u (u may be NULL); returns the
+// Rows [i0, i0 + ROWS) of F at x + scale u (u may be NULL); returns the
 // block's sum of F_i^2 (valid in every thread).
-template <typename TU>
+template <typename TU, int ROWS = kFRows>
 __device__ __forceinline__ double residual_rows(int N, double c, const double* __restrict__ x,
                                                 const TU* __restrict__ u, double scale,
                                                 const double* __restrict__ htab, double* __restrict__ xout,
                                                 double* __restrict__ F, double* __restrict__ rr, int i0)
 {
     __shared__ double xs[kFChunk];
-    __shared__ double hw[kFChunk + kFRows];
-    __shared__ double red[kFSlices][kFRows + 1];
+    constexpr int kFSlices = kFThreads / ROWS;
+    __shared__ double hw[kFChunk + ROWS];
+    __shared__ double red[kFSlices][ROWS + 1];
     __shared__ double bsum;
-    const int r = threadIdx.x % kFRows, q = threadIdx.x / kFRows;
+    const int r = threadIdx.x % ROWS, q = threadIdx.x / ROWS;
     const int i = i0 + r;
     double acc = 0.0;
     for (int j0 = 0; j0 < N; j0 += kFChunk) {
@@ -42,7 +48,7 @@ __device__ __forceinline__ double residual_rows(int N, double c, const double* _
             }
             xs[t] = v;
         }
-        for (int t = threadIdx.x; t < kFChunk + kFRows; t += blockDim.x) {
+        for (int t = threadIdx.x; t < kFChunk + ROWS; t += blockDim.x) {
             int k = i0 + j0 + t;
             hw[t] = (k < 2 * N - 1) ? htab[k] : 0.0;
         }
@@ -66,26 +72,26 @@ __device__ __forceinline__ double residual_rows(int N, double c, const double* _
         rr[i] = ri;
         f2 = fi * fi;
     }
-    // deterministic norm: per-block partial, the last block sums them in order
+    // deterministic norm: per-block partial, the last block sums them
     __syncthreads();
-    if (q == 0) {
+    if (threadIdx.x < 32) {  // (f2 is zero off the first slice)
         double v = f2;
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (r == 0) bsum = v;
+        if (threadIdx.x == 0) bsum = v;
     }
     __syncthreads();
     return bsum;
 }
 
-template <typename TU>
-__global__ void __launch_bounds__(kFRows* kFSlices)
+template <typename TU, int ROWS>
+__global__ void __launch_bounds__(kFThreads)
     k_residual(int N, double c, const double* __restrict__ x, const TU* __restrict__ u, double scale,
                const double* __restrict__ htab, double* __restrict__ xout, double* __restrict__ F,
                double* __restrict__ rr, double* __restrict__ partial, unsigned* __restrict__ counter,
                double* __restrict__ fnorm)
 {
     __shared__ bool last;
-    const double v = residual_rows<TU>(N, c, x, u, scale, htab, xout, F, rr, blockIdx.x * kFRows);
+    const double v = residual_rows<TU, ROWS>(N, c, x, u, scale, htab, xout, F, rr, blockIdx.x * ROWS);
     if (threadIdx.x == 0) partial[blockIdx.x] = v;
     if (threadIdx.x == 0) {
         __threadfence();
@@ -94,9 +100,9 @@ __global__ void __launch_bounds__(kFRows* kFSlices)
     }
     __syncthreads();
     if (last) {
-        __shared__ double buf[kFRows * kFSlices];
+        __shared__ double red[kFThreads / 32];
         __threadfence();
-        const double s = ordered_sum_staged(partial, (int)gridDim.x, buf);
+        const double s = partials_sum(partial, (int)gridDim.x, red);
         if (threadIdx.x == 0) {
             *fnorm = sqrt(s);
             *counter = 0u;
@@ -117,28 +123,41 @@ nl_status launch_htab(int N, double* htab, cudaStream_t st)
     return NL_OK;
 }
 
+template <typename TU, int ROWS>
+static void launch_residual_t(int N, double c, const double* x, const void* u, double scale, const double* htab,
+                              double* xout, double* F, double* rr, double* partial, unsigned* counter, double* fnorm,
+                              cudaStream_t st)
+{
+    k_residual<TU, ROWS><<<(unsigned)cdiv(N, ROWS), kFThreads, 0, st>>>(N, c, x, (const TU*)u, scale, htab, xout, F, rr,
+                                                                       partial, counter, fnorm);
+}
+
 nl_status launch_residual(int N, double c, const double* x, const void* u, int u_is_double, double scale,
                           const double* htab, double* xout, double* F, double* rr, double* partial,
                           unsigned* counter, double* fnorm, cudaStream_t st)
 {
-    unsigned grid = (unsigned)cdiv(N, kFRows);
+    const int sms = num_sms();
+    int rows = kFRows;
+    for (int q : {16, 8})
+        if (cdiv(cdiv(N, q), sms) * q < cdiv(cdiv(N, rows), sms) * rows) rows = q;
+    auto f = u_is_double ? (rows == 8    ? launch_residual_t<double, 8>
+                            : rows == 16 ? launch_residual_t<double, 16>
+                                         : launch_residual_t<double, 32>)
+                         : (rows == 8    ? launch_residual_t<float, 8>
+                            : rows == 16 ? launch_residual_t<float, 16>
+                                         : launch_residual_t<float, 32>);
     prof_begin("k_residual", st);
-    if (u_is_double)
-        k_residual<double><<<grid, kFRows * kFSlices, 0, st>>>(N, c, x, (const double*)u, scale, htab, xout, F,
-                                                               rr, partial, counter, fnorm);
-    else
-        k_residual<float><<<grid, kFRows * kFSlices, 0, st>>>(N, c, x, (const float*)u, scale, htab, xout, F,
-                                                              rr, partial, counter, fnorm);
+    f(N, c, x, u, scale, htab, xout, F, rr, partial, counter, fnorm, st);
     prof_end("k_residual", st);
     NL_CUDA_OK(cudaGetLastError());
     return NL_OK;
 }
 
-int residual_partials(int N) { return (int)cdiv(N, kFRows); }
+int residual_partials(int N) { return (int)cdiv(N, 8); }
 
 // Grouped residual: one block per task {instance, first row}.  Per-instance
-// block partials are summed in block order by the instance's last block.
-__global__ void __launch_bounds__(kFRows* kFSlices)
+// block partials are summed by the instance's last block.
+__global__ void __launch_bounds__(kFThreads)
     k_residual_g(const BInst* __restrict__ inst, BState* __restrict__ st, const BTask* __restrict__ tasks, int mode,
                  const double* __restrict__ htab)
 {
@@ -164,12 +183,14 @@ __global__ void __launch_bounds__(kFRows* kFSlices)
         last = (atomicAdd(&I.cnt[0], 1u) == (unsigned)(nblk - 1));
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
+    if (last) {
+        __shared__ double red[kFThreads / 32];
         __threadfence();
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += __ldcg(&I.part[b]);
-        S.fn = sqrt(s);
-        I.cnt[0] = 0u;
+        const double s = partials_sum(I.part, nblk, red);
+        if (threadIdx.x == 0) {
+            S.fn = sqrt(s);
+            I.cnt[0] = 0u;
+        }
     }
 }
 
@@ -179,7 +200,7 @@ nl_status launch_residual_g(const BInst* inst, BState* st, const BTask* tasks, i
                             const double* htab, cudaStream_t st_)
 {
     if (ntasks <= 0) return NL_OK;
-    k_residual_g<<<(unsigned)ntasks, kFRows * kFSlices, 0, st_>>>(inst, st, tasks, mode, htab);
+    k_residual_g<<<(unsigned)ntasks, kFThreads, 0, st_>>>(inst, st, tasks, mode, htab);
     NL_CUDA_OK(cudaGetLastError());
     return NL_OK;
 }
