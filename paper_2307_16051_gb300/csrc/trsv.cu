@@ -87,7 +87,11 @@ __global__ void __launch_bounds__(1024) k_perm(int N, const int* __restrict__ ip
     int c = 0;
     for (int k = a; k < e; ++k) c += (ipiv[k] != k);
     cnt[tid] = c;
-    __syncthreads();
+    if (!__syncthreads_or(c)) {  // no interchanges (every factorisation of the H-equation): no serial pass
+        for (int i = tid; i < N; i += nt) perm[i] = i;
+        if (tid == 0) list[N] = 0;
+        return;
+    }
     if (tid == 0) {
         int s = 0;
         for (int q = 0; q < nt; ++q) {
@@ -642,70 +646,104 @@ __global__ void __launch_bounds__(TB) k_invdiag_t(int N, const S* __restrict__ L
     for (int i = 0; i < TB; ++i) Uinv[i * TB + col] = x[i * (TB + 1)];
 }
 
-// The binary16 factors' 128 x 128 diagonal-block inverses, the same
-// right-looking recurrences as k_invdiag_t with the column in registers:
-// four threads per column (lane = 4 x column-in-warp + quarter), thread q
-// holding rows 32q..32q+31.  At step t the thread holding row t finalises it
-// and passes x_t to the column's other three threads with one shuffle; every
-// thread then applies x_t to all 32 of its rows with the block's column t
-// (staged transposed in shared memory with the entries the step must not
-// touch — on and above the diagonal for L, on and below it for U — set to
-// zero, so the update needs no per-row test and leaves them unchanged).
-constexpr int kInvThreads = 512;
-constexpr int kInvS = 148;  // transposed column stride (floats): quarters 36 apart; 148 t mod 32 spreads the staging stores
-constexpr size_t kInvSmem = (size_t)T2 * kInvS * sizeof(float) + T2 * sizeof(float);
+// The binary16 factors' 128 x 128 diagonal-block inverses, the recurrences of
+// k_invdiag_t with the terms of every entry in the same order, one thread per
+// column.  The rows are taken in chunks of 32 (from the last one up for U):
+// the chunk's 32 accumulators stay in registers while the finished rows t are
+// applied (the block's column t, staged transposed, is the same for every
+// thread: eight broadcast loads for 32 fused multiply-adds), then the chunk is
+// solved against its own 32 x 32 triangle.  Bound by the multiply-adds of the
+// column with the most rows (192 t of 32 and four triangles).  A warp skips the
+// rows t before (U: after) its 32 columns, where x_t is zero.  Four threads per
+// column, right-looking, each re-reading its 32 entries of column t at every
+// step, took 50 us; this takes 27 us (N <= 2048, launch included).
+constexpr int kInvThreads = 128;
+constexpr int kInvS = 132;  // stride of the transposed block (floats)
+constexpr size_t kInvSmem = (size_t)T2 * kInvS * sizeof(float) + (size_t)T2 * T2 * sizeof(float) + T2 * sizeof(float);
 
 template <bool UPPER>
 __device__ __forceinline__ void invdiag16_pass(const __half* __restrict__ LU, int64_t ld, float* __restrict__ D, int r0,
                                                int nb_)
 {
     extern __shared__ __align__(16) float inv_sm[];
-    float* At = inv_sm;             // At[t * kInvS + 36 q + r]: entry (32 q + r, t)
-    float* dg = inv_sm + T2 * kInvS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int col = warp * 8 + (lane >> 2), q = lane & 3;
-    for (int e = tid; e < T2 * T2; e += kInvThreads) {
-        const int i = e / T2, t = e % T2;  // row i, column t of the block
-        float a = 0.0f;
-        if (i < nb_ && t < nb_) {
-            const float v = __half2float(LU[(int64_t)(r0 + i) * ld + r0 + t]);
-            if (UPPER ? (i < t) : (i > t)) a = UPPER ? -v : v;
-            if (i == t) dg[t] = v;
+    float* At = inv_sm;              // At[t * kInvS + i]: entry (i, t), U's negated
+    float* X = At + T2 * kInvS;      // X[t * T2 + column]
+    float* dg = X + T2 * T2;
+    const int col = threadIdx.x, warp = threadIdx.x >> 5;
+    {
+        const int i = threadIdx.x;  // a row of the block
+        const __half* src = LU + (int64_t)(r0 + min(i, nb_ - 1)) * ld + r0;
+        const bool vec = nb_ == T2 && ((((uintptr_t)(LU + r0)) & 15) == 0) && (ld % 8 == 0);
+#pragma unroll 4
+        for (int t0 = 0; t0 < T2; t0 += 8) {
+            __align__(16) __half h[8];
+            if (vec) {
+                *reinterpret_cast<uint4*>(h) = *reinterpret_cast<const uint4*>(src + t0);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) h[e] = (i < nb_ && t0 + e < nb_) ? src[t0 + e] : __float2half_rn(0.0f);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float v = __half2float(h[e]);
+                At[(t0 + e) * kInvS + i] = UPPER ? -v : v;
+                if (t0 + e == i) dg[i] = v;
+            }
         }
-        At[t * kInvS + 36 * (i >> 5) + (i & 31)] = a;
     }
     __syncthreads();
-    float acc[32];
-#pragma unroll
-    for (int r = 0; r < 32; ++r) acc[r] = (UPPER && 32 * q + r == col && col < nb_) ? 1.0f : 0.0f;
+    const bool live = col < nb_;
     for (int s = 0; s < T2 / 32; ++s) {
-        const int tq = UPPER ? 3 - s : s;
+        const int R = UPPER ? 3 - s : s, i0 = 32 * R;
+        float acc[32];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            const int tt = UPPER ? 31 - k : k;
-            const int t = 32 * tq + tt;
-            float xt = 0.0f;
-            if (q == tq && col < nb_ && t < nb_) {
-                if (UPPER)
-                    xt = (t > col) ? 0.0f : acc[tt] / dg[t];
-                else
-                    xt = (t < col) ? 0.0f : ((t == col) ? 1.0f : -acc[tt]);
-                acc[tt] = xt;
+        for (int r = 0; r < 32; ++r) acc[r] = (UPPER && i0 + r == col && live) ? 1.0f : 0.0f;
+        if (UPPER ? R <= warp : R >= warp) {
+            // finished rows: for L the chunks warp .. R-1 in increasing order, for U warp .. R+1 in decreasing order
+            const int n = 32 * (UPPER ? warp - R : R - warp);
+            int t = UPPER ? 32 * warp + 31 : 32 * warp;
+#pragma unroll 2
+            for (int m = 0; m < n; ++m, t += UPPER ? -1 : 1) {
+                const float xt = X[t * T2 + col];
+                const float4* a4 = reinterpret_cast<const float4*>(At + t * kInvS + i0);
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    const float4 v = a4[g];
+                    acc[4 * g] = fmaf(v.x, xt, acc[4 * g]);
+                    acc[4 * g + 1] = fmaf(v.y, xt, acc[4 * g + 1]);
+                    acc[4 * g + 2] = fmaf(v.z, xt, acc[4 * g + 2]);
+                    acc[4 * g + 3] = fmaf(v.w, xt, acc[4 * g + 3]);
+                }
             }
-            xt = __shfl_sync(0xffffffffu, xt, (lane & ~3) | tq);
-            const float4* a4 = reinterpret_cast<const float4*>(At + t * kInvS + 36 * q);
 #pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                const float4 v = a4[g];
-                acc[4 * g] = fmaf(v.x, xt, acc[4 * g]);
-                acc[4 * g + 1] = fmaf(v.y, xt, acc[4 * g + 1]);
-                acc[4 * g + 2] = fmaf(v.z, xt, acc[4 * g + 2]);
-                acc[4 * g + 3] = fmaf(v.w, xt, acc[4 * g + 3]);
+            for (int k = 0; k < 32; ++k) {
+                const int tt = UPPER ? 31 - k : k, t = i0 + tt;
+                float xt = 0.0f;
+                if (live && t < nb_) {
+                    if (UPPER) xt = (t > col) ? 0.0f : acc[tt] / dg[t];
+                    else xt = (t < col) ? 0.0f : ((t == col) ? 1.0f : -acc[tt]);
+                }
+                acc[tt] = xt;
+                const float4* a4 = reinterpret_cast<const float4*>(At + t * kInvS + i0);
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {
+                    if (UPPER ? 4 * g >= tt : 4 * g + 3 <= tt) continue;
+                    const float4 v = a4[g];
+                    const float a[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int i = 4 * g + e;
+                        if (UPPER ? i < tt : i > tt) acc[i] = fmaf(a[e], xt, acc[i]);
+                    }
+                }
             }
         }
-    }
 #pragma unroll
-    for (int r = 0; r < 32; ++r) D[(32 * q + r) * T2 + col] = acc[r];
+        for (int r = 0; r < 32; ++r) {
+            X[(i0 + r) * T2 + col] = acc[r];  // (read back by this thread only)
+            D[(i0 + r) * T2 + col] = acc[r];
+        }
+    }
 }
 
 // CTA b < nblk: L^{-1} of block b; CTA nblk + b: U^{-1} of block b (U's
