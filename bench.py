@@ -151,7 +151,7 @@ def kernel_rooflines(nl, step, N, hbm_peak, tc_peak, lookahead=True):
         "k_tc_gemm": ("tensor", rest_flop if lookahead else gemm_flop, tc_peak, "TFLOP/s",
                       "measured bf16 dense (fp16 same rate)"),
         "k_tc_gemm_x": ("tensor", cross_flop, tc_peak, "TFLOP/s", "measured bf16 dense (fp16 same rate)"),
-        "k_trsv_cl": ("hbm", trsv_bytes, hbm_peak, "GB/s", "measured copy bandwidth"),
+        "k_trsv_cl": ("hbm", 2 * trsv_bytes, hbm_peak, "GB/s", "measured copy bandwidth"),
         "k_trsv_mb": ("hbm", trsv_bytes, hbm_peak, "GB/s", "measured copy bandwidth"),
         "k_gemv_residual": ("hbm", gemv_bytes, hbm_peak, "GB/s", "measured copy bandwidth"),
     }
@@ -272,7 +272,7 @@ def bench_large(nl, torch, dev, hbm_peak, tc_peak, N=32768, c=0.99, fp64=True, r
     T2 = 128
     nblk = (N + T2 - 1) // T2
     work = {"k_gemv_residual": 4.0 * N * N + 12.0 * N,
-            "k_trsv_cl": (N * N / 2.0) * 2 + nblk * T2 * T2 * 4 + 12.0 * N,
+            "k_trsv_cl": 2 * ((N * N / 2.0) * 2 + nblk * T2 * T2 * 4 + 12.0 * N),  # both triangles
             "k_trsv_mb": (N * N / 2.0) * 2 + nblk * T2 * T2 * 4 + 12.0 * N,
             "k_tc_gemm": None}
     for name in ("k_gemv_residual", "k_trsv_cl", "k_trsv_mb", "k_tc_gemm"):

@@ -96,17 +96,17 @@ typedef struct {
                             launch with 64 x 64 / 128 x 64 SIMT update tiles (nb <= 64), 5 = one
                             persistent launch with 128 x 128 tcgen05 update tiles (nb = 64) */
     int lu_path;         /* [0 = auto] no-interchange fast path with exact fallback; 1 = interchanging path only */
-    int trsv_cluster;    /* [0 = auto] half-precision triangular solves: one thread-block cluster per
-                            triangle of at most 16 CTAs (the largest of 16, 8, 4 the device can
-                            co-schedule) for N <= 10240, else one launch of independent CTAs per
+    int trsv_cluster;    /* [0 = auto] half-precision triangular solves: one thread-block cluster of
+                            at most 16 CTAs for both triangles (the largest of 16, 8, 4 the device can
+                            co-schedule) for N <= 3072, else one launch of independent CTAs per
                             triangle that hand solved entries over global memory; 4, 8 or 16 caps
                             the cluster size (any N); -1 = always the global-memory hand-off */
     int lu_stream;       /* [0 = auto] half-precision fast path: the diagonal block and the off-diagonal
-                            solves of a panel in one cooperative launch, the solves streaming one
-                            column behind the diagonal block (when its CTAs fit on the GPU at once),
-                            128 rows per CTA where possible; 256 = the same with 256 rows per CTA
-                            (half the SMs, for solves that share the GPU); -1 = two launches per
-                            panel.  Bitwise the same factors in every case */
+                            solves of a panel in one launch, the solves streaming one block of eight
+                            columns behind the diagonal block, 64 rows per CTA while all CTAs fit on
+                            the GPU at once, else 128; 256 = the same with 256 rows per CTA (fewer
+                            SMs, for solves that share the GPU); -1 = two launches per panel.
+                            Bitwise the same factors in every case */
     int ir_variant;      /* [0] IR correction (NL_IR16, and the IR part of NL_IR16_GMRES): 0 = on the
                             fly, d = U^{-1} L^{-1} r with the binary16 factors promoted to single
                             (eq. (2.16) applied to IR); 1 = the scaled half-precision correction of

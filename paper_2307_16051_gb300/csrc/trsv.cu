@@ -211,7 +211,6 @@ __global__ void __launch_bounds__(kTrsvThreads) k_trsv(int N, int nblk, const S*
 // (64 KB) is staged in shared memory and each thread prefetches its 64
 // binary16 entries of the next tile before polling.
 constexpr int T2 = 128;
-constexpr int kMbThreads = 256;  // 128 rows x 2 halves of 64 columns
 
 // A published word carries its own readiness (the epoch) and its value, and a
 // consumer reads nothing else the producer wrote, so relaxed GPU-scope accesses
@@ -225,6 +224,93 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v)
 {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// A 128 x 128 tile times a vector by 512 threads, as both half-precision solves
+// do it: lane cg = lane & 15 of a half warp takes eight columns of the four rows
+// 4 (2 warp + lane / 16).., so a row is read by 16 neighbouring lanes (whole lines),
+// a thread reads eight of the vector's entries for four rows, and the 16 lanes'
+// sums are reduced with five shuffles, which leave row e(lane) in the lane.
+// (A row quarter per thread read the whole vector from shared memory for one
+// row and every matrix line in eight pieces: twice the time per tile.)
+// Vectors of 128 floats are padded to 144 (column c at c + 4 (c / 32)).
+constexpr int kTvThreads = 512;
+constexpr int kTvPad = 144;
+__device__ __forceinline__ int tv_pos(int c) { return c + 4 * (c >> 5); }
+// rows i0 .. i0 + 3, columns c0 .. c0 + 7 (zeros outside the matrix)
+template <bool STREAM>
+__device__ __forceinline__ void tv_load_tile(const __half* __restrict__ LU, int64_t ld, int N, int i0, int c0, bool vecld,
+                                             uint4 (&t)[4])
+{
+    const bool vec = vecld && c0 + 8 <= N;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __half* src = LU + (int64_t)(i0 + e) * ld + c0;
+        if (vec && i0 + e < N) {
+            t[e] = STREAM ? __ldcs(reinterpret_cast<const uint4*>(src)) : *reinterpret_cast<const uint4*>(src);
+        } else {
+            __half h[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) h[k] = (i0 + e < N && c0 + k < N) ? src[k] : __float2half_rn(0.0f);
+            memcpy(&t[e], h, 16);
+        }
+    }
+}
+// p[e] += row e of the tile times z (the padded vector's entries 8 cg .. 8 cg + 7)
+__device__ __forceinline__ void tv_dot_tile(const uint4 (&t)[4], const float* __restrict__ z, float (&p)[4])
+{
+    const float4 a = *reinterpret_cast<const float4*>(z), b = *reinterpret_cast<const float4*>(z + 4);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __half2* h = reinterpret_cast<const __half2*>(&t[e]);
+        const float2 f0 = __half22float2(h[0]), f1 = __half22float2(h[1]), f2 = __half22float2(h[2]),
+                     f3 = __half22float2(h[3]);
+        p[e] = fmaf(f0.x, a.x, p[e]);
+        p[e] = fmaf(f0.y, a.y, p[e]);
+        p[e] = fmaf(f1.x, a.z, p[e]);
+        p[e] = fmaf(f1.y, a.w, p[e]);
+        p[e] = fmaf(f2.x, b.x, p[e]);
+        p[e] = fmaf(f2.y, b.y, p[e]);
+        p[e] = fmaf(f3.x, b.z, p[e]);
+        p[e] = fmaf(f3.y, b.w, p[e]);
+    }
+}
+// rows i0 .. i0 + 3 of a 128 x 128 inverse: columns 4 cg .. and 64 + 4 cg ..
+__device__ __forceinline__ void tv_load_inv(const float* __restrict__ D, int i0, int cg, float4 (&dq)[8])
+{
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        dq[2 * e] = *reinterpret_cast<const float4*>(D + (i0 + e) * T2 + 4 * cg);
+        dq[2 * e + 1] = *reinterpret_cast<const float4*>(D + (i0 + e) * T2 + 64 + 4 * cg);
+    }
+}
+__device__ __forceinline__ void tv_dot_inv(const float4 (&dq)[8], const float* __restrict__ acc, int cg, float (&p)[4])
+{
+    const float4 a = *reinterpret_cast<const float4*>(acc + tv_pos(4 * cg)),
+                 b = *reinterpret_cast<const float4*>(acc + tv_pos(64 + 4 * cg));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        p[e] = dq[2 * e].x * a.x;
+        p[e] = fmaf(dq[2 * e].y, a.y, p[e]);
+        p[e] = fmaf(dq[2 * e].z, a.z, p[e]);
+        p[e] = fmaf(dq[2 * e].w, a.w, p[e]);
+        p[e] = fmaf(dq[2 * e + 1].x, b.x, p[e]);
+        p[e] = fmaf(dq[2 * e + 1].y, b.y, p[e]);
+        p[e] = fmaf(dq[2 * e + 1].z, b.z, p[e]);
+        p[e] = fmaf(dq[2 * e + 1].w, b.w, p[e]);
+    }
+}
+// The sum over the 16 lanes of row e(lane) = 2 (lane & 1) + (lane / 2 & 1).
+__device__ __forceinline__ int tv_row(int lane) { return 2 * (lane & 1) + ((lane >> 1) & 1); }
+__device__ __forceinline__ float tv_reduce(const float (&p)[4], int lane)
+{
+    const bool b0 = lane & 1, b1 = lane & 2;
+    const float s0 = __shfl_xor_sync(0xffffffffu, b0 ? p[0] : p[2], 1), s1 = __shfl_xor_sync(0xffffffffu, b0 ? p[1] : p[3], 1);
+    const float q0 = (b0 ? p[2] : p[0]) + s0, q1 = (b0 ? p[3] : p[1]) + s1;
+    float v = (b1 ? q1 : q0) + __shfl_xor_sync(0xffffffffu, b1 ? q0 : q1, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    return v;
 }
 
 // Bounded poll of one published entry: false once `limit` cycles have passed
@@ -247,7 +333,7 @@ __device__ __forceinline__ bool poll_value(const unsigned long long* p, unsigned
 }
 
 template <bool LOWER>
-__global__ void __launch_bounds__(kMbThreads) k_trsv_mb(int N, int nblk, const __half* __restrict__ LU, int64_t ld,
+__global__ void __launch_bounds__(kTvThreads, 1) k_trsv_mb(int N, int nblk, const __half* __restrict__ LU, int64_t ld,
                                                        const float* __restrict__ v,
                                                        const unsigned long long* __restrict__ vin_mb,
                                                        const int* __restrict__ perm, const float* __restrict__ dinv,
@@ -255,87 +341,64 @@ __global__ void __launch_bounds__(kMbThreads) k_trsv_mb(int N, int nblk, const _
                                                        unsigned epoch, unsigned* __restrict__ err, long long wait_cycles,
                                                        const float* __restrict__ rs)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* Ds = reinterpret_cast<float*>(smem_raw);  // T2 x T2 diagonal inverse
-    __shared__ float ys[T2];
-    __shared__ float acc[T2];
-    const int tid = threadIdx.x, r = tid >> 1, h = tid & 1;
+    __shared__ __align__(16) float ys[2][kTvPad];  // the tile's vector, alternating
+    __shared__ __align__(16) float acc[kTvPad];
+    const int tid = threadIdx.x, lane = tid & 31, cg = lane & 15;
+    const int row4 = 4 * (2 * (tid >> 5) + (lane >> 4));  // this thread's four rows of a block
+    const bool vecld = ((((uintptr_t)LU) & 15) == 0) && (ld % 8 == 0);
     const float* Dinv = dinv + (LOWER ? 0 : (int64_t)nblk * T2 * T2);
     for (int g = blockIdx.x; g < nblk; g += gridDim.x) {
         const int b = LOWER ? g : nblk - 1 - g;
-        const int r0 = b * T2, row = r0 + r;
-        // stage this block's diagonal inverse (independent of the waits)
+        const int r0 = b * T2;
         __syncthreads();
-        {
-            const float4* src = reinterpret_cast<const float4*>(Dinv + (int64_t)b * T2 * T2);
-            float4* dst = reinterpret_cast<float4*>(Ds);
-            for (int q = tid; q < T2 * T2 / 4; q += kMbThreads) dst[q] = src[q];
-        }
+        float4 dq[8];  // this thread's part of the block's diagonal inverse (independent of the waits)
+        tv_load_inv(Dinv + (int64_t)b * T2 * T2, row4, cg, dq);
         if (tid < T2) {
             const int i = r0 + tid;
             float x = 0.0f;
             if (i < N)
                 x = LOWER ? (rs ? v[perm[i]] * rs[perm[i]] : v[perm[i]]) : __uint_as_float((unsigned)vin_mb[i]);
-            acc[tid] = x;
+            acc[tv_pos(tid)] = x;
         }
-        float part = 0.0f;
-        const __half* Lrow = LU + (int64_t)min(row, N - 1) * ld;
+        float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         const int cnt = LOWER ? b : nblk - 1 - b;
-        // this thread's 64 entries of tile (b, c), loaded one tile ahead of their use
-        auto fetch = [&](int c, __half2* dst) {
-            const int cb = c * T2 + h * 64;
-            if (row < N && cb + 64 <= N && (((uintptr_t)(Lrow + cb)) & 15) == 0) {
-                const uint4* p4 = reinterpret_cast<const uint4*>(Lrow + cb);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    uint4 u = __ldcs(p4 + q);  // streamed once: do not keep it in the caches
-                    memcpy(&dst[4 * q], &u, 16);
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 32; ++q) {
-                    int c0 = cb + 2 * q;
-                    float a0 = (row < N && c0 < N) ? __half2float(Lrow[c0]) : 0.0f;
-                    float a1 = (row < N && c0 + 1 < N) ? __half2float(Lrow[c0 + 1]) : 0.0f;
-                    dst[q] = __floats2half2_rn(a0, a1);
-                }
-            }
-        };
-        __half2 lv[32], nx[32];
-        if (cnt > 0) fetch(LOWER ? 0 : nblk - 1, lv);
-        for (int s = 0; s < cnt; ++s) {
+        // tile (b, c): its entries are loaded two tiles ahead of their use, streamed once (not kept in the caches)
+        auto fetch = [&](int s, uint4 (&t)[4]) {
             const int c = LOWER ? s : nblk - 1 - s;
-            if (s + 1 < cnt) fetch(LOWER ? s + 1 : nblk - 2 - s, nx);
-            __syncthreads();  // ys of the previous tile no longer in use
-            bool okp = true;
-            if (tid < T2) {
-                const int i = c * T2 + tid;
-                float y = 0.0f;
-                if (i < N) okp = poll_value(mb + i, epoch, &y, err, wait_cycles);
-                ys[tid] = y;
-            }
-            if (__syncthreads_or(!okp)) {
+            tv_load_tile<true>(LU, ld, N, r0 + row4, c * T2 + 8 * cg, vecld, t);
+        };
+        auto poll = [&](int s) -> bool {  // threads 0..127: the vector of tile s
+            if (tid >= T2) return true;
+            const int i = (LOWER ? s : nblk - 1 - s) * T2 + tid;
+            float y = 0.0f;
+            const bool okp = i >= N || poll_value(mb + i, epoch, &y, err, wait_cycles);
+            ys[s & 1][tv_pos(tid)] = y;
+            return okp;
+        };
+        uint4 t0[4], t1[4], t2[4];
+        if (cnt > 0) fetch(0, t0);
+        if (cnt > 1) fetch(1, t1);
+        for (int s = 0; s < cnt; ++s) {
+            if (s + 2 < cnt) fetch(s + 2, t2);
+            if (__syncthreads_or(!poll(s))) {  // (the other buffer's readers are at most one tile behind)
                 if (tid == 0) atomicOr(err, (unsigned)ERR_TIMEOUT_TRSV);
                 return;
             }
+            tv_dot_tile(t0, ys[s & 1] + tv_pos(8 * cg), p);
 #pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                float2 f = __half22float2(lv[q]);
-                part = fmaf(f.x, ys[h * 64 + 2 * q], part);
-                part = fmaf(f.y, ys[h * 64 + 2 * q + 1], part);
+            for (int q = 0; q < 4; ++q) {
+                t0[q] = t1[q];
+                t1[q] = t2[q];
             }
-#pragma unroll
-            for (int q = 0; q < 32; ++q) lv[q] = nx[q];
         }
-        part += __shfl_xor_sync(0xffffffffu, part, 1);
+        const float part = tv_reduce(p, lane);
+        if (cnt == 0) __syncthreads();  // (acc was written by other threads; with tiles the loop's barriers passed)
+        if (cg < 4) acc[tv_pos(row4 + tv_row(lane))] -= part;
         __syncthreads();
-        if (h == 0) acc[r] -= part;
-        __syncthreads();
-        float sum = 0.0f;
-#pragma unroll 16
-        for (int k = 0; k < 64; ++k) sum = fmaf(Ds[r * T2 + h * 64 + k], acc[h * 64 + k], sum);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        if (h == 0 && row < N) {
+        tv_dot_inv(dq, acc, cg, p);
+        const float sum = tv_reduce(p, lane);
+        const int row = r0 + row4 + tv_row(lane);
+        if (cg < 4 && row < N) {
             if (out) out[row] = sum;
             st_relaxed_u64(mb + row, ((unsigned long long)epoch << 32) | __float_as_uint(sum));
         }
@@ -343,27 +406,30 @@ __global__ void __launch_bounds__(kMbThreads) k_trsv_mb(int N, int nblk, const _
 }
 
 // ------------------------------------------------ cluster triangular solve --
-// One thread-block cluster of C CTAs (C <= 16) solves the whole triangle.
-// Block b of 128 rows belongs to CTA (step of b) mod C, which keeps the
+// One thread-block cluster of C CTAs (C <= 16) solves both triangles in one
+// launch.  Block b of 128 rows belongs to CTA (step of b) mod C, which keeps the
 // running right-hand side of its blocks in shared memory.  The owner of step
 // s forms z_b = Dinv_b acc_b and stores z_b into every CTA's shared memory
-// with st.async, each store completing a transaction count on that CTA's
-// mbarrier for step s (one mbarrier per block, used once).  A CTA waits
+// with st.async (16 bytes a lane: one instruction per warp for all 16 CTAs),
+// each store completing a transaction count on that CTA's mbarrier for step s
+// (one mbarrier per block and triangle, used once).  A CTA waits
 // only for the z it needs next; the owner of step s+1 first subtracts
 // L(b(s+1), b(s)) z_s, with the tile already in registers, then publishes
 // z_{b(s+1)} before it applies z_s to its other blocks, so the chain from
-// one block to the next is one shared-memory signal, one 128 x 32 update
-// per thread group and one 128 x 128 product with the inverse (also held
-// in registers).  Every row of the factor is read by exactly one CTA.
-// Shared vectors of 128 floats are padded to 132 (column c at c + c/32) so
-// the four column quarters fall in different banks.
-constexpr int kClThreads = 512;  // 128 rows x 4 column quarters of 32
-constexpr int kClPad = 132;
+// one block to the next is one shared-memory signal and two 128 x 128
+// products (tile and inverse, both held in registers).  The tiles off the chain are loaded one ahead of their use.
+// Every row of the factor is read by exactly one CTA.  Bound by the chain
+// (2 N / 128 steps) up to N = 4096 or so, above it by the 16 SMs' share of L2 and
+// HBM bandwidth.  Measured per solve pair: N = 256 12.5, 1024 26, 2048 49, 4096 102 us
+// (two launches, each element stored to each CTA by itself, and tiles loaded
+// when used: 20, 35, 58, 124).
+constexpr int kClThreads = kTvThreads;
+constexpr int kClPad = kTvPad;
 constexpr int kClMaxSmem = 220 * 1024;
 constexpr long long kClWaitIters = 1LL << 24;
 
-// Dynamic shared memory: nblk mbarriers, then nblk + nown padded vectors.
-__host__ __device__ inline int trsv_cl_bar_bytes(int nblk) { return (nblk * 8 + 15) & ~15; }
+// Dynamic shared memory: 2 nblk mbarriers, then nblk + nown padded vectors.
+__host__ __device__ inline int trsv_cl_bar_bytes(int nblk) { return nblk * 16; }
 inline size_t trsv_cl_smem(int nblk, int nown)
 {
     return (size_t)trsv_cl_bar_bytes(nblk) + (size_t)(nblk + nown) * kClPad * sizeof(float);
@@ -379,10 +445,11 @@ __device__ __forceinline__ uint32_t cl_mapa(uint32_t a, int rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void cl_st_async(uint32_t addr, float v, uint32_t bar)
+__device__ __forceinline__ void cl_st_async4(uint32_t addr, const float (&v)[4], uint32_t bar)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr),
-                 "r"(__float_as_uint(v)), "r"(bar)
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                 "r"(__float_as_uint(v[3])), "r"(bar)
                  : "memory");
 }
 // Bounded wait for phase 0 of a local mbarrier; false after `iters` polls
@@ -402,144 +469,104 @@ __device__ __forceinline__ bool cl_wait(uint32_t bar, long long iters = kClWaitI
     return false;
 }
 
-// Row i of the factor, columns c0 .. c0+31 (zeros outside the matrix).
-__device__ __forceinline__ void cl_load_tile(const __half* __restrict__ LU, int64_t ld, int N, int i, int c0,
-                                             bool vecld, uint4 (&t)[4])
-{
-    if (i < N && vecld && c0 + 32 <= N) {
-        const uint4* p = reinterpret_cast<const uint4*>(LU + (int64_t)i * ld + c0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) t[q] = p[q];
-    } else {
-        __half h[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-            h[k] = (i < N && c0 + k < N) ? LU[(int64_t)i * ld + c0 + k] : __float2half_rn(0.0f);
-        memcpy(t, h, 64);
-    }
-}
-__device__ __forceinline__ float cl_dot_tile(const uint4 (&t)[4], const float* __restrict__ z)
-{
-    float part = 0.0f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const __half2* h2 = reinterpret_cast<const __half2*>(&t[q]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 f = __half22float2(h2[e]);
-            part = fmaf(f.x, z[8 * q + 2 * e], part);
-            part = fmaf(f.y, z[8 * q + 2 * e + 1], part);
-        }
-    }
-    return part;
-}
+struct ClState {
+    int N, nblk, C, rank, nown;
+    const __half* LU;
+    int64_t ld;
+    bool vecld;
+    float *yv, *acc;
+    int* abort_cta;
+    unsigned* err;
+    long long wait_iters;
+};
 
+// One triangle: acc holds the right-hand side of this CTA's blocks (in the
+// triangle's block order), bar its nblk mbarriers; the solution is left in
+// every CTA's yv and, if out is given, written there.
 template <bool LOWER>
-__global__ void __launch_bounds__(kClThreads, 1) k_trsv_cl(int N, int nblk, const __half* __restrict__ LU, int64_t ld,
-                                                       const float* __restrict__ v, const int* __restrict__ perm,
-                                                       const float* __restrict__ dinv, float* __restrict__ out,
-                                                       unsigned* __restrict__ err, long long wait_iters,
-                                                       const float* __restrict__ rs)
+__device__ __forceinline__ void cl_triangle(const ClState& S, const float* __restrict__ Dinv, uint64_t* bar,
+                                            float* __restrict__ out)
 {
-    cg::cluster_group cl = cg::this_cluster();
-    const int C = (int)cl.num_blocks();
-    const int rank = (int)cl.block_rank();
-    extern __shared__ __align__(16) unsigned char cl_raw[];
-    uint64_t* bar = reinterpret_cast<uint64_t*>(cl_raw);
-    float* yv = reinterpret_cast<float*>(cl_raw + trsv_cl_bar_bytes(nblk));  // solved blocks, padded
-    float* acc = yv + (size_t)nblk * kClPad;                                       // this CTA's blocks, padded
-    __shared__ int abort_cta;
-    const int tid = threadIdx.x, row = tid >> 2, qq = tid & 3;
-    const int prow = row + (row >> 5);  // padded position of this row
-    const float* Dinv = dinv + (LOWER ? 0 : (int64_t)nblk * T2 * T2);
-    const int nown = (nblk - rank + C - 1) / C;
-    const bool vecld = ((((uintptr_t)LU) & 15) == 0) && ((ld * 2) % 16 == 0);
+    const int tid = threadIdx.x, lane = tid & 31, cg = lane & 15;
+    const int row4 = 4 * (2 * (tid >> 5) + (lane >> 4));  // this thread's four rows of a block
+    const int prow = tv_pos(row4 + tv_row(lane));         // padded position of the row whose sum it gets
+    const int C = S.C, rank = S.rank, nblk = S.nblk, nown = S.nown, N = S.N;
+    float* yv = S.yv;
+    float* acc = S.acc;
     auto blk = [&](int s) { return LOWER ? s : nblk - 1 - s; };
-    for (int j = 0; j < nown; ++j) {
-        const int bj = blk(rank + j * C);
-        for (int t = tid; t < T2; t += kClThreads) {
-            const int i = bj * T2 + t;
-            acc[j * kClPad + t + (t >> 5)] =
-                (i < N) ? (LOWER ? (rs ? v[perm[i]] * rs[perm[i]] : v[perm[i]]) : v[i]) : 0.0f;
-        }
-    }
-    if (tid == 0) {
-        abort_cta = 0;
-        for (int s = 0; s < nblk; ++s) {
-            const uint32_t a = cl_smem_u32(bar + s);
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a));
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(T2 * 4) : "memory");
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    cl.sync();  // barriers initialised and every CTA running before the first remote store
-
-    float4 dq[8];  // this thread's quarter of row `row` of the inverse of the next block it publishes
-    uint4 ct[4];   // its 32 factor entries of the next tile on its chain
-    auto load_D = [&](int b) {
-        const float4* D = reinterpret_cast<const float4*>(Dinv + (int64_t)b * T2 * T2 + row * T2 + qq * 32);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) dq[k] = D[k];
+    float4 dq[8];  // this thread's part of the inverse of the next block it publishes
+    uint4 ct[4];   // its factor entries of the next tile on its chain
+    uint4 nt[4];   // and of the next tile off the chain
+    auto load_D = [&](int b) { tv_load_inv(Dinv + (int64_t)b * T2 * T2, row4, cg, dq); };
+    auto load_tile = [&](int sb, int sc, uint4 (&t)[4]) {  // rows of step sb's block, columns of step sc's
+        tv_load_tile<false>(S.LU, S.ld, N, blk(sb) * T2 + row4, blk(sc) * T2 + 8 * cg, S.vecld, t);
+    };
+    // this CTA's first block off the chain at step s (the chain's is step s + 1's)
+    auto first_off = [&](int s) {
+        const int j = (s < rank) ? 0 : (s - rank) / C + 1;  // its blocks solved after step s
+        return (j < nown && rank + j * C == s + 1) ? j + 1 : j;
+    };
+    // acc of its block j minus a tile times z
+    auto apply = [&](int j, const uint4 (&t)[4], const float* z) {
+        float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        tv_dot_tile(t, z + tv_pos(8 * cg), p);
+        const float part = tv_reduce(p, lane);
+        if (cg < 4) acc[j * kClPad + prow] -= part;
     };
     // z_b = Dinv_b acc_b for the step s this CTA owns, stored into every CTA
     auto publish = [&](int s) {
         const int b = blk(s);
-        const float* a = acc + (s / C) * kClPad + qq * 33;
-        float sum = 0.0f;
+        float p[4];
+        tv_dot_inv(dq, acc + (s / C) * kClPad, cg, p);
+        const float sum = tv_reduce(p, lane);
+        // lane: its half warp's four rows to CTA cg
+        float v[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            sum = fmaf(dq[k].x, a[4 * k], sum);
-            sum = fmaf(dq[k].y, a[4 * k + 1], sum);
-            sum = fmaf(dq[k].z, a[4 * k + 2], sum);
-            sum = fmaf(dq[k].w, a[4 * k + 3], sum);
-        }
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        if (qq == 0) {
-            const uint32_t ya = cl_smem_u32(yv + (size_t)b * kClPad + prow), ba = cl_smem_u32(bar + s);
-            for (int c = 0; c < C; ++c) cl_st_async(cl_mapa(ya, c), sum, cl_mapa(ba, c));
-            const int i = b * T2 + row;
+        for (int e = 0; e < 4; ++e) v[e] = __shfl_sync(0xffffffffu, sum, (lane & 0x1c) | (e >> 1) | ((e & 1) << 1));
+        if (cg < C)
+            cl_st_async4(cl_mapa(cl_smem_u32(yv + (size_t)b * kClPad + tv_pos(row4)), cg), v,
+                         cl_mapa(cl_smem_u32(bar + s), cg));
+        if (out && cg < 4) {
+            const int i = b * T2 + row4 + tv_row(lane);
             if (i < N) out[i] = sum;
         }
         if (s + C < nblk) {
             // inverse and chain tile for this CTA's next step s + C
             load_D(blk(s + C));
-            cl_load_tile(LU, ld, N, blk(s + C) * T2 + row, blk(s + C - 1) * T2 + qq * 32, vecld, ct);
+            load_tile(s + C, s + C - 1, ct);
         }
     };
     if (rank < nblk) load_D(blk(rank));
-    if (rank >= 1 && rank < nblk) cl_load_tile(LU, ld, N, blk(rank) * T2 + row, blk(rank - 1) * T2 + qq * 32, vecld, ct);
+    if (rank >= 1 && rank < nblk) load_tile(rank, rank - 1, ct);
     if (rank == 0) publish(0);
+    if (first_off(0) < nown) load_tile(rank + first_off(0) * C, 0, nt);
     for (int s = 0; s < nblk; ++s) {
         const int b = blk(s);
         bool ok = false;
-        if (!*((volatile int*)&abort_cta)) {
-            ok = cl_wait(cl_smem_u32(bar + s), wait_iters);
+        if (!*((volatile int*)S.abort_cta)) {
+            ok = cl_wait(cl_smem_u32(bar + s), S.wait_iters);
             if (!ok) {
-                abort_cta = 1;
-                atomicOr(err, (unsigned)ERR_TIMEOUT_TRSV);
+                *S.abort_cta = 1;
+                atomicOr(S.err, (unsigned)ERR_TIMEOUT_TRSV);
             }
         }
-        const float* z = yv + (size_t)b * kClPad + qq * 33;
+        const float* z = yv + (size_t)b * kClPad;
         int j = (s < rank) ? 0 : (s - rank) / C + 1;  // this CTA's blocks solved after step s
         if (j < nown && rank + j * C == s + 1) {
             // next block on the chain: update with the tile already in registers, then publish it
-            const float part0 = ok ? cl_dot_tile(ct, z) : 0.0f;
-            float part = part0 + __shfl_xor_sync(0xffffffffu, part0, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            if (qq == 0) acc[j * kClPad + prow] -= part;
+            if (ok) apply(j, ct, z);
             __syncthreads();
             publish(s + 1);
             ++j;
         }
-        if (!ok) continue;
+        const int jn = s + 1 < nblk ? first_off(s + 1) : nown;  // the next step's first tile
         for (; j < nown; ++j) {
             uint4 t[4];
-            cl_load_tile(LU, ld, N, blk(rank + j * C) * T2 + row, b * T2 + qq * 32, vecld, t);
-            float part = cl_dot_tile(t, z);
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            if (qq == 0) acc[j * kClPad + prow] -= part;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t[q] = nt[q];
+            if (j + 1 < nown) load_tile(rank + (j + 1) * C, s, nt);
+            else if (jn < nown) load_tile(rank + jn * C, s + 1, nt);
+            if (ok) apply(j, t, z);
         }
     }
     // After a wait gave up, the owners of the later steps still publish them
@@ -547,8 +574,59 @@ __global__ void __launch_bounds__(kClThreads, 1) k_trsv_cl(int N, int nblk, cons
     // wait for all of them (the default bound) before leaving, so that no
     // st.async into this CTA's shared memory is still in flight when it exits.
     __syncthreads();
-    if (*((volatile int*)&abort_cta))
+    if (*((volatile int*)S.abort_cta))
         for (int s = 0; s < nblk; ++s) cl_wait(cl_smem_u32(bar + s));
+}
+
+__global__ void __launch_bounds__(kClThreads, 1) k_trsv_cl(int N, int nblk, const __half* __restrict__ LU, int64_t ld,
+                                                       const float* __restrict__ v, const int* __restrict__ perm,
+                                                       const float* __restrict__ dinv, float* __restrict__ out,
+                                                       unsigned* __restrict__ err, long long wait_iters,
+                                                       const float* __restrict__ rs)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char cl_raw[];
+    __shared__ int abort_cta;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(cl_raw);
+    ClState S;
+    S.N = N;
+    S.nblk = nblk;
+    S.C = (int)cl.num_blocks();
+    S.rank = (int)cl.block_rank();
+    S.nown = (nblk - S.rank + S.C - 1) / S.C;
+    S.LU = LU;
+    S.ld = ld;
+    S.vecld = ((((uintptr_t)LU) & 15) == 0) && ((ld * 2) % 16 == 0);
+    S.yv = reinterpret_cast<float*>(cl_raw + trsv_cl_bar_bytes(nblk));  // solved blocks, padded
+    S.acc = S.yv + (size_t)nblk * kClPad;                                // this CTA's blocks, padded
+    S.abort_cta = &abort_cta;
+    S.err = err;
+    S.wait_iters = wait_iters;
+    const int tid = threadIdx.x;
+    for (int j = 0; j < S.nown; ++j)
+        for (int t = tid; t < T2; t += kClThreads) {
+            const int i = (S.rank + j * S.C) * T2 + t;
+            S.acc[j * kClPad + tv_pos(t)] = (i < N) ? (rs ? v[perm[i]] * rs[perm[i]] : v[perm[i]]) : 0.0f;
+        }
+    if (tid == 0) abort_cta = 0;
+    for (int s = tid; s < 2 * nblk; s += kClThreads) {
+        const uint32_t a = cl_smem_u32(bar + s);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(a));
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(T2 * 4) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cl.sync();  // barriers initialised and every CTA running before the first remote store
+    cl_triangle<true>(S, dinv, bar, nullptr);
+    // every CTA holds all of y and has used it: the blocks' right-hand sides of the
+    // upper triangle, whose solution overwrites it
+    cl.sync();
+    for (int j = 0; j < S.nown; ++j)
+        for (int t = tid; t < T2; t += kClThreads) {
+            const int p = tv_pos(t), b = nblk - 1 - (S.rank + j * S.C);
+            S.acc[j * kClPad + p] = (b * T2 + t < N) ? S.yv[(size_t)b * kClPad + p] : 0.0f;
+        }
+    cl.sync();  // (read before any CTA publishes into yv)
+    cl_triangle<false>(S, dinv + (int64_t)nblk * T2 * T2, bar + nblk, out);
     cl.sync();  // no CTA leaves before every CTA has passed all of its waits
 }
 
@@ -851,12 +929,10 @@ static nl_status launch_trsv_mb(int N, const __half* LU, int64_t ld, const float
 {
     const int nblk = (int)cdiv(N, T2);
     auto kern = k_trsv_mb<LOWER>;
-    const size_t smem = (size_t)T2 * T2 * sizeof(float);
     static int max_grid = 0;
     if (max_grid == 0) {
-        if (set_max_dynamic_smem((const void*)kern) != NL_OK) return NL_ECUDA;
         int per_sm = 0;
-        NL_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMbThreads, smem));
+        NL_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTvThreads, 0));
         max_grid = std::max(1, per_sm) * num_sms();
     }
     int grid = std::min(nblk, max_grid);
@@ -868,7 +944,7 @@ static nl_status launch_trsv_mb(int N, const __half* LU, int64_t ld, const float
     void* args[] = {(void*)&N,   (void*)&nblk, (void*)&LU,  (void*)&ld,    (void*)&v,   (void*)&vin_mb, (void*)&perm,
                     (void*)&dinv, (void*)&mb, (void*)&out, (void*)&epoch, (void*)&err, (void*)&wait, (void*)&rs};
     prof_begin("k_trsv_mb", st);
-    cudaError_t le = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kMbThreads), args, smem, st);
+    cudaError_t le = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kTvThreads), args, 0, st);
     prof_end("k_trsv_mb", st);
     NL_CUDA_OK(le);
     return NL_OK;
@@ -882,8 +958,8 @@ static bool trsv_cluster_ok(int C)
     const int slot = C == 16 ? 2 : (C == 8 ? 1 : 0);
     if (avail[slot] < 0) {
         bool ok = true;
-        for (int low = 0; low < 2 && ok; ++low) {
-            const void* kern = low ? (const void*)k_trsv_cl<true> : (const void*)k_trsv_cl<false>;
+        do {
+            const void* kern = (const void*)k_trsv_cl;
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kClMaxSmem) != cudaSuccess) {
                 ok = false;
@@ -902,7 +978,7 @@ static bool trsv_cluster_ok(int C)
             cfg.numAttrs = 1;
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) ok = false;
-        }
+        } while (false);
         cudaGetLastError();
         avail[slot] = ok ? 1 : 0;
     }
@@ -912,10 +988,11 @@ static bool trsv_cluster_ok(int C)
 // Cluster size for nblk blocks under the request req (0 = largest available,
 // -1 = none, else the largest available <= req); 0 = use the mailbox solve.
 // Automatic choice: the cluster's 16 SMs stream the whole factor, so beyond
-// 80 blocks (N > 10240) the mailbox solve over all SMs is faster (measured on
-// GB300: 197 vs 247 us at N = 8192, 379 vs 368 us at 12288, 676 vs 489 us at
-// 16384 per triangle).
-constexpr int kClAutoMaxBlocks = 80;
+// 24 blocks (N > 3072) the mailbox solve over all SMs is faster (measured on
+// GB300 per solve pair: 49 vs 54 us at N = 2048, 102 vs 96 us at 4096, 297 vs
+// 192 us at 8192; mailbox alone 282 us at 12000, 377 us at 16384, where a row
+// half per thread with its inverse in shared memory took 600 and 980).
+constexpr int kClAutoMaxBlocks = 24;
 static int trsv_cluster_size(int nblk, int req)
 {
     if (req < 0 || (req == 0 && nblk > kClAutoMaxBlocks)) return 0;
@@ -928,7 +1005,6 @@ static int trsv_cluster_size(int nblk, int req)
     return 0;
 }
 
-template <bool LOWER>
 static nl_status launch_trsv_cl(int N, const __half* LU, int64_t ld, const float* v, float* out, const TrsvWork& w,
                                 int C, cudaStream_t st)
 {
@@ -951,7 +1027,7 @@ static nl_status launch_trsv_cl(int N, const __half* LU, int64_t ld, const float
     const float* dinv = (const float*)w.dinv;
     prof_begin("k_trsv_cl", st);
     const long long wait = w.wait_limit == 0 ? kClWaitIters : (w.wait_limit < 0 ? 0LL : (long long)w.wait_limit);
-    cudaError_t le = cudaLaunchKernelEx(&cfg, k_trsv_cl<LOWER>, N, nblk, LU, ld, v, perm, dinv, out, w.err, wait, w.rs);
+    cudaError_t le = cudaLaunchKernelEx(&cfg, k_trsv_cl, N, nblk, LU, ld, v, perm, dinv, out, w.err, wait, w.rs);
     prof_end("k_trsv_cl", st);
     NL_CUDA_OK(le);
     return NL_OK;
@@ -962,11 +1038,8 @@ nl_status trsv_solve16(int N, const __half* LU, int64_t ld, const float* v, floa
 {
     const int C = trsv_cluster_size((int)cdiv(N, T2), w.cluster);
     if (C > 0) {
-        float* y = (float*)w.y;
-        nl_status s = launch_trsv_cl<true>(N, LU, ld, v, y, w, C, st);
-        if (s == NL_OK) s = launch_trsv_cl<false>(N, LU, ld, y, z, w, C, st);
-        if (launches) *launches += 2;
-        return s;
+        if (launches) *launches += 1;
+        return launch_trsv_cl(N, LU, ld, v, z, w, C, st);
     }
     unsigned long long* mbf = (unsigned long long*)w.y;
     unsigned long long* mbb = mbf + N;
