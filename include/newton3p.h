@@ -147,9 +147,10 @@ typedef struct {
     int lu_lookahead;    /* [0 = on] half-precision fast path with the tensor-core update (lu_nb <= 128):
                             after each panel only the trailing matrix's first 128-row and 128-column
                             tile strips (which hold the next panel) are updated on the solve's
-                            stream, and the rest of the update runs on a second stream of the same
-                            priority while the next panel is factored; the two are joined before
-                            the next update.  -1 = one update per panel.  Bitwise the same factors */
+                            stream (with lu_nb = 128 by the next panel's own launch), and the rest of
+                            the update runs on a second stream one priority step lower while the
+                            next panel is factored; the two are joined before the next update.
+                            -1 = one update per panel.  Bitwise the same factors */
 } nl_config;
 
 #define NL_MAX_HIST 128
@@ -565,7 +566,7 @@ nl_status nl_k_jacobian64(int64_t N, double c, const double* r, double* J64, int
  * gemm are ignored, and *info_host is also set (to -1) after a binary16
  * overflow, returned as NL_ENUMERIC; 4 = as 0 with look-ahead
  * (nl_config.lu_lookahead; same result; the call creates and destroys a
- * second stream).
+ * second stream; path 0 does so too from N = 1024 with the tcgen05 update).
  * With the tcgen05 update the entries of a row in columns N ..
  * round_up(N, 8) - 1 (inside ld) may be overwritten (the tensor-memory copies
  * store whole 16-byte units at the matrix's right edge).

@@ -715,6 +715,12 @@ nl_status tc_gemm16_update(int M, int Nc, int K, const __half* A, int64_t lda, c
     return NL_OK;
 }
 
+bool tc_encode_operand(const __half* p, int rows, int64_t ld, TmapBytes* out)
+{
+    static_assert(sizeof(TmapBytes) == sizeof(CUtensorMap), "tensor-map size");
+    return encode_2d(reinterpret_cast<CUtensorMap*>(out), p, 128, (uint64_t)rows, (uint64_t)ld, kTcBK, kTcBM);
+}
+
 bool tc_encode_instance_maps(const __half* A, int N, int64_t ld, const __half* ut, int nb, TmapBytes* out2)
 {
     static_assert(sizeof(TmapBytes) == sizeof(CUtensorMap), "tensor-map size");

@@ -192,6 +192,8 @@ nl_status launch_gemv_residual_g(const BInst* inst, BState* st, const BTask* tas
 // cross: only the first 128-column tile column and the first 128-row tile row of C.
 // max_ctas > 0 caps the grid of a small shallow update (K < 256, at most 8 tiles per SM).
 bool tc_gemm_supported();
+// Tensor map of an update operand (rows x 128 binary16, K-major): 64 x 128 boxes, 128-byte swizzle, zero fill.
+bool tc_encode_operand(const __half* p, int rows, int64_t ld, TmapBytes* out);
 // C <- C - A B on the tensor cores for binary32 C and binary32 operands holding
 // binary16 values (the two-level LU's inner updates), K <= 128, any M, Nc.
 nl_status tc_update_f32(int M, int Nc, int K, const float* A, int64_t lda, const float* B, int64_t ldb, float* C,

@@ -850,6 +850,10 @@ struct Diag16 {
     static constexpr size_t smem = (size_t)WMAX * LD * 4 + (size_t)WMAX * HLD * 2;
 };
 constexpr size_t kDiag16Smem = Diag16<128>::smem;
+// k_panel16x: the operand slabs of the update's tile, behind what the CTA holds otherwise
+constexpr size_t kCrossOpsOff = 103 * 1024;
+constexpr size_t kCrossSmem = kCrossOpsOff + 1024 + 4 * 16384;
+static_assert(kDiag16Smem <= kCrossOpsOff, "the block lies before the operands");
 
 // fl32(a b + c), a and b binary16 (bits)
 __device__ __forceinline__ float fma_h(unsigned short a, unsigned short b, float c)
@@ -898,6 +902,125 @@ __device__ __forceinline__ void store8(float* p, const float* v)
     reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
+// The look-ahead's part of a trailing update inside the next panel's own CTAs
+// (k_panel16x): a CTA's tile C - L21 U12, rounded to binary16, where the tile has
+// already been loaded into shared memory as binary32 (X[r * 132 + c] by rows, or
+// X[c * 132 + r] for a column CTA): the same tcgen05 products in the same order as
+// the update kernel's tile, so bitwise the same entries, which need not go
+// through memory before they are factored.  Two 64-wide slabs of each operand by
+// TMA into ops (64 KB, 1024-byte aligned), eight MMAs of K = 16 into 128 TMEM
+// columns, then every thread takes 32 columns of one row.  cross_begin starts the
+// loads (before the CTA loads its tile), cross_end applies the product.  It takes
+// about 2 us of a panel; as a launch of its own between the panels it took 6 us
+// and a second launch gap of 3.
+struct CrossTile {
+    const CUtensorMap *a, *b;  // L21 from the panel's first row on; U12^T from its first column on
+    int arow, brow;            // this CTA's tile
+};
+constexpr long long kCrossWait = 2000000000LL;  // cycles: about a second
+__device__ __forceinline__ void cross_begin(const CrossTile& T, uint32_t ops, uint64_t* bar, uint32_t* tslot)
+{
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(128u));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (threadIdx.x == 32) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[0])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[1])));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        const uint32_t bl = smem_u32(&bar[0]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bl), "r"(4u * 16384u) : "memory");
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            tma_load_2d(ops + q * 16384u, T.a, 64 * q, T.arow, bl);
+            tma_load_2d(ops + 32768u + q * 16384u, T.b, 64 * q, T.brow, bl);
+        }
+    }
+}
+
+// COLS: X holds columns (rows of 128 t each), else rows; n: lines held.  False after a timeout.
+template <bool COLS>
+__device__ __forceinline__ bool cross_end(uint32_t ops, uint64_t* bar, const uint32_t* tslot, float* X, int n, unsigned* err)
+{
+    __shared__ int dead;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) dead = 0;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();  // the tile is in X, the TMEM address and the barriers are set
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *(volatile const uint32_t*)tslot, bl = smem_u32(&bar[0]), bm = smem_u32(&bar[1]);
+    if (threadIdx.x == 32) {
+        if (!mbar_wait(bl, 0, kCrossWait)) {
+            atomicOr(err, (unsigned)ERR_TIMEOUT_OTHER);
+            *(volatile int*)&dead = 1;
+            mbar_wait(bl, 0, kCrossWait);  // let copies in flight land
+        } else {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            constexpr uint32_t idesc = tc_idesc_mn(128, 128);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t off = (uint32_t)(k >> 2) * 16384u + (uint32_t)(k & 3) * 32u;
+                const uint64_t ad = sw128_desc(ops + off), bd = sw128_desc(ops + 32768u + off);
+                const uint32_t acc = k ? 1u : 0u;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bm) : "memory");
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    bool good = !*(volatile int*)&dead;  // CTA-uniform
+    const bool waited = good ? mbar_wait(bm, 0, kCrossWait) : true;
+    if (__syncthreads_or(!waited)) {
+        if (threadIdx.x == 0) {
+            atomicOr(err, (unsigned)ERR_TIMEOUT_OTHER);
+            mbar_wait(bm, 0, kCrossWait);  // let the MMAs in flight finish
+        }
+        good = false;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int q = warp & 3, c0 = (warp >> 2) * 32, row = q * 32 + lane;  // TMEM lane, first column
+    if (good && (COLS ? c0 < n : q * 32 < n)) {  // (n: a multiple of 32)
+        uint32_t r[32];
+        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+              "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
+              "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+              "=r"(r[30]), "=r"(r[31])
+            : "r"(taddr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (COLS) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                float* x = X + (c0 + e) * 132 + row;
+                *x = round_h(*x - __uint_as_float(r[e]));
+            }
+        } else {
+            float4* x = reinterpret_cast<float4*>(X + row * 132 + c0);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 v = x[e];
+                x[e] = make_float4(round_h(v.x - __uint_as_float(r[4 * e])), round_h(v.y - __uint_as_float(r[4 * e + 1])),
+                                   round_h(v.z - __uint_as_float(r[4 * e + 2])), round_h(v.w - __uint_as_float(r[4 * e + 3])));
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128u));
+    }
+    return good;
+}
+
 // The published copy of a factored diagonal block (k_panel16): 64-bit words
 // {epoch, two binary16 values}; a word is its own ready flag.
 //   word k * 64 + e / 2, e > k even:           u_ke, u_k(e+1)
@@ -932,11 +1055,13 @@ __device__ __forceinline__ void diag16_publish(int s, int w8, const unsigned sho
 
 // PUB: also publish the block as it is factored, for the streaming solves of
 // k_panel16.  stage (may be null): U11, L11^T and the pivots for k_offdiag16.
-template <bool PUB = false, typename S_ = __half, int WMAX = 128, int NT = kD16Threads>
+// CROSS: the block first takes its part of the last update (ct).
+template <bool PUB = false, typename S_ = __half, int WMAX = 128, int NT = kD16Threads, bool CROSS = false>
 __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, int K, int w,
                                                int* __restrict__ ipiv, int* __restrict__ flag,
                                                float* __restrict__ stage,
-                                               unsigned long long* __restrict__ pub = nullptr, unsigned epoch = 0)
+                                               unsigned long long* __restrict__ pub = nullptr, unsigned epoch = 0,
+                                               const CrossTile* ct = nullptr, unsigned* err = nullptr)
 {
     if (*(volatile int*)flag) return;
     using G = Diag16<WMAX>;
@@ -950,6 +1075,10 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int w8 = (w + 7) & ~7, nq = w8 >> 3;
     const bool vec = (w % 8 == 0) && ((((uintptr_t)(A + (int64_t)K * lda + K)) & 15) == 0) && (lda % 8 == 0);
+    __shared__ __align__(8) uint64_t xbar[2];
+    __shared__ uint32_t xslot;
+    const uint32_t ops = (smem_u32(lsh) + (uint32_t)kCrossOpsOff + 1023u) & ~1023u;
+    if constexpr (CROSS) cross_begin(*ct, ops, xbar, &xslot);
     // load, eight columns per thread, padded with the identity to w8
     for (int p = tid; p < w8 * nq; p += NT) {
         const int i = p / nq, C = 8 * (p - i * nq);
@@ -966,8 +1095,9 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
         }
         store8(S + i * LD + C, v);
     }
-    __syncthreads();
     bool bad = false;
+    if constexpr (CROSS) bad = !cross_end<false>(ops, xbar, &xslot, S, 128, err);
+    __syncthreads();
     const int r = lane & 7;
     const int pubv = wid - 8;  // warps 8..15 publish
     const bool pubw = wid >= 8;
@@ -1236,6 +1366,8 @@ constexpr int kPnlXld = 132;    // floats
 constexpr int kPnlMld = 136;    // binary16
 constexpr size_t kPnlSmem = (size_t)kPnlRows * kPnlXld * 4 + (size_t)128 * kPnlMld * 2 + 128 * 4 + 16 * 8;
 static_assert(kPnlSmem >= kDiag16Smem, "the diagonal block's CTA uses the same launch");
+static_assert((size_t)128 * kPnlXld * 4 + (size_t)128 * kPnlMld * 2 + 128 * 4 + 16 * 8 <= kCrossOpsOff,
+              "a streaming CTA of 128 lines lies before the operands");
 constexpr long long kPnlSpin = 1LL << 22;
 
 // Fetch lane: up to five pairs of published words (16 bytes each; bit v of todo:
@@ -1289,15 +1421,15 @@ __device__ __forceinline__ void pnl_apply(const uint4& hist, const unsigned shor
 }
 
 // One streaming CTA: ROWS = rows of L21, else columns of U12; rpc lines (a multiple of 32).
-template <bool ROWS, typename S = __half>
+template <bool ROWS, typename S = __half, bool CROSS = false>
 __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, int K, int w, int N, int blk,
                                                int rpc, __half* __restrict__ Ut, int ldut, int ut_col0, int ut_k0,
                                                int* __restrict__ flag, const unsigned long long* __restrict__ pub,
-                                               unsigned epoch, unsigned* __restrict__ err)
+                                               unsigned epoch, unsigned* __restrict__ err, const CrossTile* ct = nullptr)
 {
     extern __shared__ __align__(16) float psm[];
     float* X = psm;                                                                   // X[line * kPnlXld + t]
-    unsigned short* M = reinterpret_cast<unsigned short*>(X + kPnlRows * kPnlXld);    // M[k * kPnlMld + e]
+    unsigned short* M = reinterpret_cast<unsigned short*>(X + (CROSS ? 128 : kPnlRows) * kPnlXld);  // M[k * kPnlMld + e]
     float* pv = reinterpret_cast<float*>(M + 128 * kPnlMld);                          // unrounded pivots (rows)
     uint64_t* ready = reinterpret_cast<uint64_t*>(pv + 128);
     __shared__ int gave_up;
@@ -1308,6 +1440,10 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
     if (tid < 16) asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"((unsigned)__cvta_generic_to_shared(&ready[tid])));
     const bool vec = (w % 8 == 0) && (lda % 8 == 0) && ((((uintptr_t)(A + K)) & 15) == 0);
     const bool cvec = (lda % 8 == 0) && ((((uintptr_t)(A + line0)) & 15) == 0);  // eight columns at a time
+    __shared__ __align__(8) uint64_t xbar[2];
+    __shared__ uint32_t xslot;
+    const uint32_t ops = (smem_u32(psm) + (uint32_t)kCrossOpsOff + 1023u) & ~1023u;
+    if constexpr (CROSS) cross_begin(*ct, ops, xbar, &xslot);
     if (ROWS) {
         for (int p = tid; p < rpc * nq; p += kPnlThreads) {
             const int r = p / nq, C = 8 * (p - r * nq);
@@ -1342,8 +1478,9 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
             X[c * kPnlXld + t] = (t < w) ? ld_elem(A + (int64_t)(K + t) * lda + line0 + min(c, nlive - 1)) : 0.0f;
         }
     }
+    bool bad = false, dead = false;
+    if constexpr (CROSS) dead = !cross_end<!ROWS>(ops, xbar, &xslot, X, rpc, err);
     __syncthreads();
-    bool bad = false;
     if (warp >= kPnlFetchW) {
         bool ok = true;
         for (int q = 0; q < nq; ++q) {
@@ -1411,7 +1548,7 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
         }
         if (tid >= nlive) bad = false;
     }
-    if (__syncthreads_or(bad) && tid == 0) atomicOr(flag, 1);
+    if (__syncthreads_or(bad || dead) && tid == 0) atomicOr(flag, 1);
     if (gave_up) {
         if (tid == 0) {
             // a timeout (not an abandoned fast path) is an error; either way the
@@ -1525,6 +1662,39 @@ __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16(S* __restrict__ A, i
         panel16_stream<true, S>(A, lda, K, w, N, r - 1, rpc, Ut, ldut, ut_col0, ut_k0, flag, pub, epoch, err);
     else
         panel16_stream<false, S>(A, lda, K, w, N, r - 1 - nrb, rpc, Ut, ldut, ut_col0, ut_k0, flag, pub, epoch, err);
+}
+
+// k_panel16 for a panel of 128 columns after a panel of 128 whose update has not
+// touched the panel's rows and columns yet: every CTA first applies it to its own
+// tile (cross_begin / cross_end).  mA: L21 of the last panel from row K on, mB: its
+// U12^T from column K on.  rpc: 64 or 128.
+__global__ void __launch_bounds__(kPnlThreads, 1) k_panel16x(const __grid_constant__ CUtensorMap mA,
+                                                            const __grid_constant__ CUtensorMap mB,
+                                                            __half* __restrict__ A, int64_t lda, int K, int w, int N,
+                                                            int nrb, int rpc, int* __restrict__ ipiv, int* __restrict__ flag,
+                                                            __half* __restrict__ Ut, int ldut,
+                                                            unsigned long long* __restrict__ pub, unsigned epoch,
+                                                            unsigned* __restrict__ err, int* __restrict__ tickets, int slot)
+{
+    __shared__ int role;
+    if (threadIdx.x == 0) {
+        const int t = atomicAdd(&tickets[slot], 1);
+        if (t == 0) tickets[slot ^ 1] = 0;
+        if (t == (int)gridDim.x - 1) tickets[slot] = 0;
+        role = t;
+    }
+    __syncthreads();
+    const int r = role;
+    if (r == 0) {
+        const CrossTile ct{&mA, &mB, 0, 0};
+        diag_lu16_body<true, __half, 128, kD16Threads, true>(A, lda, K, w, ipiv, flag, nullptr, pub, epoch, &ct, err);
+    } else if (r <= nrb) {
+        const CrossTile ct{&mA, &mB, w + (r - 1) * rpc, 0};
+        panel16_stream<true, __half, true>(A, lda, K, w, N, r - 1, rpc, Ut, ldut, K + w, 0, flag, pub, epoch, err, &ct);
+    } else {
+        const CrossTile ct{&mA, &mB, 0, w + (r - 1 - nrb) * rpc};
+        panel16_stream<false, __half, true>(A, lda, K, w, N, r - 1 - nrb, rpc, Ut, ldut, K + w, 0, flag, pub, epoch, err, &ct);
+    }
 }
 
 // k_offdiag16: L21 = A21 U11^{-1} (row role) and U12 = L11^{-1} A12 (column
@@ -1996,7 +2166,8 @@ static nl_status panel16_setup()
     static std::atomic<bool> done{false};
     if (done.load(std::memory_order_acquire)) return NL_OK;
     if (set_max_dynamic_smem((const void*)k_panel16<__half>) != NL_OK ||
-        set_max_dynamic_smem((const void*)k_panel16<float>) != NL_OK)
+        set_max_dynamic_smem((const void*)k_panel16<float>) != NL_OK ||
+        set_max_dynamic_smem((const void*)k_panel16x) != NL_OK)
         return NL_ECUDA;
     done.store(true, std::memory_order_release);
     return NL_OK;
@@ -2015,8 +2186,10 @@ static std::atomic<unsigned> g_panel_epoch{0};
 
 template <typename S>
 static nl_status launch_panel16(S* A, int64_t ld, int K, int wd, int N, int* ipiv, const LuWork& w, __half* Ut,
-                                int ldut, cudaStream_t st, int slot, int ut_col0 = -1, int ut_k0 = 0)
+                                int ldut, cudaStream_t st, int slot, int ut_col0 = -1, int ut_k0 = 0,
+                                const __half* ut_prev = nullptr)
 {
+    // ut_prev: U12^T of the last panel (128 columns), whose update of this panel's tiles is still to be done
     if (ut_col0 < 0) ut_col0 = K + wd;
     const int rest = N - K - wd;
     int rpc = panel16_rows_per_cta(rest, w.stream);
@@ -2029,6 +2202,23 @@ static nl_status launch_panel16(S* A, int64_t ld, int K, int wd, int N, int* ipi
     unsigned* err = tc_error_word();
     if (!err) err = (unsigned*)(w.info + 2);  // (a word of the info block nobody else uses)
     int* tickets = w.info + 8;  // two counters (+8, +9) of the info block; slot: the panel's index mod 2
+    if constexpr (std::is_same<S, __half>::value) {
+        if (ut_prev) {
+            TmapBytes mA, mB;
+            if (!tc_encode_operand(A + (int64_t)K * ld + K - 128, N - K, ld, &mA) ||
+                !tc_encode_operand(ut_prev, N - K, ldut, &mB)) {
+                set_error("panel: cuTensorMapEncodeTiled failed");
+                return NL_ECUDA;
+            }
+            prof_begin("k_panel16", st);
+            k_panel16x<<<1 + 2 * nrb, kPnlThreads, kCrossSmem, st>>>(
+                reinterpret_cast<const CUtensorMap&>(mA), reinterpret_cast<const CUtensorMap&>(mB), A, ld, K, wd, N, nrb, rpc,
+                ipiv, flag, Ut, ldut, pub, epoch, err, tickets, slot);
+            prof_end("k_panel16", st);
+            NL_CUDA_OK(cudaGetLastError());
+            return NL_OK;
+        }
+    }
     prof_begin("k_panel16", st);
     k_panel16<S><<<1 + 2 * nrb, kPnlThreads, kPnlSmem, st>>>(A, ld, K, wd, N, nrb, rpc, ipiv, flag, Ut, ldut,
                                                             ut_col0, ut_k0, pub, epoch, err, tickets, slot);
@@ -2093,6 +2283,10 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
         return NL_ECUDA;
     };
     auto ut_of = [&](int K) { return (la && ((K / nb) & 1)) ? w.ut2 : w.ut; };
+    // With panels of 128 the next panel's own CTAs take the cross (k_panel16x), while it has
+    // rows below it and its CTAs hold at most 128 lines; cross_ut: U12^T of the panel whose cross is left to the next.
+    const __half* cross_ut = nullptr;
+    const bool merge = la && nb == kLaTile && w.stream == 0;
     // the update after the panel at K (width wd)
     auto update = [&](int K, int wd, bool tc, const __half* utp) -> nl_status {
         const int rest = N - K - wd, q = K / nb;
@@ -2106,7 +2300,10 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
             const bool side_now = rest > kLaTile;
             if (side_now) NL_CUDA_OK(cudaEventRecord(w.ev_fork, st));
             NL_TRY(join_ok(join.wait(q - 1)));  // the rest of update q - 1 wrote the cross's tiles
-            NL_TRY(tc_gemm16_update(rest, rest, wd, L21, ld, utp, nb, A22, ld, st, w.flag, false, true));
+            if (merge && wd == kLaTile && side_now) {
+                cross_ut = utp;
+                --nl;
+            } else NL_TRY(tc_gemm16_update(rest, rest, wd, L21, ld, utp, nb, A22, ld, st, w.flag, false, true));
             if (side_now) {
                 const int m2 = rest - kLaTile;
                 NL_TRY(join_ok(join.wait(q - 2)));  // ev_join[q % 2] is free again
@@ -2136,13 +2333,16 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
                         pub_cleared = true;
                     }
                     __half* utp = tc ? ut_of(K) : nullptr;
-                    NL_TRY(launch_panel16(A, ld, K, wd, N, ipiv, w, utp, nb, st, (K / nb) & 1));
+                    const __half* cu = cross_ut;
+                    cross_ut = nullptr;
+                    NL_TRY(launch_panel16(A, ld, K, wd, N, ipiv, w, utp, nb, st, (K / nb) & 1, -1, 0, cu));
                     NL_TRY(update(K, wd, tc, utp));
                     nl += 2;
                     continue;
                 }
                 prof_begin("k_diag_lu16", st);
-                k_diag_lu16<__half><<<1, kD16Threads, kDiag16Smem, st>>>(A, ld, K, wd, ipiv, w.flag, (float*)w.stage);
+                k_diag_lu16<__half><<<1, kD16Threads, kDiag16Smem, st>>>(A, ld, K, wd, ipiv, w.flag,
+                                                                      rest > 0 ? (float*)w.stage : nullptr);
                 prof_end("k_diag_lu16", st);
             } else {
                 prof_begin("k_diag_lu", st);
@@ -2301,7 +2501,8 @@ static nl_status lu16_factor_2lvl(int N, __half* A, int64_t ld, int* ipiv, int W
                 ++nl;
             } else {
                 prof_begin("k_diag_lu16", st);
-                k_diag_lu16<float><<<1, kD16Threads, kDiag16Smem, st>>>(P, ldp, K, wd, ipiv, w.flag, (float*)w.stage);
+                k_diag_lu16<float><<<1, kD16Threads, kDiag16Smem, st>>>(P, ldp, K, wd, ipiv, w.flag,
+                                                                     rest > 0 ? (float*)w.stage : nullptr);
                 prof_end("k_diag_lu16", st);
                 ++nl;
                 if (rest > 0) {
