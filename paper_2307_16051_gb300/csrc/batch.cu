@@ -1570,7 +1570,7 @@ nl_status nl_lusolve_grouped(int count, const int64_t* N, const void* const* LU,
     NL_TRY(batch_trsv_smem_setup());
     cudaStream_t st = (cudaStream_t)stream;
     GSolve* d = nullptr;
-    NL_CUDA_OK(cudaMallocAsync((void**)&d, sizeof(GSolve) * count, st));
+    NL_CUDA_OK(ws_malloc_async((void**)&d, sizeof(GSolve) * count, st));
     NL_CUDA_OK(cudaMemcpyAsync(d, items.data(), sizeof(GSolve) * count, cudaMemcpyHostToDevice, st));
     const size_t smem = (size_t)round_up(nmax, 32) * (fp64 ? 8 : 4);
     if (fp64) k_trsv_grouped<double, double><<<count, kBtThreads, smem, st>>>(d);

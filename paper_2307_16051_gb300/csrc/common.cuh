@@ -40,6 +40,15 @@ int num_sms();
 // hook nl_debug_fail_allocs has allocations left to fail.
 cudaError_t dev_malloc(void** p, size_t bytes);
 
+// Stream-ordered workspace of a kernel-level entry point, released with
+// cudaFreeAsync: from the library's own memory pool on the current device,
+// which keeps up to kWsKeep bytes of released memory across synchronisations
+// (the default pool returns all of it to the system at each one and maps it
+// again at the next call: 190 us of a call that synchronises).  dev_malloc gives
+// the kept memory back before it reports that the device is full.
+constexpr size_t kWsKeep = (size_t)256 << 20;
+cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st);
+
 // Carves 256-byte aligned sub-buffers out of one device allocation (a null
 // base only measures: off is the size needed).
 struct Carver {

@@ -31,6 +31,39 @@ static thread_local char g_err[512] = "";
 // of the library's handles fail as if the device were out of memory.
 static std::atomic<int> g_fail_allocs{0};
 
+// The current device's workspace pool (created on first use; null where pools are not supported).
+constexpr int kWsMaxDevices = 64;
+static std::mutex g_ws_mu;
+static cudaMemPool_t g_ws_pool[kWsMaxDevices] = {};
+static cudaMemPool_t ws_pool(bool create)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kWsMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(g_ws_mu);
+    if (!g_ws_pool[dev] && create) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kWsKeep;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            if (pool) cudaMemPoolDestroy(pool);
+            return nullptr;
+        }
+        g_ws_pool[dev] = pool;
+    }
+    return g_ws_pool[dev];
+}
+static bool ws_trim()
+{
+    cudaMemPool_t pool = ws_pool(false);
+    return pool && cudaMemPoolTrimTo(pool, 0) == cudaSuccess;
+}
+
 cudaError_t dev_malloc(void** p, size_t bytes)
 {
     int n = g_fail_allocs.load();
@@ -40,7 +73,19 @@ cudaError_t dev_malloc(void** p, size_t bytes)
             return cudaErrorMemoryAllocation;
         }
     }
-    return cudaMalloc(p, bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ws_trim()) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
+cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st)
+{
+    cudaMemPool_t pool = ws_pool(true);
+    if (!pool) return cudaMallocAsync(p, bytes, st);
+    return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
 void set_error(const char* fmt, ...)
@@ -1083,7 +1128,7 @@ nl_status nl_k_residual(int64_t N, double c, const double* x, const void* u, int
     double *htab = nullptr, *partial = nullptr;
     unsigned* counter = nullptr;
     const size_t np = residual_partials(n);
-    NL_CUDA_OK(cudaMallocAsync((void**)&htab, sizeof(double) * (2 * n + np) + 256, st));
+    NL_CUDA_OK(ws_malloc_async((void**)&htab, sizeof(double) * (2 * n + np) + 256, st));
     partial = htab + 2 * n;
     counter = (unsigned*)(partial + np);
     NL_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(unsigned), st));
@@ -1104,7 +1149,7 @@ nl_status nl_k_residual_fft(int64_t N, double c, const double* x, const void* u,
     cudaStream_t st = (cudaStream_t)stream;
     const int n = (int)N;
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMallocAsync(&wk, fft_work_bytes(n), st));
+    NL_CUDA_OK(ws_malloc_async(&wk, fft_work_bytes(n), st));
     FftPlan p;
     fft_work_carve(wk, n, &p);
     nl_status s = fft_prepare(p, st);
@@ -1123,7 +1168,7 @@ static nl_status jacobian_entry(int64_t N, double c, const double* r, float* J32
     cudaStream_t st = (cudaStream_t)stream;
     const int n = (int)N;
     double* htab = nullptr;
-    NL_CUDA_OK(cudaMallocAsync((void**)&htab, sizeof(double) * 2 * n, st));
+    NL_CUDA_OK(ws_malloc_async((void**)&htab, sizeof(double) * 2 * n, st));
     nl_status s = launch_htab(n, htab, st);
     if (s == NL_OK) s = launch_jacobian(n, c, r, htab, J32, ld32, (__half*)J16, ld16, st, rs);
     cudaFreeAsync(htab, st);
@@ -1155,7 +1200,7 @@ nl_status nl_k_jacobian64(int64_t N, double c, const double* r, double* J64, int
     cudaStream_t st = (cudaStream_t)stream;
     const int n = (int)N;
     double* htab = nullptr;
-    NL_CUDA_OK(cudaMallocAsync((void**)&htab, sizeof(double) * 2 * n, st));
+    NL_CUDA_OK(ws_malloc_async((void**)&htab, sizeof(double) * 2 * n, st));
     nl_status s = launch_htab(n, htab, st);
     if (s == NL_OK) s = launch_jacobian64(n, c, r, htab, J64, ld, st);
     cudaFreeAsync(htab, st);
@@ -1177,7 +1222,7 @@ static nl_status lu_entry(int64_t N, S* A, int64_t ld, int32_t* ipiv, int nb, in
     const size_t lw = lu_work_bytes(n, nb, fp64);
     const size_t copy = (path == 1) ? 0 : (size_t)n * ld * sizeof(S);
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMallocAsync(&wk, lw + copy + 256, st));
+    NL_CUDA_OK(ws_malloc_async(&wk, lw + copy + 256, st));
     LuWork w;
     lu_work_carve(wk, n, nb, fp64, &w);
     if (path == 2) {  // the fast path with two launches per panel (no streaming panel)
@@ -1241,7 +1286,7 @@ static nl_status lu_entry(int64_t N, S* A, int64_t ld, int32_t* ipiv, int nb, in
 static nl_status lu16_arith_entry(int n, __half* A, int64_t ld, int32_t* ipiv, int32_t* info_host, cudaStream_t st)
 {
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMallocAsync(&wk, lu_work_bytes(n, 128, false) + 256, st));
+    NL_CUDA_OK(ws_malloc_async(&wk, lu_work_bytes(n, 128, false) + 256, st));
     LuWork w;
     lu_work_carve(wk, n, 128, false, &w);
     int iflag[2] = {0, 0};
@@ -1309,7 +1354,7 @@ nl_status nl_lu32(int64_t N, float* A, int64_t ld, int32_t* ipiv, int nb, int32_
     cudaStream_t st = (cudaStream_t)stream;
     const int n = (int)N;
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMallocAsync(&wk, lu_work_bytes(n, nb, false) + 256, st));
+    NL_CUDA_OK(ws_malloc_async(&wk, lu_work_bytes(n, nb, false) + 256, st));
     LuWork w;
     lu_work_carve(wk, n, nb, false, &w);
     int info = 0;
@@ -1336,7 +1381,7 @@ static nl_status lusolve_entry(int64_t N, const S* LU, int64_t ld, const int32_t
     const int n = (int)N;
     void* wk = nullptr;
     const size_t bytes = trsv_work_bytes(n, fp64);
-    NL_CUDA_OK(cudaMallocAsync(&wk, bytes, st));
+    NL_CUDA_OK(ws_malloc_async(&wk, bytes, st));
     NL_CUDA_OK(cudaMemsetAsync(wk, 0, bytes, st));
     TrsvWork w;
     trsv_work_carve(wk, n, fp64, &w);
@@ -1403,7 +1448,7 @@ nl_status nl_k_gemv_residual(int64_t N, const float* A, int64_t ld, const float*
     const int n = (int)N;
     const size_t np = gemv_partials(n);
     double* partial = nullptr;
-    NL_CUDA_OK(cudaMallocAsync((void**)&partial, sizeof(double) * np + 256, st));
+    NL_CUDA_OK(ws_malloc_async((void**)&partial, sizeof(double) * np + 256, st));
     unsigned* counter = (unsigned*)(partial + np);
     NL_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(unsigned), st));
     nl_status s = launch_gemv_residual(n, A, ld, b, u, r, partial, counter, rnorm_dev, st);
@@ -1421,6 +1466,47 @@ nl_status nl_k_gemm16_update(int64_t M, int64_t Nc, int64_t K, const void* A, in
     return gemm16_update((int)M, (int)Nc, (int)K, (const __half*)A, lda, (const __half*)B, ldb, (__half*)C, ldc, gemm,
                          (cudaStream_t)stream);
 }
+
+// 64 bytes of pinned host memory for a call's scalars, from a small free list
+// (allocating and freeing pinned memory synchronises and takes longer than a small solve).
+namespace {
+struct PinnedWords {
+    double* p = nullptr;
+    PinnedWords()
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu());
+            if (!list().empty()) {
+                p = list().back();
+                list().pop_back();
+            }
+        }
+        if (!p && cudaMallocHost((void**)&p, 64) != cudaSuccess) p = nullptr;
+    }
+    ~PinnedWords()
+    {
+        if (!p) return;
+        {
+            std::lock_guard<std::mutex> lock(mu());
+            if (list().size() < 16) {
+                list().push_back(p);
+                return;
+            }
+        }
+        cudaFreeHost(p);
+    }
+    static std::mutex& mu()
+    {
+        static std::mutex m;
+        return m;
+    }
+    static std::vector<double*>& list()
+    {
+        static std::vector<double*>* l = new std::vector<double*>();  // (never destroyed: calls may outlive statics)
+        return *l;
+    }
+};
+}  // namespace
 
 nl_status nl_linsolve16(int64_t N, const float* J32, int64_t ld32, const void* LU16, int64_t ld16, const int32_t* ipiv,
                         const float* b, float* u, double eta, int maxit, int solver, int m, double gtol, int gcycles,
@@ -1447,10 +1533,11 @@ nl_status nl_linsolve16(int64_t N, const float* J32, int64_t ld32, const void* L
         bytes = cv.off + 256;
     }
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMallocAsync(&wk, bytes, st));
+    NL_CUDA_OK(ws_malloc_async(&wk, bytes, st));
     NL_CUDA_OK(cudaMemsetAsync(wk, 0, bytes, st));
-    double* pin = nullptr;
-    if (cudaMallocHost((void**)&pin, 64) != cudaSuccess) {
+    PinnedWords words;
+    double* pin = words.p;
+    if (!pin) {
         cudaFreeAsync(wk, st);
         set_error("nl_linsolve16: pinned allocation failed");
         return NL_ENOMEM;
@@ -1482,7 +1569,6 @@ nl_status nl_linsolve16(int64_t N, const float* J32, int64_t ld32, const void* L
     cudaMemcpyAsync(&e, tw.err, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
     cudaFreeAsync(wk, st);
     cudaStreamSynchronize(st);
-    cudaFreeHost(pin);
     if ((s == NL_OK && e) || s == NL_ETIMEOUT) {
         set_error("triangular solve: a bounded wait gave up");
         return NL_ETIMEOUT;
