@@ -447,16 +447,16 @@ __global__ void __launch_bounds__(kTrsmThreads) k_trsm_u12(S* __restrict__ A, in
 __device__ __forceinline__ float absT(float x) { return fabsf(x); }
 __device__ __forceinline__ double absT(double x) { return fabs(x); }
 
-// Diagonal block [K, K+w)^2 (w <= 128) in one CTA, held in shared memory,
-// in 32-column chunks c (padding beyond w is identity):
-//  (a) one warp factors the 32 x 32 diagonal sub-block, lane r = row r: at
-//      step t row t is final, its U entries are rounded, and the rows below
-//      form their multipliers and update;
-//  (b) groups of eight lanes solve the rows below the sub-block against its
-//      U, and (c) the columns right of it against its L (as k_offdiag does);
-//  (d) all threads apply the rank-32 update to the rest of the block.
+// Diagonal block [K, K+w)^2 (w <= 128) in one CTA, held in shared memory
+// (double precision: the F64 baseline).  Right-looking with look-ahead, one
+// barrier per column: at step k the first wp / 32 warps (a row per thread) take
+// column k + 1 alone (update, pivot check, division), while the others apply
+// column k's multipliers to the columns right of it (lanes along a row).  The
+// bound is the double-precision pipe (two multiply-adds per SM and cycle: w^3 / 3
+// of them, 22 us at w = 64, and the divisions, about 13 us).  Measured, w = 64:
+// 64 us; a warp per 32 x 32 sub-block with the pivot row by shuffles and solves by
+// groups of eight lanes took 243.
 constexpr int kDiagThreads = 512;
-constexpr int kOffG = 8;  // lanes per row / column group
 
 // Block [K, K+w)^2 of A into shared memory W (ld ldw), identity-padded to
 // wp; 16-byte vector loads when the row segments allow them.
@@ -513,55 +513,6 @@ __device__ __forceinline__ void store_block(S* __restrict__ A, int64_t lda, int 
     }
 }
 
-template <typename T, bool RND>
-__device__ __forceinline__ void group_row_solve(T* W, int ldw, int c0, int r, int g, unsigned gmask, bool& bad)
-{
-    // row r, chunk columns c0 + 4g .. c0 + 4g + 3, against U = W[c0.., c0..]
-    T acc[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = W[r * ldw + c0 + 4 * g + k];
-#pragma unroll
-    for (int tt = 0; tt < 32; ++tt) {
-        T l = T(0);
-        if (g == tt / 4) {
-            const T utt = W[(c0 + tt) * ldw + c0 + tt];
-            const T x = acc[tt % 4];
-            if (!(absT(x) <= absT(utt)) || !(utt != T(0))) bad = true;
-            l = maybe_round(x / utt, RND);
-            acc[tt % 4] = l;
-        }
-        l = __shfl_sync(gmask, l, tt / 4, kOffG);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (4 * g + k > tt) acc[k] = fma(-l, W[(c0 + tt) * ldw + c0 + 4 * g + k], acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) W[r * ldw + c0 + 4 * g + k] = acc[k];
-}
-
-template <typename T, bool RND>
-__device__ __forceinline__ void group_col_solve(T* W, int ldw, int c0, int col, int g, unsigned gmask)
-{
-    // column col, chunk rows c0 + 4g .. c0 + 4g + 3, against L = W[c0.., c0..]
-    T acc[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = W[(c0 + 4 * g + k) * ldw + col];
-#pragma unroll
-    for (int tt = 0; tt < 32; ++tt) {
-        T u = T(0);
-        if (g == tt / 4) {
-            u = maybe_round(acc[tt % 4], RND);
-            acc[tt % 4] = u;
-        }
-        u = __shfl_sync(gmask, u, tt / 4, kOffG);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (4 * g + k > tt) acc[k] = fma(-W[(c0 + 4 * g + k) * ldw + c0 + tt], u, acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) W[(c0 + 4 * g + k) * ldw + col] = acc[k];
-}
-
 template <typename T, typename S, bool RND>
 __device__ __forceinline__ void diag_lu_body(S* __restrict__ A, int64_t lda, int K, int w,
                                                              int* __restrict__ ipiv, int* __restrict__ flag,
@@ -572,77 +523,42 @@ __device__ __forceinline__ void diag_lu_body(S* __restrict__ A, int64_t lda, int
     T* W = reinterpret_cast<T*>(smem_raw);
     const int wp = (w + 31) & ~31, ldw = wp + 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int grp = tid / kOffG, g = tid % kOffG;
-    const unsigned gmask = 0xffu << ((tid & 31) & ~(kOffG - 1));
+    const int wa = wp / 32;  // warps that take the next column
+    __shared__ T piv[2];     // the pivots, alternating
     load_block<T, S, kDiagThreads>(A, lda, K, w, wp, W, ldw, tid);
     __syncthreads();
     bool bad = false;
-    const int nc = wp / 32;
-    for (int c = 0; c < nc; ++c) {
-        const int c0 = 32 * c;
-        if (warp == 0) {
-            // lane r holds row c0 + r of the sub-block; after step t the row
-            // array is shifted by one so that a[0] is always column c0 + t
-            T* Wr = W + (c0 + lane) * ldw + c0;
-            T a[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) a[j] = Wr[j];
-            for (int t = 0; t < 32; ++t) {
-                const T utt = __shfl_sync(0xffffffffu, maybe_round(a[0], RND), t);
-                // rows below form their multiplier; finished rows use l = 0
-                T l = T(0);
-                if (lane > t) {
-                    if (!(absT(a[0]) <= absT(utt)) || !(utt != T(0))) bad = true;
-                    l = maybe_round(a[0] / utt, RND);
+    for (int k = -1; k < w - 1; ++k) {
+        const T* Wk = W + k * ldw;  // row k: U from the diagonal on (k = -1: nothing to apply)
+        if (warp < wa) {
+            const int i = tid, c = k + 1;
+            T x = T(0);
+            if (i > k) x = W[i * ldw + c];
+            if (k >= 0 && i > k) x = fma(-W[i * ldw + k], Wk[c], x);
+            if (i == c) {
+                x = maybe_round(x, RND);
+                piv[c & 1] = x;
+                W[c * ldw + c] = x;
+            }
+            __syncwarp();
+            asm volatile("bar.sync 1, %0;" ::"r"(32 * wa) : "memory");
+            const T u = piv[c & 1];
+            if (i > c) {  // (padding rows too: zero against a zero pivot is left to the interchanging path)
+                if (!(absT(x) <= absT(u)) || !(u != T(0))) bad = true;
+                W[i * ldw + c] = maybe_round(x / u, RND);
+            }
+        } else if (k >= 0) {
+            const int nv = kDiagThreads / 32 - wa;
+            for (int j = k + 2 + lane; j < w; j += 32) {
+                const T u = Wk[j];
+                for (int i = k + 1 + warp - wa; i < w; i += nv) {
+                    T x = fma(-W[i * ldw + k], u, W[i * ldw + j]);
+                    if (RND && i == k + 1) x = maybe_round(x, RND);  // row k + 1 is final
+                    W[i * ldw + j] = x;
                 }
-                a[0] = (lane == t) ? utt : ((lane > t) ? l : a[0]);
-                if (lane >= t) Wr[t] = a[0];
-#pragma unroll
-                for (int j = 1; j < 32; ++j) {
-                    const T uj = __shfl_sync(0xffffffffu, maybe_round(a[j], RND), t);
-                    a[j] = (lane == t) ? uj : fma(-l, uj, a[j]);
-                }
-                if (lane == t) {
-#pragma unroll
-                    for (int j = 1; j < 32; ++j)
-                        if (t + j < 32) Wr[t + j] = a[j];  // U entries of row t
-                }
-#pragma unroll
-                for (int j = 0; j < 31; ++j) a[j] = a[j + 1];
-                a[31] = T(0);
             }
         }
         __syncthreads();
-        const int rest = wp - c0 - 32;
-        // (b) rows below and (c) columns right of the sub-block: one group each
-        for (int q = grp; q < 2 * rest; q += kDiagThreads / kOffG) {
-            if (q < rest) group_row_solve<T, RND>(W, ldw, c0, c0 + 32 + q, g, gmask, bad);
-            else group_col_solve<T, RND>(W, ldw, c0, c0 + 32 + (q - rest), g, gmask);
-        }
-        __syncthreads();
-        if (rest > 0) {
-            // (d) rows/cols [c0+32, wp): 2 x 2 entries per thread, t in order
-            const int nb2 = rest / 2;
-            for (int e = tid; e < nb2 * nb2; e += kDiagThreads) {
-                const int i = c0 + 32 + 2 * (e / nb2), j = c0 + 32 + 2 * (e % nb2);
-                T a00 = W[i * ldw + j], a01 = W[i * ldw + j + 1];
-                T a10 = W[(i + 1) * ldw + j], a11 = W[(i + 1) * ldw + j + 1];
-#pragma unroll 8
-                for (int t = c0; t < c0 + 32; ++t) {
-                    const T l0 = W[i * ldw + t], l1 = W[(i + 1) * ldw + t];
-                    const T u0 = W[t * ldw + j], u1 = W[t * ldw + j + 1];
-                    a00 = fma(-l0, u0, a00);
-                    a01 = fma(-l0, u1, a01);
-                    a10 = fma(-l1, u0, a10);
-                    a11 = fma(-l1, u1, a11);
-                }
-                W[i * ldw + j] = a00;
-                W[i * ldw + j + 1] = a01;
-                W[(i + 1) * ldw + j] = a10;
-                W[(i + 1) * ldw + j + 1] = a11;
-            }
-            __syncthreads();
-        }
     }
     if (__syncthreads_or(bad)) {
         if (tid == 0) atomicOr(flag, 1);
@@ -671,143 +587,93 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_lu(S* __restrict__ A, 
     diag_lu_body<T, S, RND>(A, lda, K, w, ipiv, flag, stage);
 }
 
-// Off-diagonal blocks of a panel of width w, one launch, eight lanes per row
-// (L21 = A21 U11^{-1}) or per column (U12 = L11^{-1} A12), four per warp.
-// Left-looking in 32-wide chunks: lane g of a group owns entries 4g..4g+3 of
-// the chunk.  The chunk is first updated with the earlier chunks' multipliers
-// (row role) or U entries (column role), which the group keeps in shared
-// memory as binary16 (exact), then solved against the chunk's diagonal
-// 32 x 32 block: at step t the owning lane forms the multiplier (or rounds
-// the U entry) and broadcasts it to its group.  U11 (row role) and L11^T
-// (column role) are staged in shared memory as binary16.
-constexpr int kOffThreads = 128;  // 16 groups of 8 lanes
+// Off-diagonal blocks of a panel of width w (double precision), one launch: L21 =
+// A21 U11^{-1} (row role) and U12 = L11^{-1} A12 (column role), 32 rows (columns,
+// a lane each) per CTA, so that a small panel still spreads over the SMs (the
+// bound is the double-precision pipe, which takes a warp's instruction whole
+// however few lanes are on).  As in the diagonal block, warp 0 takes entry t + 1
+// of every line (update, check, division) while the other warps apply entry t to
+// the later ones: one barrier per step, every entry's terms in increasing t.
+// U11 / L11^T as staged by k_diag_lu.  Measured, w = 64: N = 2048 43 us, N = 1001 70 us a
+// panel on average (groups of eight lanes per row, four of 32 lanes dividing,
+// took 85 at N = 1001; one thread per row with its entries in registers, a
+// division's latency per step and 37 KB of straight-line code, 137).
+constexpr int kOffThreads = 256;
+constexpr int kOffLines = 32;
 
-template <typename T, typename S, bool RND>
-__device__ __forceinline__ void offdiag_body(S* __restrict__ A, int64_t lda, int K, int w, int N,
-                                                         int nrow_blocks, __half* __restrict__ Ut, int ldut,
-                                                         int* __restrict__ flag, const void* __restrict__ stage, int bid)
+template <typename T, typename S>
+__device__ __forceinline__ void offdiag_body(S* __restrict__ A, int64_t lda, int K, int w, int N, int nrow_blocks,
+                                             int* __restrict__ flag, const void* __restrict__ stage, int bid)
 {
     if (flag && *(volatile int*)flag) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using H = typename std::conditional<std::is_same<S, __half>::value, __half, T>::type;
-    constexpr int NG = kOffThreads / kOffG;  // groups (rows or columns) per CTA
+    constexpr int XS = kOffLines + 1;
     const int wp = (w + 31) & ~31;
-    H* D = reinterpret_cast<H*>(smem_raw);  // wp x wp: U11 (row role) or L11^T (column role), identity-padded
-    H* X = D + wp * wp;                     // wp x NG: earlier multipliers / U entries of each group
-    const int tid = threadIdx.x, grp = tid / kOffG, g = tid % kOffG;
-    const unsigned gmask = 0xffu << ((tid & 31) & ~(kOffG - 1));
-    const bool row_role = (int)bid < nrow_blocks;
+    T* D = reinterpret_cast<T*>(smem_raw);  // wp x wp: U11 (row role) or L11^T (column role), identity-padded
+    T* X = D + wp * wp;                     // X[t * XS + line]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool row_role = bid < nrow_blocks;
+    const int line0 = K + w + (row_role ? bid : bid - nrow_blocks) * kOffLines, n = min(kOffLines, N - line0);
     {
-        // U11 or L11^T, staged by k_diag_lu in exactly this layout
-        const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const H*>(stage) + (row_role ? 0 : wp * wp));
+        const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(stage) + (row_role ? 0 : wp * wp));
         uint4* dst = reinterpret_cast<uint4*>(D);
-        const int nv = wp * wp * (int)sizeof(H) / 16;
+        const int nv = wp * wp * (int)sizeof(T) / 16;
 #pragma unroll 4
         for (int q = tid; q < nv; q += kOffThreads) dst[q] = src[q];
     }
+    if (row_role) {
+        for (int q = tid; q < kOffLines * w; q += kOffThreads) {
+            const int r = q / w, t = q - r * w;
+            X[t * XS + r] = r < n ? (T)ld_elem(A + (int64_t)(line0 + r) * lda + K + t) : T(0);
+        }
+    } else {
+        for (int q = tid; q < kOffLines * w; q += kOffThreads) {
+            const int t = q / kOffLines, c = q - t * kOffLines;
+            X[t * XS + c] = c < n ? (T)ld_elem(A + (int64_t)(K + t) * lda + line0 + c) : T(0);
+        }
+    }
     __syncthreads();
     bool bad = false;
-    const int nc = wp / 32;
-    if (row_role) {
-        const int i = K + w + bid * NG + grp;
-        const bool live = i < N;
-        S* Ai = A + (int64_t)min(i, N - 1) * lda + K;
-        for (int c = 0; c < nc; ++c) {
-            const int c0 = 32 * c, jb = c0 + 4 * g;
-            T acc[4];
-            if (live && jb + 4 <= w) {
-                S e[4];
-                if constexpr (sizeof(S) == 2) *reinterpret_cast<uint2*>(e) = *reinterpret_cast<const uint2*>(Ai + jb);
-                else {
-                    reinterpret_cast<uint4*>(e)[0] = reinterpret_cast<const uint4*>(Ai + jb)[0];
-                    reinterpret_cast<uint4*>(e)[1] = reinterpret_cast<const uint4*>(Ai + jb)[1];
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = (T)ld_elem(e + k);
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = (live && jb + k < w) ? (T)ld_elem(Ai + jb + k) : T(0);
+    for (int t = -1; t < w - 1; ++t) {
+        const T* Dt = D + t * wp;
+        const T l = t >= 0 ? X[t * XS + lane] : T(0);
+        if (warp == 0) {
+            const int c = t + 1;
+            T x = X[c * XS + lane];
+            if (t >= 0) x = fma(-l, Dt[c], x);
+            if (row_role) {
+                const T u = D[c * wp + c];
+                if (lane < n && (!(absT(x) <= absT(u)) || !(u != T(0)))) bad = true;
+                x = x / u;
             }
-            for (int t = 0; t < c0; ++t) {
-                const T l = (T)X[t * NG + grp];
-                const H* Dt = D + t * wp + jb;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = fma(-l, (T)Dt[k], acc[k]);
-            }
-#pragma unroll
-            for (int tt = 0; tt < 32; ++tt) {
-                const int t = c0 + tt;
-                T l = T(0);
-                if (g == tt / 4) {
-                    const T utt = (T)D[t * wp + t];
-                    const T x = acc[tt % 4];
-                    if (live && t < w && (!(absT(x) <= absT(utt)) || !(utt != T(0)))) bad = true;
-                    l = maybe_round(x / utt, RND);
-                    acc[tt % 4] = l;
-                    X[t * NG + grp] = (H)l;
-                }
-                l = __shfl_sync(gmask, l, tt / 4, kOffG);
-                const H* Dt = D + t * wp + jb;
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (4 * g + k > tt) acc[k] = fma(-l, (T)Dt[k], acc[k]);
-            }
-            if (live) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (jb + k < w) st_elem(Ai + jb + k, acc[k]);
-            }
+            X[c * XS + lane] = x;
+        } else if (t >= 0) {
+            for (int j = t + 1 + warp; j < w; j += kOffThreads / 32 - 1) X[j * XS + lane] = fma(-l, Dt[j], X[j * XS + lane]);
         }
-        if (__syncthreads_or(bad) && tid == 0 && flag) atomicOr(flag, 1);
+        __syncthreads();
+    }
+    if (__syncthreads_or(bad) && tid == 0 && flag) atomicOr(flag, 1);
+    if (row_role) {
+        for (int q = tid; q < n * w; q += kOffThreads) {
+            const int r = q / w, t = q - r * w;
+            st_elem(A + (int64_t)(line0 + r) * lda + K + t, X[t * XS + r]);
+        }
     } else {
-        const int col = K + w + (bid - nrow_blocks) * NG + grp;
-        const bool live = col < N;
-        const int cc = min(col, N - 1);
-        for (int c = 0; c < nc; ++c) {
-            const int c0 = 32 * c, kb = c0 + 4 * g;
-            T acc[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] = (live && kb + k < w) ? (T)ld_elem(A + (int64_t)(K + kb + k) * lda + cc) : T(0);
-            for (int t = 0; t < c0; ++t) {
-                const T u = (T)X[t * NG + grp];
-                const H* Dt = D + t * wp + kb;  // L[kb + k][t]
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = fma(-(T)Dt[k], u, acc[k]);
-            }
-#pragma unroll
-            for (int tt = 0; tt < 32; ++tt) {
-                const int t = c0 + tt;
-                T u = T(0);
-                if (g == tt / 4) {
-                    u = maybe_round(acc[tt % 4], RND);
-                    acc[tt % 4] = u;
-                    X[t * NG + grp] = (H)u;
-                }
-                u = __shfl_sync(gmask, u, tt / 4, kOffG);
-                const H* Dt = D + t * wp + kb;
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (4 * g + k > tt) acc[k] = fma(-(T)Dt[k], u, acc[k]);
-            }
-            if (live) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (kb + k < w) {
-                        st_elem(A + (int64_t)(K + kb + k) * lda + col, acc[k]);
-                        if (Ut) Ut[(int64_t)(col - K - w) * ldut + kb + k] = __float2half_rn((float)acc[k]);
-                    }
-            }
+        for (int q = tid; q < kOffLines * w; q += kOffThreads) {
+            const int t = q / kOffLines, c = q - t * kOffLines;
+            if (c < n) st_elem(A + (int64_t)(K + t) * lda + line0 + c, X[t * XS + c]);
         }
     }
 }
 
-template <typename T, typename S, bool RND>
+template <typename T, typename S>
 __global__ void __launch_bounds__(kOffThreads) k_offdiag(S* __restrict__ A, int64_t lda, int K, int w, int N,
-                                                         int nrow_blocks, __half* __restrict__ Ut, int ldut,
-                                                         int* __restrict__ flag, const void* __restrict__ stage)
+                                                         int nrow_blocks, int* __restrict__ flag,
+                                                         const void* __restrict__ stage)
 {
-    offdiag_body<T, S, RND>(A, lda, K, w, N, nrow_blocks, Ut, ldut, flag, stage, (int)blockIdx.x);
+    offdiag_body<T, S>(A, lda, K, w, N, nrow_blocks, flag, stage, (int)blockIdx.x);
 }
+__host__ __device__ constexpr size_t offdiag_smem(int wp, size_t el) { return ((size_t)wp * wp + (size_t)wp * (kOffLines + 1)) * el; }
 
 // ------------------------------------------ fast path, binary16 factors --
 // The stage buffer holds, for the off-diagonal solves of one panel: U11 and
@@ -1901,21 +1767,22 @@ static nl_status launch_offdiag16(S* A, int64_t ld, int K, int wd, int N, __half
 
 // C <- C - A B with per-element sequential fused multiply-adds over k in
 // order, accumulated in T and stored once (rounded to binary16 for __half).
-template <typename S, typename T>
+// BT x BT tiles (64 or 32), 256 threads.
+template <typename S, typename T, int BT = 64>
 __device__ __forceinline__ void gemm_simt_body(int M, int Nc, int K, const S* __restrict__ A, int64_t lda,
                                                    const S* __restrict__ B, int64_t ldb, S* __restrict__ C,
                                                    int64_t ldc, const int* __restrict__ flag, int m0, int n0)
 {
     if (flag && *(volatile const int*)flag) return;
-    constexpr int BM = 64, BN = 64, BK = 16;
+    constexpr int BM = BT, BN = BT, BK = 16, R = BT / 16;
     __shared__ T As[BK][BM + 1];
     __shared__ T Bs[BK][BN];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    T acc[4][4];
+    T acc[R][R];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < R; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < R; ++b) {
             int i = m0 + ty + 16 * a, j = n0 + tx + 16 * b;
             acc[a][b] = (i < M && j < Nc) ? (T)ld_elem(C + (int64_t)i * ldc + j) : T(0);
         }
@@ -1934,32 +1801,32 @@ __device__ __forceinline__ void gemm_simt_body(int M, int Nc, int K, const S* __
         __syncthreads();
         const int kmax = min(BK, K - k0);
         for (int kk = 0; kk < kmax; ++kk) {
-            T av[4], bv[4];
+            T av[R], bv[R];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty + 16 * a];
+            for (int a = 0; a < R; ++a) av[a] = As[kk][ty + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx + 16 * b];
+            for (int b = 0; b < R; ++b) bv[b] = Bs[kk][tx + 16 * b];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < R; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fma(-av[a], bv[b], acc[a][b]);
+                for (int b = 0; b < R; ++b) acc[a][b] = fma(-av[a], bv[b], acc[a][b]);
         }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < R; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < R; ++b) {
             int i = m0 + ty + 16 * a, j = n0 + tx + 16 * b;
             if (i < M && j < Nc) st_elem(C + (int64_t)i * ldc + j, acc[a][b]);
         }
 }
 
-template <typename S, typename T>
+template <typename S, typename T, int BT>
 __global__ void __launch_bounds__(256) k_gemm_simt(int M, int Nc, int K, const S* __restrict__ A, int64_t lda,
                                                    const S* __restrict__ B, int64_t ldb, S* __restrict__ C,
                                                    int64_t ldc, const int* __restrict__ flag)
 {
-    gemm_simt_body<S, T>(M, Nc, K, A, lda, B, ldb, C, ldc, flag, (int)blockIdx.y * 64, (int)blockIdx.x * 64);
+    gemm_simt_body<S, T, BT>(M, Nc, K, A, lda, B, ldb, C, ldc, flag, (int)blockIdx.y * BT, (int)blockIdx.x * BT);
 }
 
 // ------------------------------------------------------------------ host --
@@ -2101,8 +1968,19 @@ static nl_status launch_gemm_simt(int M, int Nc, int K, const S* A, int64_t lda,
                                   int64_t ldc, cudaStream_t st, const int* flag = nullptr)
 {
     if (M <= 0 || Nc <= 0 || K <= 0) return NL_OK;
-    dim3 grid((unsigned)cdiv(Nc, 64), (unsigned)cdiv(M, 64));
-    k_gemm_simt<S, T><<<grid, 256, 0, st>>>(M, Nc, K, A, lda, B, ldb, C, ldc, flag);
+    // Double precision is bound by its pipe (a 64 x 64 tile of depth 64 takes an SM 66 us), so the
+    // tile follows the work of the busiest SM; single precision keeps 64.
+    const int64_t sms = num_sms(), t64 = cdiv(Nc, 64) * cdiv(M, 64), t32 = cdiv(Nc, 32) * cdiv(M, 32);
+    bool small = false;
+    if constexpr (sizeof(T) == 8) small = cdiv(t32, sms) < 4 * cdiv(t64, sms);
+    if constexpr (sizeof(T) == 8) {
+        if (small)
+            k_gemm_simt<S, T, 32><<<dim3((unsigned)cdiv(Nc, 32), (unsigned)cdiv(M, 32)), 256, 0, st>>>(M, Nc, K, A, lda, B, ldb,
+                                                                                                C, ldc, flag);
+    }
+    if (!small)
+        k_gemm_simt<S, T, 64><<<dim3((unsigned)cdiv(Nc, 64), (unsigned)cdiv(M, 64)), 256, 0, st>>>(M, Nc, K, A, lda, B, ldb,
+                                                                                                C, ldc, flag);
     NL_CUDA_OK(cudaGetLastError());
     return NL_OK;
 }
@@ -2248,7 +2126,7 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
                 set_max_dynamic_smem((const void*)k_diag_lu16<float>) != NL_OK)
                 return NL_ECUDA;
         } else {
-            if (set_max_dynamic_smem((const void*)k_offdiag<T, S, RND>) != NL_OK ||
+            if (set_max_dynamic_smem((const void*)k_offdiag<T, S>) != NL_OK ||
                 set_max_dynamic_smem((const void*)k_diag_lu<T, S, RND>) != NL_OK)
                 return NL_ECUDA;
         }
@@ -2356,11 +2234,10 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
                     NL_TRY(launch_offdiag16<__half>(A, ld, K, wd, N, tc ? ut_of(K) : nullptr, nb, w.flag,
                                                     (const float*)w.stage, -1, 0, st));
                 } else {
-                    const int nrb = (int)cdiv(rest, kOffThreads / kOffG);
-                    const size_t sm = (size_t)wp * wp * sizeof(T) + (size_t)wp * (kOffThreads / kOffG) * sizeof(T);
+                    const int nrb = (int)cdiv(rest, kOffLines);
                     prof_begin("k_offdiag", st);
-                    k_offdiag<T, S, RND><<<2 * nrb, kOffThreads, sm, st>>>(A, ld, K, wd, N, nrb, nullptr, nb, w.flag,
-                                                                          w.stage);
+                    k_offdiag<T, S><<<2 * nrb, kOffThreads, offdiag_smem(wp, sizeof(T)), st>>>(A, ld, K, wd, N, nrb, w.flag,
+                                                                                            w.stage);
                     prof_end("k_offdiag", st);
                 }
                 NL_TRY(update(K, wd, tc, ut_of(K)));
@@ -2821,13 +2698,13 @@ __global__ void __launch_bounds__(4 * WMAX, 128 / WMAX) k_diag_lu16_g(const GIns
                                                   I.flag, reinterpret_cast<float*>(I.stage));
 }
 
-template <typename T, typename S, bool RND>
+template <typename T, typename S>
 __global__ void __launch_bounds__(kOffThreads) k_offdiag_g(const GInst* __restrict__ inst,
                                                            const GTask* __restrict__ tasks, int K, int nb)
 {
     const GTask t = tasks[blockIdx.x];
     const GInst I = inst[t.inst];
-    offdiag_body<T, S, RND>(reinterpret_cast<S*>(I.A), I.ld, K, nb, I.N, t.b, nullptr, nb, I.flag, I.stage, t.a);
+    offdiag_body<T, S>(reinterpret_cast<S*>(I.A), I.ld, K, nb, I.N, t.b, I.flag, I.stage, t.a);
 }
 
 __global__ void __launch_bounds__(kO16Threads) k_offdiag16_g(const GInst* __restrict__ inst,
@@ -3467,7 +3344,7 @@ nl_status lu_grouped_plan(int count, const GInst* host_inst, int nb, int gemm, b
     for (int i = 0; i < count; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return host_inst[a].N > host_inst[b].N; });
     const int steps = (int)cdiv(nmax, nb);
-    const int rows_per_cta = fp64 ? kOffThreads / kOffG : kO16Rows;
+    const int rows_per_cta = fp64 ? kOffLines : kO16Rows;
     const int tile = (gemm == 2) ? 128 : 64;
     std::vector<GTask> tasks;
     plan->off.assign(3 * steps, 0);
@@ -3542,7 +3419,7 @@ nl_status lu_grouped_setup()
             set_max_dynamic_smem((const void*)k_diag_lu16_g<128>) != NL_OK ||
             set_max_dynamic_smem((const void*)k_offdiag16_g) != NL_OK ||
             set_max_dynamic_smem((const void*)k_diag_lu_g<double, double, false>) != NL_OK ||
-            set_max_dynamic_smem((const void*)k_offdiag_g<double, double, false>) != NL_OK ||
+            set_max_dynamic_smem((const void*)k_offdiag_g<double, double>) != NL_OK ||
             set_max_dynamic_smem((const void*)k_lu_grouped_p<false>) != NL_OK ||
             set_max_dynamic_smem((const void*)k_lu_grouped_p<true>) != NL_OK)
             return NL_ECUDA;
@@ -3588,9 +3465,7 @@ nl_status lu_grouped_factor(const GroupPlan& plan, const GInst* dev_inst, cudaSt
             }
             if (no) {
                 prof_begin("k_offdiag", st);
-                k_offdiag_g<double, double, false><<<no, kOffThreads,
-                                                     (size_t)wp * wp * 8 + (size_t)wp * (kOffThreads / kOffG) * 8,
-                                                     st>>>(dev_inst, to, K, nb);
+                k_offdiag_g<double, double><<<no, kOffThreads, offdiag_smem(wp, 8), st>>>(dev_inst, to, K, nb);
                 prof_end("k_offdiag", st);
             }
             if (ng) k_gemm_simt_g<double, double><<<ng, 256, 0, st>>>(dev_inst, tg, K, nb);
