@@ -677,8 +677,8 @@ __host__ __device__ constexpr size_t offdiag_smem(int wp, size_t el) { return ((
 
 // ------------------------------------------ fast path, binary16 factors --
 // The stage buffer holds, for the off-diagonal solves of one panel: U11 and
-// L11^T (wp x wp binary32 each, the exact binary16 values, identity / zero
-// padded) and the unrounded pivots a_tt (kStagePivOff floats in).
+// -L11^T (wp x wp binary16 each, identity / zero padded) and the unrounded
+// pivots a_tt (kStagePivOff floats in).
 constexpr int kStagePivOff = 2 * 128 * 128;
 
 // k_diag_lu16: the diagonal block [K, K+w)^2 (w <= 128) in one CTA, right-looking
@@ -920,7 +920,7 @@ __device__ __forceinline__ void diag16_publish(int s, int w8, const unsigned sho
 }
 
 // PUB: also publish the block as it is factored, for the streaming solves of
-// k_panel16.  stage (may be null): U11, L11^T and the pivots for k_offdiag16.
+// k_panel16.  stage (may be null): U11, -L11^T and the pivots for k_offdiag16.
 // CROSS: the block first takes its part of the last update (ct).
 template <bool PUB = false, typename S_ = __half, int WMAX = 128, int NT = kD16Threads, bool CROSS = false>
 __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, int K, int w,
@@ -1179,15 +1179,16 @@ __device__ __forceinline__ void diag_lu16_body(S_* __restrict__ A, int64_t lda, 
             if (C + c < w) st_elem(dst + c, h_val((c & 1) ? h_hi(hw[c / 2]) : h_lo(hw[c / 2])));
     }
     if (stage) {
-        // U11 and L11^T (binary32, identity / zero padded to wp) and the pivots
+        // U11 and -L11^T (binary16, identity / zero padded to wp) and the pivots
         const int wp = (w + 31) & ~31;
-        float* SU = stage;
-        float* SL = stage + wp * wp;
-        for (int p = tid; p < wp * wp; p += NT) {
-            const int i = p / wp, j = p - i * wp;
-            SU[p] = (i < w && j < w) ? (j >= i ? h_val(Hs[i * HLD + j]) : 0.0f) : (i == j ? 1.0f : 0.0f);
-            SL[p] = (i < w && j < w && j > i) ? h_val(Hs[j * HLD + i] ^ 0x8000u) : 0.0f;
-        }
+        unsigned short* SU = reinterpret_cast<unsigned short*>(stage);
+        unsigned short* SL = SU + wp * wp;
+        for (int i = wid; i < wp; i += NW)
+            for (int j = lane; j < wp; j += 32) {
+                const bool in = i < w && j < w;
+                SU[i * wp + j] = in ? (j >= i ? Hs[i * HLD + j] : (unsigned short)0) : (unsigned short)(i == j ? 0x3c00 : 0);
+                SL[i * wp + j] = (in && j > i) ? Hs[j * HLD + i] : (unsigned short)0;
+            }
         if (tid < w) stage[kStagePivOff + tid] = rc[tid].z;
     }
     if (tid < w) ipiv[K + tid] = K + tid;
@@ -1274,12 +1275,12 @@ __device__ __forceinline__ void pnl_wait_ready(uint32_t bar, int* gave_up)
     *(volatile int*)gave_up = 1;
 }
 
-// x[e] += h_k M[k][e], k = 0..7 in order: block b's finished eight (hist) applied to eight later entries
-__device__ __forceinline__ void pnl_apply(const uint4& hist, const unsigned short* __restrict__ M, float (&x)[8])
+// x[e] += h_k M[k][e], k = 0..7 in order: a block's finished eight (hist) applied to eight later entries
+__device__ __forceinline__ void pnl_apply(const uint4& hist, const unsigned short* __restrict__ M, int ldm, float (&x)[8])
 {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const uint4 m = *reinterpret_cast<const uint4*>(M + k * kPnlMld);
+        const uint4 m = *reinterpret_cast<const uint4*>(M + k * ldm);
         const unsigned short h = h_at(hist, k);
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[e] = fma_h(h, h_at(m, e), x[e]);
@@ -1380,7 +1381,7 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
                 float x[8];
                 *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xl);
                 *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(xl + 4);
-                if (q > 0) pnl_apply(*reinterpret_cast<const uint4*>(xl - 8), M + B0 * kPnlMld + C0, x);
+                if (q > 0) pnl_apply(*reinterpret_cast<const uint4*>(xl - 8), M + B0 * kPnlMld + C0, kPnlMld, x);
                 unsigned short h[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
@@ -1405,7 +1406,7 @@ __device__ __forceinline__ void panel16_stream(S* __restrict__ A, int64_t lda, i
                     float x[8];
                     *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(xl + C);
                     *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(xl + C + 4);
-                    pnl_apply(*reinterpret_cast<const uint4*>(xl + B0), M + B0 * kPnlMld + C, x);
+                    pnl_apply(*reinterpret_cast<const uint4*>(xl + B0), M + B0 * kPnlMld + C, kPnlMld, x);
                     *reinterpret_cast<float4*>(xl + C) = make_float4(x[0], x[1], x[2], x[3]);
                     *reinterpret_cast<float4*>(xl + C + 4) = make_float4(x[4], x[5], x[6], x[7]);
                 }
@@ -1565,18 +1566,21 @@ __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16x(const __grid_consta
 
 // k_offdiag16: L21 = A21 U11^{-1} (row role) and U12 = L11^{-1} A12 (column
 // role) for a panel of width w, one thread per row (or column), 128 per CTA.
-// A thread takes its row in 32-wide chunks: the chunk is first updated with
-// the row's multipliers of the earlier chunks (kept in shared memory, one
-// column of X per thread), then solved against the chunk's diagonal 32 x 32
-// block of U11: at step t the thread checks its pre-division value against
-// the unrounded pivot, forms l = fl16(x_t / u_tt) and updates the rest of
-// the chunk.  The column role is the same with L11 and no division (U
-// entries rounded to binary16 as they are formed), and also writes U12^T for
-// the tensor-core update.  U11 / L11^T come from the stage as binary32 (exact
-// binary16 values) and are read by all threads at once (broadcast).  Every
-// entry takes its updates in increasing t, as in right-looking elimination;
-// with no shuffles or group hand-offs the per-step chain is one multiplier
-// formation and one fused multiply-add.
+// A thread takes its row in blocks of eight, left-looking: the block is first
+// updated with the row's earlier blocks (kept in shared memory as binary16, the
+// multipliers negated), then solved against its diagonal 8 x 8 block of U11: at
+// step t the thread checks its pre-division value against the unrounded pivot and
+// forms l = fl16(x_t / u_tt).  The column role is the same with -L11 and no
+// division (U entries rounded to binary16 as they are formed), and also writes
+// U12^T for the tensor-core update.  U11 / -L11^T come from the stage as
+// binary16 and are read by all threads at once (broadcast), eight entries a
+// load, for fma.rn.f32.f16.  Every entry takes its updates in increasing t, as in
+// right-looking elimination.  Bound by the multiply-adds where a launch fills the
+// GPU, else by one CTA's time; the loops are short on purpose: the former
+// straight-line solve of 32 entries ran from instruction memory once per chunk,
+// and a line's entries are all loaded at the start (loaded block by block they
+// were the longest stall).  A launch of a few CTAs at w = 64 takes 16 us (42
+// before); the 512-instance batch's grouped factorisation 3.4 ms (4.2).
 constexpr int kO16Threads = 128;
 constexpr int kO16Rows = 128;  // rows or columns per CTA
 
@@ -1584,7 +1588,7 @@ constexpr int kO16Rows = 128;  // rows or columns per CTA
 // 128-column panels (twice the warps per SM at one CTA per SM)
 __host__ __device__ size_t offdiag16_smem(int wp, int R = kO16Rows)
 {
-    return ((size_t)wp * wp + (size_t)wp * R + 2 * wp) * sizeof(float);
+    return ((size_t)wp * wp + (size_t)wp * R) * 2 + 2 * wp * sizeof(float);
 }
 
 template <typename S = __half, int ROWS = kO16Rows>
@@ -1597,137 +1601,120 @@ __device__ __forceinline__ void offdiag16_body(S* __restrict__ A, int64_t lda, i
     if (ut_col0 < 0) ut_col0 = K + w;
     if (tid_in < 0 && *(volatile int*)flag) return;  // (a group of a larger CTA: its caller checked)
     extern __shared__ __align__(16) float osm[];
-    const int wp = (w + 31) & ~31, nc = wp / 32;
+    const int wp = (w + 31) & ~31;
     // tid_in / smem: a group of 128 threads of a larger CTA and its own shared region (the
     // persistent grouped factorisation runs four such groups side by side)
-    float* D = smem ? smem : osm;    // U11 (row role) or L11^T (column role), wp x wp
-    float* X = D + wp * wp;          // X[t * ROWS + tid]: this thread's multipliers / U entries
-    float* pv = X + wp * ROWS;          // |a_tt|, unrounded
-    float* rinv = pv + wp;           // rcp_neg_abs(u_tt)
+    unsigned short* D = reinterpret_cast<unsigned short*>(smem ? smem : osm);  // U11 (rows) or -L11^T (columns), wp x wp
+    unsigned short* X = D + wp * wp;   // every thread's finished blocks: multipliers (negated) / U entries
+    float* pv = reinterpret_cast<float*>(X + wp * ROWS);  // a_tt, unrounded
+    float* rinv = pv + wp;             // rcp_neg_abs(u_tt)
     const int tid = tid_in >= 0 ? tid_in : (int)threadIdx.x;
     const bool row_role = bid < nrow_blocks;
     {
-        const float4* s4 = reinterpret_cast<const float4*>(stage + (row_role ? 0 : wp * wp));
-        float4* d4 = reinterpret_cast<float4*>(D);
-        const int nv = wp * wp / 4;
+        const uint4* s4 = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned short*>(stage) +
+                                                         (row_role ? 0 : wp * wp));
+        uint4* d4 = reinterpret_cast<uint4*>(D);
+        const int nv = wp * wp / 8;
 #pragma unroll 4
         for (int v = tid; v < nv; v += ROWS) d4[v] = s4[v];
-        if (tid < wp) pv[tid] = fabsf(stage[kStagePivOff + tid]);
+        if (tid < wp) pv[tid] = tid < w ? stage[kStagePivOff + tid] : 1.0f;
     }
     __syncthreads();
-    if (row_role && tid < wp) rinv[tid] = rcp_neg_abs(D[tid * wp + tid]);
+    if (row_role && tid < wp) rinv[tid] = rcp_neg_abs(h_val(D[tid * wp + tid]));
     __syncthreads();
     const int idx = K + w + (row_role ? bid : bid - nrow_blocks) * ROWS + tid;
     const bool live = idx < N;
-    float* Xt = X + tid;
-    if (row_role) {
-        bool bad = false;
-        S* R = A + (int64_t)min(idx, N - 1) * lda + K;
-        const bool vec = (w % 32 == 0) && ((((uintptr_t)(A + K)) & 15) == 0) && (lda % 8 == 0);
-        for (int c = 0; c < nc; ++c) {
-            const int j0 = 32 * c;
-            float x[32];
-            if (vec && live) {
+    uint4* H = reinterpret_cast<uint4*>(X) + tid;     // H[q * ROWS]: block q of this thread
+    S* R = A + (int64_t)min(idx, N - 1) * lda + K;    // the row, or
+    S* Cl = A + (int64_t)K * lda + min(idx, N - 1);   // the column
+    const bool vec = (w % 8 == 0) && ((((uintptr_t)(A + K)) & 15) == 0) && (lda % 8 == 0);
+    const bool uvec = Ut && idx >= ut_col0 && (w % 8 == 0) && (ldut % 8 == 0) && (ut_k0 % 8 == 0) && ((((uintptr_t)Ut) & 15) == 0);
+    __half* ut = Ut + (Ut ? (int64_t)(idx - ut_col0) * ldut + ut_k0 : 0);
+    const int nq = (w + 7) >> 3;
+    bool bad = false;
+    constexpr bool kHalf = std::is_same<S, __half>::value;
+    if constexpr (kHalf) {
+        // every block's entries first, all loads in flight, to where its solved ones will stand
+#pragma unroll 4
+        for (int q = 0; q < nq; ++q) {
+            uint4 v;
+            if (row_role && vec) {
+                v = *reinterpret_cast<const uint4*>(R + 8 * q);
+            } else {
+                unsigned short e[8];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) load8(R + j0 + 8 * q, x + 8 * q);
+                for (int k = 0; k < 8; ++k) {
+                    const int t = 8 * q + k;
+                    e[k] = t < w ? __half_as_ushort(row_role ? R[t] : Cl[(int64_t)t * lda]) : (unsigned short)0;
+                }
+                v = make_uint4(h_pack(e[0], e[1]), h_pack(e[2], e[3]), h_pack(e[4], e[5]), h_pack(e[6], e[7]));
+            }
+            H[q * ROWS] = v;
+        }
+    }
+#pragma unroll 1
+    for (int q = 0; q < nq; ++q) {
+        const int C = 8 * q;
+        float x[8];
+        if constexpr (kHalf) {
+            const uint4 v = H[q * ROWS];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = h_val(h_at(v, k));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                x[k] = (C + k < w) ? ld_elem(row_role ? R + C + k : Cl + (int64_t)(C + k) * lda) : 0.0f;
+        }
+#pragma unroll 1
+        for (int b = 0; b < q; ++b) pnl_apply(H[b * ROWS], D + 8 * b * wp + C, wp, x);
+        unsigned short h[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint4 m = *reinterpret_cast<const uint4*>(D + (C + k) * wp + C);
+            if (row_role) {
+                const float p = pv[C + k];
+                bad |= live && C + k < w && !(fabsf(x[k]) <= fabsf(p));
+                h[k] = h_bits(div_neg(x[k], p, rinv[C + k], fabsf(h_val(h_at(m, k)))));
+            } else {
+                h[k] = h_bits(x[k]);
+            }
+#pragma unroll
+            for (int e = k + 1; e < 8; ++e) x[e] = fma_h(h[k], h_at(m, e), x[e]);
+        }
+        uint4 hv = make_uint4(h_pack(h[0], h[1]), h_pack(h[2], h[3]), h_pack(h[4], h[5]), h_pack(h[6], h[7]));
+        H[q * ROWS] = hv;
+        if (!live) continue;
+        if (row_role) {
+            hv.x ^= 0x80008000u; hv.y ^= 0x80008000u; hv.z ^= 0x80008000u; hv.w ^= 0x80008000u;
+            if (vec) {
+                if constexpr (std::is_same<S, __half>::value) {
+                    *reinterpret_cast<uint4*>(R + C) = hv;
+                } else {
+                    float v[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = h_val(h_at(hv, e));
+                    store8(R + C, v);
+                }
             } else {
 #pragma unroll
-                for (int k = 0; k < 32; ++k) x[k] = (live && j0 + k < w) ? ld_elem(R + j0 + k) : 0.0f;
+                for (int e = 0; e < 8; ++e)
+                    if (C + e < w) st_elem(R + C + e, h_val(h_at(hv, e)));
             }
-#pragma unroll 8
-            for (int t = 0; t < j0; ++t) {
-                const float l = Xt[t * ROWS];
-                const float4* Dt = reinterpret_cast<const float4*>(D + t * wp + j0);
+        } else {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 d = Dt[q];
-                    x[4 * q + 0] = fmaf(-l, d.x, x[4 * q + 0]);
-                    x[4 * q + 1] = fmaf(-l, d.y, x[4 * q + 1]);
-                    x[4 * q + 2] = fmaf(-l, d.z, x[4 * q + 2]);
-                    x[4 * q + 3] = fmaf(-l, d.w, x[4 * q + 3]);
-                }
-            }
+            for (int e = 0; e < 8; ++e)
+                if (C + e < w) st_elem(Cl + (int64_t)(C + e) * lda, h_val(h_at(hv, e)));
+            if (uvec) {
+                *reinterpret_cast<uint4*>(ut + C) = hv;  // U12^T row (the tensor-core B operand)
+            } else if (Ut && idx >= ut_col0) {
 #pragma unroll
-            for (int tt = 0; tt < 32; ++tt) {
-                const int t = j0 + tt;
-                const float* Dt = D + t * wp + j0;
-                if (live && t < w && !(fabsf(x[tt]) <= pv[t])) bad = true;
-                const float u = Dt[tt], l = -round_h(div_neg(x[tt], u, rinv[t], fabsf(u)));
-                x[tt] = l;
-#pragma unroll
-                for (int k = tt + 1; k < 32; ++k) x[k] = fmaf(-l, Dt[k], x[k]);
-            }
-            // the chunk's multipliers for the later chunks (no shared-memory stores inside
-            // the solve, so the loads of U11 can move ahead of the division chain)
-#pragma unroll
-            for (int tt = 0; tt < 32; ++tt) Xt[(j0 + tt) * ROWS] = x[tt];
-            if (live) {
-                if (vec) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) store8(R + j0 + 8 * q, x + 8 * q);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k)
-                        if (j0 + k < w) st_elem(R + j0 + k, x[k]);
-                }
+                for (int e = 0; e < 8; ++e)
+                    if (C + e < w) ut[C + e] = __ushort_as_half(h_at(hv, e));
             }
         }
+    }
+    if (row_role) {  // (the groups of a larger CTA share a role)
         if (__syncthreads_or(bad) && tid == 0) atomicOr(flag, 1);
-    } else {
-        const int col = min(idx, N - 1);
-        for (int c = 0; c < nc; ++c) {
-            const int k0 = 32 * c;
-            float x[32];
-#pragma unroll
-            for (int k = 0; k < 32; ++k)
-                x[k] = (live && k0 + k < w) ? ld_elem(A + (int64_t)(K + k0 + k) * lda + col) : 0.0f;
-#pragma unroll 8
-            for (int t = 0; t < k0; ++t) {
-                const float u = Xt[t * ROWS];
-                const float4* Dt = reinterpret_cast<const float4*>(D + t * wp + k0);  // L[k0 + k][t]
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 d = Dt[q];
-                    x[4 * q + 0] = fmaf(-d.x, u, x[4 * q + 0]);
-                    x[4 * q + 1] = fmaf(-d.y, u, x[4 * q + 1]);
-                    x[4 * q + 2] = fmaf(-d.z, u, x[4 * q + 2]);
-                    x[4 * q + 3] = fmaf(-d.w, u, x[4 * q + 3]);
-                }
-            }
-#pragma unroll
-            for (int tt = 0; tt < 32; ++tt) {
-                const int t = k0 + tt;
-                const float* Dt = D + t * wp + k0;
-                const float u = round_h(x[tt]);
-                x[tt] = u;
-#pragma unroll
-                for (int k = tt + 1; k < 32; ++k) x[k] = fmaf(-Dt[k], u, x[k]);
-            }
-#pragma unroll
-            for (int tt = 0; tt < 32; ++tt) Xt[(k0 + tt) * ROWS] = x[tt];
-            if (live) {
-#pragma unroll
-                for (int k = 0; k < 32; ++k)
-                    if (k0 + k < w) st_elem(A + (int64_t)(K + k0 + k) * lda + col, x[k]);
-                if (Ut && idx >= ut_col0) {
-                    // U12^T row (the tensor-core B operand): 32 consecutive entries
-                    __half* u0 = Ut + (int64_t)(idx - ut_col0) * ldut + ut_k0 + k0;
-                    if (k0 + 32 <= w && (ldut % 8 == 0) && (ut_k0 % 8 == 0) && ((((uintptr_t)Ut) & 15) == 0)) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            __align__(16) __half h[8];
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) h[k] = __float2half_rn(x[8 * q + k]);
-                            reinterpret_cast<uint4*>(u0)[q] = *reinterpret_cast<const uint4*>(h);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 32; ++k)
-                            if (k0 + k < w) u0[k] = __float2half_rn(x[k]);
-                    }
-                }
-            }
-        }
     }
 }
 
