@@ -497,7 +497,7 @@ struct nl_batch {
     std::vector<double> c;
     std::vector<int64_t> off;  // packed vector offsets
     std::vector<int> ld;
-    int nmax = 0, total_rows = 0;
+    int nmax = 0, maxld = 0;
     cudaStream_t st = nullptr, s1 = nullptr, s2 = nullptr;
     bool own_streams = false, own_st = true;
     // device memory
@@ -517,7 +517,6 @@ struct nl_batch {
     std::vector<GInst> hgin, hgin64;
     BTask *res_tasks = nullptr, *gemv_tasks = nullptr;
     int n_res = 0, n_gemv = 0;
-    int* row_off = nullptr;
     int* order = nullptr;
     double* htab = nullptr;
     float* htab32 = nullptr;  // the same table rounded to single (the Jacobian's entries use it)
@@ -621,7 +620,7 @@ static nl_status batch_time_lu16(nl_batch* B, double* ms_out)
     for (int rep = 0; rep < 3 && s == NL_OK; ++rep) {
         if (cudaMemsetAsync(B->flags, 0, sizeof(int) * B->count, B->st) != cudaSuccess) s = NL_ECUDA;
         if (s == NL_OK)
-            s = launch_jacobian_g(B->dinst, B->dst, B->row_off, B->count, B->total_rows, B->htab, B->htab32, 0,
+            s = launch_jacobian_g(B->dinst, B->dst, B->res_tasks, B->n_res, B->maxld, B->htab, B->htab32, 0,
                                   B->st);
         if (s != NL_OK) break;
         cudaEventRecord(e0, B->st);
@@ -743,7 +742,7 @@ static nl_status batch_autotune(nl_batch* B)
             for (int rep = 0; rep < 2 && s == NL_OK; ++rep) {
                 if (cudaMemsetAsync(B->flags, 0, sizeof(int) * B->count, B->st) != cudaSuccess) s = NL_ECUDA;
                 if (s == NL_OK)
-                    s = launch_jacobian_g(B->dinst, B->dst, B->row_off, B->count, B->total_rows, B->htab, B->htab32,
+                    s = launch_jacobian_g(B->dinst, B->dst, B->res_tasks, B->n_res, B->maxld, B->htab, B->htab32,
                                           0, B->st);
                 if (s != NL_OK) break;
                 cudaEventRecord(e0, B->st);
@@ -825,7 +824,6 @@ nl_status nl_batch_create(int count, const int64_t* N, const double* c, const nl
         B->ld[i] = (int)round_up(N[i], 64);
         B->nmax = std::max(B->nmax, B->N[i]);
     }
-    B->total_rows = (int)B->off[count];
     const int64_t tot = B->off[count];
     if (cudaStreamCreateWithFlags(&B->st, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&B->s1, cudaStreamNonBlocking) != cudaSuccess ||
@@ -852,8 +850,7 @@ nl_status nl_batch_create(int count, const int64_t* N, const double* c, const nl
     }
     B->n_res = (int)rt.size();
     B->n_gemv = (int)gt.size();
-    std::vector<int> row_off(count + 1);
-    for (int i = 0; i <= count; ++i) row_off[i] = (int)B->off[i];
+    for (int i = 0; i < count; ++i) B->maxld = std::max(B->maxld, (int)B->ld[i]);
     // sizes
     auto carve = [&](Carver& cv) {
         cv.take<BInst>(count);
@@ -866,7 +863,6 @@ nl_status nl_batch_create(int count, const int64_t* N, const double* c, const nl
         cv.take<int>(count);  // flags
         cv.take<BTask>(rt.size());
         cv.take<BTask>(gt.size());
-        cv.take<int>(count + 1);
         cv.take<int>(count);
         cv.take<double>(2 * (size_t)B->nmax);
         cv.take<float>(2 * (size_t)B->nmax);
@@ -913,7 +909,6 @@ nl_status nl_batch_create(int count, const int64_t* N, const double* c, const nl
     B->flags = flags;
     B->res_tasks = cv.take<BTask>(rt.size());
     B->gemv_tasks = cv.take<BTask>(gt.size());
-    B->row_off = cv.take<int>(count + 1);
     B->order = cv.take<int>(count);
     B->htab = cv.take<double>(2 * (size_t)B->nmax);
     B->htab32 = cv.take<float>(2 * (size_t)B->nmax);
@@ -1015,7 +1010,6 @@ nl_status nl_batch_create(int count, const int64_t* N, const double* c, const nl
         cudaMemcpy(B->gin, B->hgin.data(), sizeof(GInst) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(B->res_tasks, rt.data(), sizeof(BTask) * rt.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(B->gemv_tasks, gt.data(), sizeof(BTask) * gt.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(B->row_off, row_off.data(), sizeof(int) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(B->order, order.data(), sizeof(int) * count, cudaMemcpyHostToDevice) != cudaSuccess) {
         set_error("nl_batch_create: table upload failed");
         batch_free(B);
@@ -1157,7 +1151,7 @@ static nl_status batch_build_graph(nl_batch* B, int fp64)
         k_b_cond<<<1, 1, 0, s0>>>(B->ctl, 0, 1, C.newton_maxit, hN);
         if ((s = add_while_node(s0, s1, hN)) != NL_OK) break;
         // ---- Newton step body (s1)
-        if ((s = launch_jacobian_g(inst, B->dst, B->row_off, count, B->total_rows, B->htab, B->htab32, fp64, s1)) !=
+        if ((s = launch_jacobian_g(inst, B->dst, B->res_tasks, B->n_res, B->maxld, B->htab, B->htab32, fp64, s1)) !=
             NL_OK)
             break;
         nodes_step = 1;

@@ -182,8 +182,9 @@ int gemv_block_rows();      // rows per block of the grouped residual GEMV
 // Modes 1 and 2 skip instances that are not BS_ACTIVE.  The last block of an instance writes st.fn.
 nl_status launch_residual_g(const BInst* inst, BState* st, const BTask* tasks, int ntasks, int mode,
                             const double* htab, cudaStream_t st_);
-// J32/J16 (fp64 = 0) or J64 (fp64 = 1) of the BS_ACTIVE instances; rows = total rows, row_off[count + 1].
-nl_status launch_jacobian_g(const BInst* inst, const BState* st, const int* row_off, int count, int rows,
+// J32/J16 (fp64 = 0) or J64 (fp64 = 1) of the BS_ACTIVE instances; tasks of residual_block_rows() rows, maxld the
+// largest row stride.
+nl_status launch_jacobian_g(const BInst* inst, const BState* st, const BTask* tasks, int ntasks, int maxld,
                             const double* htab, const float* htab32, int fp64, cudaStream_t st_);
 // r = b - J32 u of instances with lin_active; the last block of an instance writes st.nr_new.
 nl_status launch_gemv_residual_g(const BInst* inst, BState* st, const BTask* tasks, int ntasks, cudaStream_t st_);

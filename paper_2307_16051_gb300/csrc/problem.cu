@@ -308,62 +308,77 @@ nl_status launch_jacobian64(int N, double c, const double* rr, const double* hta
     return NL_OK;
 }
 
-// Grouped Jacobian: one block per row of one instance (row_off gives the
-// instance's first global row), the same arithmetic as k_jacobian /
-// k_jacobian64.  Instances that are not BS_ACTIVE are skipped.
+// Grouped Jacobian: one block per task {instance, first of kFRows rows}, the
+// same arithmetic as k_jacobian / k_jacobian64.  Instances that are not BS_ACTIVE
+// are skipped.  Bound by the stores (6 bytes an entry).  The rows' factors
+// (double arithmetic with a division) are formed once by one lane each and the
+// Hankel window is staged once for the 32 rows; a thread takes four columns of
+// its rows, one new window entry per row.  A block per row, which searched its
+// instance and formed its factor in one thread, took 778 us for the 512-instance
+// batch (1.9 GB of stores); this takes 251.
+constexpr int kJgMaxLd = 8192;  // largest row stride of an instance (N <= 8192)
+constexpr size_t kJgSmem = (kJgMaxLd + kFRows) * sizeof(float);
 __global__ void __launch_bounds__(256) k_jacobian_g(const BInst* __restrict__ inst, const BState* __restrict__ st,
-                                                    const int* __restrict__ row_off, int count,
-                                                    const double* __restrict__ htab,
+                                                    const BTask* __restrict__ tasks, const double* __restrict__ htab,
                                                     const float* __restrict__ htab32, int fp64)
 {
-    const int g = blockIdx.x;
-    int lo = 0, hi = count - 1;  // last instance with row_off[k] <= g
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (row_off[mid] <= g) lo = mid;
-        else hi = mid - 1;
+    extern __shared__ float hs[];  // hs[q] = h[i0 + q]
+    __shared__ double wd[kFRows];
+    const BTask tk = tasks[blockIdx.x];
+    if (st[tk.inst].status != BS_ACTIVE) return;
+    const BInst& I = inst[tk.inst];
+    const int i0 = tk.i0, N = I.N, ld = I.ld, rows = min(kFRows, N - i0), tid = threadIdx.x;
+    if (tid < rows) {
+        const int i = i0 + tid;
+        const double ri = I.rr[i];
+        wd[tid] = I.c / (2.0 * (double)N) * ri * ri * ((double)i + 0.5);
     }
-    const BInst& I = inst[lo];
-    if (st[lo].status != BS_ACTIVE) return;
-    const int i = g - row_off[lo], N = I.N;
-    const double ri = I.rr[i];
+    if (!fp64)
+        for (int q = tid; q < ld + rows; q += 256) hs[q] = (i0 + q < 2 * N - 1) ? htab32[i0 + q] : 0.0f;
+    __syncthreads();
     if (fp64) {
-        const double w = I.c / (2.0 * (double)N) * ri * ri * ((double)i + 0.5);
-        double* Ji = reinterpret_cast<double*>(I.J) + (int64_t)i * I.ld;
-        for (int j = threadIdx.x; j < I.ld; j += blockDim.x)
-            Ji[j] = (j < N) ? fma(-w, htab[i + j], (i == j) ? 1.0 : 0.0) : 0.0;
+        double* J = reinterpret_cast<double*>(I.J) + (int64_t)i0 * ld;
+        for (int q = tid; q < rows * ld; q += 256) {
+            const int r = q / ld, j = q - r * ld, i = i0 + r;
+            J[q] = (j < N) ? fma(-wd[r], htab[i + j], (i == j) ? 1.0 : 0.0) : 0.0;
+        }
         return;
     }
-    // the row factor once per row (double arithmetic), the Hankel entries from the single table
-    __shared__ float wsh;
-    if (threadIdx.x == 0) wsh = (float)(I.c / (2.0 * (double)N) * ri * ri * ((double)i + 0.5));
-    __syncthreads();
-    const float w = wsh;
-    for (int j0 = threadIdx.x * kJCols; j0 < I.ld; j0 += blockDim.x * kJCols) {
-        float v[kJCols];
-#pragma unroll
-        for (int t = 0; t < kJCols; ++t) {
-            const int j = j0 + t;
-            float e = 0.0f;
-            if (j < N) e = fmaf(-w, htab32[i + j], (i == j) ? 1.0f : 0.0f);
-            v[t] = e;
+    // groups of four columns; with fewer groups than threads, sets of them share the rows
+    const int ng = ld >> 2, ns = ng < 256 ? 256 / ng : 1, set = ng < 256 ? tid / ng : 0;
+    if (set >= ns) return;
+    const int ra = rows * set / ns, rb = rows * (set + 1) / ns;
+    for (int g = tid - set * ng; g < ng; g += 256) {
+        const int j = 4 * g;
+        float h0 = hs[ra + j], h1 = hs[ra + j + 1], h2 = hs[ra + j + 2];
+        float* p = I.J32 + (int64_t)(i0 + ra) * ld + j;
+        __half* ph = reinterpret_cast<__half*>(I.J) + (int64_t)(i0 + ra) * ld + j;
+        for (int r = ra; r < rb; ++r, p += ld, ph += ld) {
+            const float h3 = hs[r + j + 3], w = (float)wd[r];
+            const int di = i0 + r - j;  // the diagonal's place in the group
+            const float v0 = j < N ? fmaf(-w, h0, di == 0 ? 1.0f : 0.0f) : 0.0f;
+            const float v1 = j + 1 < N ? fmaf(-w, h1, di == 1 ? 1.0f : 0.0f) : 0.0f;
+            const float v2 = j + 2 < N ? fmaf(-w, h2, di == 2 ? 1.0f : 0.0f) : 0.0f;
+            const float v3 = j + 3 < N ? fmaf(-w, h3, di == 3 ? 1.0f : 0.0f) : 0.0f;
+            *reinterpret_cast<float4*>(p) = make_float4(v0, v1, v2, v3);
+            const __half2 a = __floats2half2_rn(v0, v1), b = __floats2half2_rn(v2, v3);
+            *reinterpret_cast<uint2*>(ph) =
+                make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b));
+            h0 = h1;
+            h1 = h2;
+            h2 = h3;
         }
-        float4* p = reinterpret_cast<float4*>(I.J32 + (int64_t)i * I.ld + j0);
-        p[0] = make_float4(v[0], v[1], v[2], v[3]);
-        p[1] = make_float4(v[4], v[5], v[6], v[7]);
-        __align__(16) __half h[kJCols];
-#pragma unroll
-        for (int t = 0; t < kJCols; ++t) h[t] = __float2half_rn(v[t]);
-        *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(I.J) + (int64_t)i * I.ld + j0) =
-            *reinterpret_cast<uint4*>(h);
     }
 }
 
-nl_status launch_jacobian_g(const BInst* inst, const BState* st, const int* row_off, int count, int rows,
+// tasks: of residual_block_rows() rows; maxld: the largest instance's row stride
+nl_status launch_jacobian_g(const BInst* inst, const BState* st, const BTask* tasks, int ntasks, int maxld,
                             const double* htab, const float* htab32, int fp64, cudaStream_t st_)
 {
-    if (rows <= 0) return NL_OK;
-    k_jacobian_g<<<(unsigned)rows, 256, 0, st_>>>(inst, st, row_off, count, htab, htab32, fp64);
+    if (ntasks <= 0) return NL_OK;
+    const size_t smem = fp64 ? 0 : ((size_t)maxld + kFRows) * sizeof(float);
+    static_assert(kJgSmem <= 48 * 1024, "no opt-in needed");
+    k_jacobian_g<<<(unsigned)ntasks, 256, smem, st_>>>(inst, st, tasks, htab, htab32, fp64);
     NL_CUDA_OK(cudaGetLastError());
     return NL_OK;
 }
