@@ -1534,7 +1534,7 @@ __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16(S* __restrict__ A, i
 // k_panel16 for a panel of 128 columns after a panel of 128 whose update has not
 // touched the panel's rows and columns yet: every CTA first applies it to its own
 // tile (cross_begin / cross_end).  mA: L21 of the last panel from row K on, mB: its
-// U12^T from column K on.  rpc: 64 or 128.
+// U12^T from column K on.  rpc: 64, 96 or 128.
 __global__ void __launch_bounds__(kPnlThreads, 1) k_panel16x(const __grid_constant__ CUtensorMap mA,
                                                             const __grid_constant__ CUtensorMap mB,
                                                             __half* __restrict__ A, int64_t lda, int K, int w, int N,
@@ -2038,13 +2038,20 @@ static nl_status panel16_setup()
     return NL_OK;
 }
 
-// Lines (rows, columns) per streaming CTA, one CTA per SM: 64 while all fit on
-// the GPU at once, else 128 (a launch of several waves keeps going: a CTA that
-// starts after the diagonal block is done finds every word published).
+// Lines (rows, columns) per streaming CTA, one CTA per SM: 64 while they take
+// at most half of the SMs (the rest is for the look-ahead's update and for other
+// streams' solves), then 96 while all fit on the GPU at once, else 128 (a
+// launch of several waves keeps going: a CTA that starts after the diagonal
+// block is done finds every word published).  Few lines make the tail after the
+// last published block short, few CTAs leave SMs to the work beside it.  Measured
+// with 64 as long as all fit, with 96 (128) from half of the SMs on: a solve at
+// N = 4096 9.60, 9.44 (9.96) ms, five at once 24.0, 22.6 (22.5) ms, one
+// factorisation at N = 8192 3.04, 2.97 ms; 96 at every size: 9.58, 22.5, 2.97 ms.
 static int panel16_rows_per_cta(int rest, int pref = 0)
 {
     if (pref == kPnlRows) return kPnlRows;
-    return 1 + 2 * (int)cdiv(rest, 64) <= num_sms() ? 64 : 128;
+    if (1 + 2 * (int)cdiv(rest, 64) <= num_sms() / 2) return 64;
+    return 1 + 2 * (int)cdiv(rest, 96) <= num_sms() ? 96 : 128;
 }
 
 static std::atomic<unsigned> g_panel_epoch{0};
