@@ -383,8 +383,10 @@ struct nl_solver {
 static int lu_nb_alloc(const nl_config& d) { return d.lu_nb == -1 ? 512 : (d.lu_nb > 0 ? d.lu_nb : 128); }
 
 // Whether F is evaluated through the FFT convolution (nl_config.fft_f).  The
-// automatic choice takes it from N = 4096, where its four launches (about
-// 45 us) beat the direct sum (61 us at N = 4096, 2.1 ms at N = 32768, GB300).
+// automatic choice takes it from N = 4096, where its four launches (31 us, 48
+// at N = 32768) beat the direct sum (52 us, 2.1 ms at N = 32768, GB300).  They
+// are level at N = 3000; in between the direct sum's smaller rounding errors
+// are worth its up to 20 us of a step.
 constexpr int kFftAutoMinN = 4096;
 static bool uses_fft(int n, const nl_config& d) { return d.fft_f == 1 || (d.fft_f == 0 && n >= kFftAutoMinN); }
 
