@@ -663,65 +663,110 @@ void trsv_work_carve(void* base, int N, bool fp64, TrsvWork* w)
     w->scan = (int*)p;
 }
 
-// Diagonal-block inverses for block size TB, one thread per column, both
-// right-looking: once X's row t of the column is final, it is applied to every
-// later row, so the loop over rows has no dependence chain.  L (unit lower):
-// entry i of column c is -sum_{t=c}^{i-1} l_it x_t with the terms added in
-// increasing t, x_c = 1.  U: x_t = s_t / u_tt with s_i = [i == c] -
-// sum_{t>i} u_it x_t, the terms added in decreasing t.  Entries outside the
-// block (a ragged last block) are zero.
-// x[i] <- fma(a[i], y, x[i]) for rows i in [i0, i1) of one column (stride TB + 1);
-// rows in groups of four so the shared-memory loads run ahead of the stores.
-// fma(a, -y, x) is the same operation as fma(-a, y, x).
-template <typename T, int TB>
-__device__ __forceinline__ void axpy_col(const T* __restrict__ a, T* __restrict__ x, int i0, int i1, T y)
+// Diagonal-block inverses for block size TB, right-looking: once X's row t of
+// a column is final, it is applied to every later row, so the rows have no
+// dependence chain among them.  L (unit lower): entry i of column c is
+// -sum_{t=c}^{i-1} l_it x_t with the terms added in increasing t, x_c = 1.  U:
+// x_t = s_t / u_tt with s_i = [i == c] - sum_{t>i} u_it x_t, the terms added in
+// decreasing t.  Entries outside the block (a ragged last block) are zero.
+//
+// A CTA takes one triangle of one block and kInvC columns, eight threads per
+// column: thread (c, g) keeps the rows i = g mod 8 in registers, and the owner
+// of row t hands x_t to the others through shared memory, one barrier per step.
+// Bound in double precision: an instruction occupies its warp for about 65
+// cycles until four warps keep the SM's few units busy (then 19 each), so the
+// work is spread over all SMs, four warps each.  One thread per column and both
+// triangles in one CTA of two warps took 162 us at N = 1001; this takes 38 (41 at N = 2048).
+constexpr int kInvC = 16, kInvG = 8;
+
+// s / u for u's reciprocal r (correctly rounded; 0: outside the range where this
+// is safe): the quotient corrected once by its exact remainder, which rounds as
+// the division does (P. Markstein, IBM J. Res. Dev. 34, 1990), with three
+// dependent instructions on the chain instead of a division's.
+template <typename T>
+__device__ __forceinline__ T inv_div(T s, T u, T r)
 {
-    constexpr int S = TB + 1;
-    int i = i0;
-    for (; i + 4 <= i1; i += 4) {
-        const T a0 = a[i * S], a1 = a[(i + 1) * S], a2 = a[(i + 2) * S], a3 = a[(i + 3) * S];
-        const T x0 = x[i * S], x1 = x[(i + 1) * S], x2 = x[(i + 2) * S], x3 = x[(i + 3) * S];
-        x[i * S] = fma(a0, y, x0);
-        x[(i + 1) * S] = fma(a1, y, x1);
-        x[(i + 2) * S] = fma(a2, y, x2);
-        x[(i + 3) * S] = fma(a3, y, x3);
+    if constexpr (std::is_same<T, double>::value) {
+        if (r != 0.0) {
+            const double q = __dmul_rn(s, r);
+            return __fma_rn(__fma_rn(-q, u, s), r, q);
+        }
     }
-    for (; i < i1; ++i) x[i * S] = fma(a[i * S], y, x[i * S]);
+    return s / u;
 }
 
 template <typename S, typename T, int TB>
-__global__ void __launch_bounds__(TB) k_invdiag_t(int N, const S* __restrict__ LU, int64_t ld, T* __restrict__ dinv,
-                                                  int nblk)
+__global__ void __launch_bounds__(kInvC * kInvG) k_invdiag_t(int N, const S* __restrict__ LU, int64_t ld,
+                                                             T* __restrict__ dinv, int nblk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* A = reinterpret_cast<T*>(smem_raw);  // TB x (TB+1)
-    T* X = A + TB * (TB + 1);
-    const int b = blockIdx.x, r0 = b * TB, nb_ = min(TB, N - r0);
-    const int col = threadIdx.x;
-    T* x = X + col;  // this thread's column: x[i * (TB + 1)]
-    for (int i = 0; i < TB; ++i)
-        A[i * (TB + 1) + col] = (i < nb_ && col < nb_) ? (T)ld_elem(LU + (int64_t)(r0 + i) * ld + r0 + col) : T(0);
-    for (int i = 0; i < TB; ++i) x[i * (TB + 1)] = T(0);
+    T* At = reinterpret_cast<T*>(smem_raw);  // At[t * (TB + 1) + i]: entry (i, t)
+    __shared__ T xs[2][kInvC], rd[TB];
+    constexpr int R = TB / kInvG, kGroups = TB / kInvC, W = TB + 1;
+    const int b = blockIdx.x / (2 * kGroups), tri = (blockIdx.x / kGroups) & 1, c0 = (blockIdx.x % kGroups) * kInvC;
+    const int r0 = b * TB, nb_ = min(TB, N - r0), tid = threadIdx.x;
+    const int c = tid % kInvC, g = tid / kInvC, col = c0 + c;
+    for (int e = tid; e < TB * TB; e += kInvC * kInvG) {
+        const int i = e / TB, j = e % TB;
+        At[j * W + i] = (i < nb_ && j < nb_) ? (T)ld_elem(LU + (int64_t)(r0 + i) * ld + r0 + j) : T(0);
+    }
     __syncthreads();
-    // L^{-1}
-    for (int t = 0; t < nb_; ++t) {
-        if (t < col || col >= nb_) continue;
-        const T xt = (t == col) ? T(1) : -x[t * (TB + 1)];
-        x[t * (TB + 1)] = xt;
-        axpy_col<T, TB>(A + t, x, t + 1, nb_, xt);
+    T acc[R];  // rows g + 8 r
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = T(0);
+    if (tri == 0) {
+#pragma unroll
+        for (int tb = 0; tb < R; ++tb)
+            for (int tg = (8 * tb < c0 ? 8 : 0); tg < 8; ++tg) {  // (c0: a multiple of eight)
+                const int t = 8 * tb + tg;
+                if (t >= nb_) break;
+                if (g == tg) {
+                    if (t >= col) acc[tb] = t == col ? T(1) : -acc[tb];
+                    xs[t & 1][c] = acc[tb];
+                }
+                __syncthreads();
+                const T xt = xs[t & 1][c];
+                if (t >= col) {
+                    const T* a = At + t * W + g;
+                    if (g > tg) acc[tb] = fma(a[8 * tb], xt, acc[tb]);
+#pragma unroll
+                    for (int r = tb + 1; r < R; ++r) acc[r] = fma(a[8 * r], xt, acc[r]);
+                }
+            }
+    } else {
+        if (tid < TB) {
+            const T u = At[tid * W + tid];
+            // (r is normal, and neither q nor the remainder leaves the normal range for any s worth the name)
+            rd[tid] = fabs(u) >= T(1e-30) && fabs(u) <= T(1e30) ? T(1) / u : T(0);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = g + 8 * r == col && col < nb_ ? T(1) : T(0);
+        __syncthreads();
+#pragma unroll
+        for (int tb = R - 1; tb >= 0; --tb)
+            for (int tg = 7; tg >= 0; --tg) {
+                const int t = 8 * tb + tg;
+                if (t >= nb_ || t >= c0 + kInvC) continue;
+                if (g == tg) {
+                    if (t <= col && col < nb_) acc[tb] = inv_div(acc[tb], At[t * W + t], rd[t]);
+                    xs[t & 1][c] = acc[tb];
+                }
+                __syncthreads();
+                const T xt = -xs[t & 1][c];
+                if (t <= col && col < nb_) {
+                    const T* a = At + t * W + g;
+                    if (g < tg) acc[tb] = fma(a[8 * tb], xt, acc[tb]);
+#pragma unroll
+                    for (int r = 0; r < tb; ++r) acc[r] = fma(a[8 * r], xt, acc[r]);
+                }
+            }
     }
-    T* Linv = dinv + (int64_t)b * TB * TB;
-    for (int i = 0; i < TB; ++i) Linv[i * TB + col] = x[i * (TB + 1)];
-    // U^{-1}
-    for (int i = 0; i < TB; ++i) x[i * (TB + 1)] = (i == col && col < nb_) ? T(1) : T(0);
-    for (int t = nb_ - 1; t >= 0; --t) {
-        if (t > col || col >= nb_) continue;
-        const T xt = x[t * (TB + 1)] / A[t * (TB + 1) + t];
-        x[t * (TB + 1)] = xt;
-        axpy_col<T, TB>(A + t, x, 0, t, -xt);
+    T* out = dinv + (int64_t)(tri * nblk + b) * TB * TB;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = g + 8 * r;
+        out[i * TB + col] = i < nb_ && col < nb_ ? acc[r] : T(0);
     }
-    T* Uinv = dinv + (int64_t)(nblk + b) * TB * TB;
-    for (int i = 0; i < TB; ++i) Uinv[i * TB + col] = x[i * (TB + 1)];
 }
 
 // The binary16 factors' 128 x 128 diagonal-block inverses, the recurrences of
@@ -863,7 +908,8 @@ static nl_status prepare_impl(int N, const S* LU, int64_t ld, const int* ipiv, c
     if constexpr (std::is_same<S, __half>::value && !fp64)
         k_invdiag16<<<2 * nblk, kInvThreads, kInvSmem, st>>>(N, LU, ld, (float*)w.dinv, nblk);
     else
-        k_invdiag_t<S, T, TB><<<nblk, TB, (size_t)2 * TB * (TB + 1) * sizeof(T), st>>>(N, LU, ld, (T*)w.dinv, nblk);
+        k_invdiag_t<S, T, TB><<<2 * nblk * (TB / kInvC), kInvC * kInvG, (size_t)TB * (TB + 1) * sizeof(T), st>>>(
+            N, LU, ld, (T*)w.dinv, nblk);
     prof_end("k_invdiag", st);
     NL_CUDA_OK(cudaGetLastError());
     if (launches) *launches += 2;
