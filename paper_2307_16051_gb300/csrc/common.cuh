@@ -122,6 +122,26 @@ __device__ __forceinline__ float div_round_h(float a, float u)
     return -round_h(div_neg(a, u, rcp_neg_abs(u), fabsf(u)));
 }
 
+// s / u by u's reciprocal r = rcp_in_range(u), for chains of quotients by divisors
+// known beforehand: the quotient corrected once by its exact remainder, which
+// rounds as the division does (P. Markstein, IBM J. Res. Dev. 34, 1990), with
+// three dependent instructions on the chain instead of a division's (and none
+// of its slow paths: a zero numerator takes one).  r = 0, and the division as it
+// stands: u out of the range in which neither r nor the remainder can leave the
+// normal numbers for any quotient that matters, or not finite.
+__device__ __forceinline__ double rcp_in_range(double u)
+{
+    return fabs(u) >= 1e-30 && fabs(u) <= 1e30 ? 1.0 / u : 0.0;
+}
+__device__ __forceinline__ float rcp_in_range(float) { return 0.0f; }
+__device__ __forceinline__ double div_by(double s, double u, double r)
+{
+    if (r == 0.0) return s / u;
+    const double q = __dmul_rn(s, r);
+    return __fma_rn(__fma_rn(-q, u, s), r, q);
+}
+__device__ __forceinline__ float div_by(float s, float u, float) { return s / u; }
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
 {

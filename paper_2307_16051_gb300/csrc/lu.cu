@@ -594,10 +594,13 @@ __global__ void __launch_bounds__(kDiagThreads, 1) k_diag_lu(S* __restrict__ A, 
 // however few lanes are on).  As in the diagonal block, warp 0 takes entry t + 1
 // of every line (update, check, division) while the other warps apply entry t to
 // the later ones: one barrier per step, every entry's terms in increasing t.
-// U11 / L11^T as staged by k_diag_lu.  Measured, w = 64: N = 2048 43 us, N = 1001 70 us a
-// panel on average (groups of eight lanes per row, four of 32 lanes dividing,
-// took 85 at N = 1001; one thread per row with its entries in registers, a
-// division's latency per step and 37 KB of straight-line code, 137).
+// U11 / L11^T as staged by k_diag_lu.  The quotients are products with the
+// pivots' reciprocals, made once and corrected (div_by): three dependent
+// instructions of a step instead of a division's dozen.  Measured, w = 64: 39 us a
+// panel at N = 1001 and 2048 (with divisions 70 and 43: the empty lines of a
+// ragged last CTA divide zeros, which is the division's slow path; groups of
+// eight lanes per row, four of 32 lanes dividing, took 85 at N = 1001; one thread
+// per row with its entries in registers, 137).
 constexpr int kOffThreads = 256;
 constexpr int kOffLines = 32;
 
@@ -608,6 +611,7 @@ __device__ __forceinline__ void offdiag_body(S* __restrict__ A, int64_t lda, int
     if (flag && *(volatile int*)flag) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int XS = kOffLines + 1;
+    __shared__ T rd[128];  // row role: rcp_in_range(u_tt)
     const int wp = (w + 31) & ~31;
     T* D = reinterpret_cast<T*>(smem_raw);  // wp x wp: U11 (row role) or L11^T (column role), identity-padded
     T* X = D + wp * wp;                     // X[t * XS + line]
@@ -633,6 +637,8 @@ __device__ __forceinline__ void offdiag_body(S* __restrict__ A, int64_t lda, int
         }
     }
     __syncthreads();
+    if (row_role && tid < w) rd[tid] = rcp_in_range(D[tid * wp + tid]);
+    __syncthreads();
     bool bad = false;
     for (int t = -1; t < w - 1; ++t) {
         const T* Dt = D + t * wp;
@@ -644,7 +650,7 @@ __device__ __forceinline__ void offdiag_body(S* __restrict__ A, int64_t lda, int
             if (row_role) {
                 const T u = D[c * wp + c];
                 if (lane < n && (!(absT(x) <= absT(u)) || !(u != T(0)))) bad = true;
-                x = x / u;
+                x = div_by(x, u, rd[c]);
             }
             X[c * XS + lane] = x;
         } else if (t >= 0) {

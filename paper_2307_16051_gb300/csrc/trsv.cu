@@ -679,22 +679,6 @@ void trsv_work_carve(void* base, int N, bool fp64, TrsvWork* w)
 // triangles in one CTA of two warps took 162 us at N = 1001; this takes 38 (41 at N = 2048).
 constexpr int kInvC = 16, kInvG = 8;
 
-// s / u for u's reciprocal r (correctly rounded; 0: outside the range where this
-// is safe): the quotient corrected once by its exact remainder, which rounds as
-// the division does (P. Markstein, IBM J. Res. Dev. 34, 1990), with three
-// dependent instructions on the chain instead of a division's.
-template <typename T>
-__device__ __forceinline__ T inv_div(T s, T u, T r)
-{
-    if constexpr (std::is_same<T, double>::value) {
-        if (r != 0.0) {
-            const double q = __dmul_rn(s, r);
-            return __fma_rn(__fma_rn(-q, u, s), r, q);
-        }
-    }
-    return s / u;
-}
-
 template <typename S, typename T, int TB>
 __global__ void __launch_bounds__(kInvC * kInvG) k_invdiag_t(int N, const S* __restrict__ LU, int64_t ld,
                                                              T* __restrict__ dinv, int nblk)
@@ -735,9 +719,7 @@ __global__ void __launch_bounds__(kInvC * kInvG) k_invdiag_t(int N, const S* __r
             }
     } else {
         if (tid < TB) {
-            const T u = At[tid * W + tid];
-            // (r is normal, and neither q nor the remainder leaves the normal range for any s worth the name)
-            rd[tid] = fabs(u) >= T(1e-30) && fabs(u) <= T(1e30) ? T(1) / u : T(0);
+            rd[tid] = rcp_in_range(At[tid * W + tid]);
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] = g + 8 * r == col && col < nb_ ? T(1) : T(0);
@@ -748,7 +730,7 @@ __global__ void __launch_bounds__(kInvC * kInvG) k_invdiag_t(int N, const S* __r
                 const int t = 8 * tb + tg;
                 if (t >= nb_ || t >= c0 + kInvC) continue;
                 if (g == tg) {
-                    if (t <= col && col < nb_) acc[tb] = inv_div(acc[tb], At[t * W + t], rd[t]);
+                    if (t <= col && col < nb_) acc[tb] = div_by(acc[tb], At[t * W + t], rd[t]);
                     xs[t & 1][c] = acc[tb];
                 }
                 __syncthreads();
