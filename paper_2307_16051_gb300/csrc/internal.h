@@ -51,8 +51,8 @@ struct LuWork {
     int* flag = nullptr;      // device int (info + 1): set when the no-interchange fast path failed
     void* stage = nullptr;    // diagonal-block factors staged for the off-diagonal solves (<= 256 KB)
     unsigned long long* pub = nullptr;  // 128 x 128 {epoch, value} words: columns published by k_panel16
-    int stream = 0;           // binary16 fast path: 0 = one streaming launch per panel when it fits (128 rows per
-                              // CTA when possible), 256 = the same with 256 rows per CTA, -1 = two launches
+    int stream = 0;           // binary16 fast path: 0 = one streaming launch per panel (64, 96 or 128 rows per
+                              // CTA), 256 = the same with 256 rows per CTA, -1 = two launches
     float* p32 = nullptr;     // two-level LU (outer block > 128): single-precision shadow of the matrix, N x ldp32,
                               // of which the current outer block's row and column strips are used
     int64_t ldp32 = 0;
