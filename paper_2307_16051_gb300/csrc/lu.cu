@@ -560,6 +560,8 @@ __device__ __forceinline__ void diag_lu_body(S* __restrict__ A, int64_t lda, int
         }
         __syncthreads();
     }
+    // every pivot (the last one has no row below it that would have checked it)
+    if (tid < w && !(absT(W[tid * ldw + tid]) > T(0))) bad = true;
     if (__syncthreads_or(bad)) {
         if (tid == 0) atomicOr(flag, 1);
         return;
