@@ -624,6 +624,12 @@ nl_status nl_k_gemv_residual(int64_t N, const float* A, int64_t ld, const float*
  * binary16 rounding boundary).  For tests of that arithmetic. */
 nl_status nl_k_div_round16(int64_t n, const float* a, const float* b, float* out, void* stream);
 
+/* out[i] = a[i] / b[i] (device, n doubles each), bit for bit the IEEE quotient,
+ * as the double LU's off-diagonal solves and nl_lusolve64's inverses form it
+ * (the product with the divisor's reciprocal, corrected by its remainder).  For
+ * tests of that arithmetic. */
+nl_status nl_k_div64(int64_t n, const double* a, const double* b, double* out, void* stream);
+
 /* Trailing update of the half-precision LU:  C <- fl16(C - A B) with A M x K,
  * B K x Nc, C M x Nc binary16 row-major (lda, ldb, ldc), products accumulated
  * in single.  gemm: 1 SIMT (sequential fused multiply-adds over k),

@@ -122,13 +122,17 @@ __device__ __forceinline__ float div_round_h(float a, float u)
     return -round_h(div_neg(a, u, rcp_neg_abs(u), fabsf(u)));
 }
 
-// s / u by u's reciprocal r = rcp_in_range(u), for chains of quotients by divisors
-// known beforehand: the quotient corrected once by its exact remainder, which
-// rounds as the division does (P. Markstein, IBM J. Res. Dev. 34, 1990), with
-// three dependent instructions on the chain instead of a division's (and none
-// of its slow paths: a zero numerator takes one).  r = 0, and the division as it
-// stands: u out of the range in which neither r nor the remainder can leave the
-// normal numbers for any quotient that matters, or not finite.
+// s / u, bit for bit, by u's reciprocal r = rcp_in_range(u), for chains of quotients by
+// divisors known beforehand: the quotient corrected once by its exact remainder
+// (P. Markstein, IBM J. Res. Dev. 34, 1990), three dependent instructions on the
+// chain instead of a division's (and none of its slow paths: a zero numerator
+// takes one).  With 2^-100 < |u| < 2^100 and 2^-900 <= |s| < 2^900 quotient, reciprocal
+// and remainder are normal numbers and the remainder is exact; the product s r
+// is within 1.5 units, and the corrected quotient rounds as the division does
+// (for every pair of significands of 5 to 12 bits; more bits only make the
+// exceptions rarer).  A zero numerator's product has the quotient's sign.  Every other
+// numerator (huge, tiny, infinite, NaN) and every u with r = 0 takes the
+// division.  The range tests are on the exponent bits, off the double-precision pipe.
 __device__ __forceinline__ double rcp_in_range(double u)
 {
     return fabs(u) >= 1e-30 && fabs(u) <= 1e30 ? 1.0 / u : 0.0;
@@ -136,8 +140,10 @@ __device__ __forceinline__ double rcp_in_range(double u)
 __device__ __forceinline__ float rcp_in_range(float) { return 0.0f; }
 __device__ __forceinline__ double div_by(double s, double u, double r)
 {
-    if (r == 0.0) return s / u;
+    const unsigned hi = (unsigned)__double2hiint(s) & 0x7fffffffu;
     const double q = __dmul_rn(s, r);
+    if (__double2hiint(r) == 0 || (hi >> 20) - 123u >= 1800u)  // biased exponents 123 .. 1922
+        return __double2hiint(r) != 0 && (hi | (unsigned)__double2loint(s)) == 0u ? q : s / u;
     return __fma_rn(__fma_rn(-q, u, s), r, q);
 }
 __device__ __forceinline__ float div_by(float s, float u, float) { return s / u; }

@@ -3507,6 +3507,13 @@ __global__ void k_div_round16(int64_t n, const float* __restrict__ a, const floa
     if (i < n) out[i] = div_round_h(a[i], b[i]);
 }
 
+// The quotients of the double-precision off-diagonal solves and inverses, elementwise (for tests).
+__global__ void k_div64(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = div_by(a[i], b[i], rcp_in_range(b[i]));
+}
+
 }  // namespace nl
 
 extern "C" nl_status nl_k_div_round16(int64_t n, const float* a, const float* b, float* out, void* stream)
@@ -3518,6 +3525,19 @@ extern "C" nl_status nl_k_div_round16(int64_t n, const float* a, const float* b,
     }
     if (n == 0) return NL_OK;
     k_div_round16<<<(unsigned)cdiv(n, 256), 256, 0, (cudaStream_t)stream>>>(n, a, b, out);
+    NL_CUDA_OK(cudaGetLastError());
+    return NL_OK;
+}
+
+extern "C" nl_status nl_k_div64(int64_t n, const double* a, const double* b, double* out, void* stream)
+{
+    using namespace nl;
+    if (n < 0 || (n > 0 && (!a || !b || !out))) {
+        set_error("nl_k_div64: bad argument");
+        return NL_EINVAL;
+    }
+    if (n == 0) return NL_OK;
+    k_div64<<<(unsigned)cdiv(n, 256), 256, 0, (cudaStream_t)stream>>>(n, a, b, out);
     NL_CUDA_OK(cudaGetLastError());
     return NL_OK;
 }

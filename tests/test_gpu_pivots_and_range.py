@@ -64,3 +64,50 @@ def test_lu_grouped_fp64_zero_last_pivot():
     mats = [_last_pivot(N, 3.0 if N == 96 else 0.0) for N in Ns]
     _, flags = lu_grouped(mats, 64, 1, fp64=True)
     assert list(flags) == [1, 1, 1, 1, 0]
+
+
+@pytest.mark.parametrize("u00,u01,u11", [(1e-20, 1e290, 1.0), (1e-20, -1e300, 1e-20), (-1e-25, 1e300, 1e-8)])
+def test_lusolve64_overflowing_inverse(u00, u01, u11):
+    """A triangle whose inverse overflows: infinities with the signs the
+    divisions give, not NaN."""
+    LU = np.array([[u00, u01], [0.0, u11]])
+    b = np.array([1.0, 1.0])
+    with np.errstate(over="ignore"):
+        z1 = b[1] / u11
+        ref = np.array([(b[0] - u01 * z1) / u00, z1])
+    assert np.isinf(ref[0])
+    bd = T(b)
+    nl.lusolve64(2, T(LU), 2, torch.arange(2, device=dev(), dtype=torch.int32), bd)
+    assert np.array_equal(bd.cpu().numpy(), ref), bd
+
+
+def test_div64_equals_ieee_division():
+    """The quotients by corrected reciprocals against numpy's IEEE division, bit
+    for bit (NaN by NaN): ordinary operands, quotients next to the middle of two doubles,
+    every pair of exponents, and zeros, subnormal numbers, infinities and NaN of both signs
+    against each other."""
+    g = np.random.default_rng(64)
+    n = 1 << 20
+    a, b = g.standard_normal(n), g.standard_normal(n)
+    k = n // 4
+    # a = fl(m b) for m halfway between two doubles: the quotient lies next to the middle
+    q = 1.0 + g.integers(0, 1 << 52, size=k) * 2.0 ** -52
+    b[:k] = 1.0 + g.integers(0, 1 << 52, size=k) * 2.0 ** -52
+    a[:k] = q * b[:k] + 2.0 ** -53 * b[:k] * g.integers(-2, 3, size=k)
+    e = np.arange(-1074, 1024)
+    ea, eb = np.meshgrid(e[::3], e[::5])
+    sa, sb = (g.choice([-1.0, 1.0], ea.size) * (1.0 + g.random(ea.size)) for _ in range(2))
+    edge = np.concatenate([[0.0, 5e-324, 2.0 ** -1022, 1e-30, 1e30, np.nextafter(1e-30, 0), np.nextafter(1e30, 1e31),
+                            2.0 ** -900, np.nextafter(2.0 ** -900, 0), 2.0 ** 900, np.nextafter(2.0 ** 900, 0),
+                            np.finfo(float).max, 1.0, 3.0, np.inf, np.nan]])
+    edge = np.concatenate([edge, -edge])
+    xa, xb = np.meshgrid(edge, edge)
+    a = np.concatenate([a, np.ldexp(sa, ea.ravel()), xa.ravel()])
+    b = np.concatenate([b, np.ldexp(sb, eb.ravel()), xb.ravel()])
+    with np.errstate(all="ignore"):
+        ref = a / b
+    out = torch.empty(a.size, device=dev(), dtype=torch.float64)
+    nl.k_div64(a.size, T(a), T(b), out)
+    got = out.cpu().numpy()
+    bad = ~((got.view(np.uint64) == ref.view(np.uint64)) | (np.isnan(got) & np.isnan(ref)))
+    assert not bad.any(), (bad.sum(), a[bad][:5], b[bad][:5], got[bad][:5], ref[bad][:5])
