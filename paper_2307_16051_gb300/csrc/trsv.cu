@@ -550,6 +550,9 @@ __device__ __forceinline__ void cl_triangle(const ClState& S, const float* __res
                 atomicOr(S.err, (unsigned)ERR_TIMEOUT_TRSV);
             }
         }
+        // one answer per warp (apply's shuffles name all lanes): lanes may see the bound or the abort word differently
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, ok);
         const float* z = yv + (size_t)b * kClPad;
         int j = (s < rank) ? 0 : (s - rank) / C + 1;  // this CTA's blocks solved after step s
         if (j < nown && rank + j * C == s + 1) {

@@ -138,3 +138,27 @@ def test_persistent_grouped_lu_wait_runs_out(gemm):
     assert not flags.any() and not rflags.any()
     for a, b in zip(out, ref):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,cluster", [(256, 0), (1000, 8), (3072, 0), (4096, 4), (4096, 16)])
+@pytest.mark.parametrize("limit", [-1, 1, 2])
+def test_cluster_solve_waits_run_out_in_part(N, cluster, limit):
+    """The one-launch cluster solve (both triangles) when its waits run out: all of
+    them (-1), or those whose block has not arrived within one or two polls, so
+    that some warps and CTAs give up and others do not.  The launch ends, the
+    solve returns NL_ETIMEOUT or, if no wait ran out, the solution, and a
+    handle with the default limit converges on the same context."""
+    c = 0.9
+    with nl.Solver(N, c, trsv_cluster=cluster) as s:
+        xr, st = s.solve(tol=1e-10, mode="IR16")
+        assert st == nl.NL_OK
+    for _ in range(3):
+        with nl.Solver(N, c, trsv_cluster=cluster, wait_limit=limit) as s:
+            st, x = _solve_raw(s, "IR16")
+            assert st == nl.NL_ETIMEOUT or (limit > 0 and st == nl.NL_OK and np.array_equal(x, xr)), nl.STATUS_NAMES[st]
+            if st == nl.NL_ETIMEOUT:
+                assert "gave up" in nl.last_error()
+        torch.cuda.synchronize()  # the device answers
+    with nl.Solver(N, c, trsv_cluster=cluster) as s:
+        x, st = s.solve(tol=1e-10, mode="IR16")
+        assert st == nl.NL_OK and np.array_equal(x, xr)
