@@ -83,7 +83,11 @@ cudaError_t dev_malloc(void** p, size_t bytes)
 
 cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st)
 {
-    cudaMemPool_t pool = ws_pool(true);
+    // In a capture the memory belongs to the graph whatever the pool, and making the pool is
+    // not allowed there.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? ws_pool(true) : nullptr;
     if (!pool) return cudaMallocAsync(p, bytes, st);
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
