@@ -10,6 +10,8 @@
 // half-precision factors; success at ||b - J32 u|| <= eta ||b||, failure
 // when the residual norm increases (the best iterate is kept), Section 3.1.
 // Control runs on the host; each decision reads one device scalar back.
+#include <cuda.h>
+
 #include <atomic>
 #include <chrono>
 #include <type_traits>
@@ -31,32 +33,63 @@ static thread_local char g_err[512] = "";
 // of the library's handles fail as if the device were out of memory.
 static std::atomic<int> g_fail_allocs{0};
 
-// The current device's workspace pool (created on first use; null where pools are not supported).
-constexpr int kWsMaxDevices = 64;
+// The identity of the calling thread's current context, unique for the life of the
+// process: a device reset ends a context with everything made in it, so whatever is
+// kept between calls is kept by this.  0: unknown (then nothing is kept).
+static unsigned long long context_id()
+{
+    using Fn = CUresult(CUDAAPI*)(CUcontext, unsigned long long*);
+    static const Fn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Fn>(f);
+    }();
+    unsigned long long id = 0;
+    if (!get) return 0;
+    if (get(nullptr, &id) == CUDA_SUCCESS) return id;
+    int dev = 0;  // (a thread without a context yet: its device's, made current)
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return 0;
+    return get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// The current context's workspace pool (created on first use; null where pools are not
+// supported, and for a context beyond the kWsMaxContexts-th of the process).
+constexpr int kWsMaxContexts = 64;
 static std::mutex g_ws_mu;
-static cudaMemPool_t g_ws_pool[kWsMaxDevices] = {};
+static struct {
+    unsigned long long ctx;
+    cudaMemPool_t pool;
+} g_ws_pool[kWsMaxContexts];
+static int g_ws_pools = 0;
 static cudaMemPool_t ws_pool(bool create)
 {
+    const unsigned long long ctx = context_id();
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kWsMaxDevices) return nullptr;
+    if (!ctx || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lock(g_ws_mu);
-    if (!g_ws_pool[dev] && create) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t pool = nullptr;
-        uint64_t keep = kWsKeep;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            if (pool) cudaMemPoolDestroy(pool);
-            return nullptr;
-        }
-        g_ws_pool[dev] = pool;
+    for (int k = 0; k < g_ws_pools; ++k)
+        if (g_ws_pool[k].ctx == ctx) return g_ws_pool[k].pool;
+    if (!create || g_ws_pools == kWsMaxContexts) return nullptr;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kWsKeep;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        if (pool) cudaMemPoolDestroy(pool);
+        return nullptr;
     }
-    return g_ws_pool[dev];
+    g_ws_pool[g_ws_pools++] = {ctx, pool};
+    return pool;
 }
 static bool ws_trim()
 {
@@ -1473,43 +1506,45 @@ nl_status nl_k_gemm16_update(int64_t M, int64_t Nc, int64_t K, const void* A, in
                          (cudaStream_t)stream);
 }
 
-// 64 bytes of pinned host memory for a call's scalars, from a small free list
-// (allocating and freeing pinned memory synchronises and takes longer than a small solve).
+// 64 bytes of pinned host memory for a call's scalars, kept between calls (allocating and
+// freeing pinned memory synchronises and takes longer than a small solve): at most
+// kPinnedKept blocks in the process, each for calls in the context it was made in.
 namespace {
 struct PinnedWords {
+    static constexpr int kPinnedKept = 16;
+    struct Kept {
+        double* p;
+        unsigned long long ctx;
+    };
+    inline static Kept kept[kPinnedKept];
+    inline static std::mutex mu;
+    const unsigned long long ctx = context_id();
     double* p = nullptr;
     PinnedWords()
     {
-        {
-            std::lock_guard<std::mutex> lock(mu());
-            if (!list().empty()) {
-                p = list().back();
-                list().pop_back();
-            }
+        if (ctx) {
+            std::lock_guard<std::mutex> lock(mu);
+            for (Kept& k : kept)
+                if (k.p && k.ctx == ctx) {
+                    p = k.p;
+                    k.p = nullptr;
+                    break;
+                }
         }
         if (!p && cudaMallocHost((void**)&p, 64) != cudaSuccess) p = nullptr;
     }
     ~PinnedWords()
     {
         if (!p) return;
-        {
-            std::lock_guard<std::mutex> lock(mu());
-            if (list().size() < 16) {
-                list().push_back(p);
-                return;
-            }
+        if (ctx) {
+            std::lock_guard<std::mutex> lock(mu);
+            for (Kept& k : kept)
+                if (!k.p) {
+                    k = {p, ctx};
+                    return;
+                }
         }
         cudaFreeHost(p);
-    }
-    static std::mutex& mu()
-    {
-        static std::mutex m;
-        return m;
-    }
-    static std::vector<double*>& list()
-    {
-        static std::vector<double*>* l = new std::vector<double*>();  // (never destroyed: calls may outlive statics)
-        return *l;
     }
 };
 }  // namespace
