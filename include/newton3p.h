@@ -260,6 +260,13 @@ const char* nl_version(void);
  * for count < 0. */
 nl_status nl_debug_fail_allocs(int count);
 
+/* Test hook for a full device: after `skip` attempts, the next `count` attempts
+ * of the library to allocate device memory, for anything, find the device full.
+ * Before a call reports that, it gives back the workspace memory that the library
+ * keeps and tries once more, so count = 1 goes unnoticed once a workspace has
+ * been kept.  (0, 0) turns it off.  NL_EINVAL for negative arguments. */
+nl_status nl_debug_device_full(int skip, int count);
+
 /* ----------------------------------------------------------------------- */
 /* Batched solves: many independent instances of eq. (3.2), each with its   */
 /* own N and c, advanced together on the device.                            */

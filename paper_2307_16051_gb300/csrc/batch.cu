@@ -1493,7 +1493,7 @@ nl_status nl_lu_grouped(int count, const int64_t* N, void* const* A, const int64
         bytes = cv.off + 256;
     }
     void* wk = nullptr;
-    NL_CUDA_OK(cudaMalloc(&wk, bytes));
+    NL_CUDA_OK(trim_malloc(&wk, bytes));
     Carver cv(wk);
     GInst* dg = cv.take<GInst>(count);
     int* flags = cv.take<int>(count);

@@ -36,7 +36,11 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int num_sms();
 
-// cudaMalloc for the handles' device pools; fails on purpose while the test
+// cudaMalloc that gives the workspaces kept by ws_malloc_async's pool back and
+// tries again before it reports that the device is full: every device allocation
+// of the library that is not from that pool.
+cudaError_t trim_malloc(void** p, size_t bytes);
+// The same for the handles' device pools; fails on purpose while the test
 // hook nl_debug_fail_allocs has allocations left to fail.
 cudaError_t dev_malloc(void** p, size_t bytes);
 
@@ -44,8 +48,8 @@ cudaError_t dev_malloc(void** p, size_t bytes);
 // cudaFreeAsync: from the library's own memory pool on the current device,
 // which keeps up to kWsKeep bytes of released memory across synchronisations
 // (the default pool returns all of it to the system at each one and maps it
-// again at the next call: 190 us of a call that synchronises).  dev_malloc gives
-// the kept memory back before it reports that the device is full.
+// again at the next call: 190 us of a call that synchronises).  trim_malloc gives
+// the kept memory back, and so does this when the device is full.
 constexpr size_t kWsKeep = (size_t)256 << 20;
 cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st);
 

@@ -609,7 +609,7 @@ bool tc_gemm_supported()
         return false;
     }
     g_encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-    if (cudaMalloc((void**)&g_tc_err, sizeof(unsigned)) != cudaSuccess) return false;
+    if (trim_malloc((void**)&g_tc_err, sizeof(unsigned)) != cudaSuccess) return false;
     cudaMemset(g_tc_err, 0, sizeof(unsigned));
     if (set_max_dynamic_smem((const void*)k_tc_gemm) != NL_OK) return false;
     if (set_max_dynamic_smem((const void*)k_tc_gemm_g) != NL_OK) return false;

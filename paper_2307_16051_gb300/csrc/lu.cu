@@ -3307,7 +3307,7 @@ static nl_status lu_grouped_plan_p(int count, const GInst* host_inst, int nb, in
     const size_t mb = maps.size() * sizeof(TmapBytes);
     plan->bytes = round_up(qb, 256) + round_up(cb, 256) + mb;
     void* p = nullptr;
-    NL_CUDA_OK(cudaMalloc(&p, plan->bytes));
+    NL_CUDA_OK(trim_malloc(&p, plan->bytes));
     plan->tasks = reinterpret_cast<GTask*>(p);  // the allocation's base (freed through it)
     plan->ptasks = reinterpret_cast<PTask*>(p);
     plan->ctl = reinterpret_cast<int*>((char*)p + round_up(qb, 256));
@@ -3394,7 +3394,7 @@ nl_status lu_grouped_plan(int count, const GInst* host_inst, int nb, int gemm, b
     const size_t tb = tasks.size() * sizeof(GTask), mb = maps.size() * sizeof(TmapBytes);
     plan->bytes = round_up(tb, 256) + mb + 256;
     void* p = nullptr;
-    NL_CUDA_OK(cudaMalloc(&p, plan->bytes));
+    NL_CUDA_OK(trim_malloc(&p, plan->bytes));
     plan->tasks = reinterpret_cast<GTask*>(p);
     plan->maps = mb ? reinterpret_cast<TmapBytes*>((char*)p + round_up(tb, 256)) : nullptr;
     if (tb) NL_CUDA_OK(cudaMemcpy(plan->tasks, tasks.data(), tb, cudaMemcpyHostToDevice));

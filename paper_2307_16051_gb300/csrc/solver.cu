@@ -97,21 +97,42 @@ static bool ws_trim()
     return pool && cudaMemPoolTrimTo(pool, 0) == cudaSuccess;
 }
 
-cudaError_t dev_malloc(void** p, size_t bytes)
+// Test hook (nl_debug_device_full): after g_full_skip attempts the next g_full_count find the device full.
+static std::atomic<int> g_full_skip{0}, g_full_count{0};
+static bool take_one(std::atomic<int>& left)
 {
-    int n = g_fail_allocs.load();
-    while (n > 0) {
-        if (g_fail_allocs.compare_exchange_weak(n, n - 1)) {
-            *p = nullptr;
-            return cudaErrorMemoryAllocation;
-        }
-    }
-    cudaError_t e = cudaMalloc(p, bytes);
+    int n = left.load();
+    while (n > 0)
+        if (left.compare_exchange_weak(n, n - 1)) return true;
+    return false;
+}
+template <typename Alloc>
+static cudaError_t malloc_or_trim(Alloc alloc)
+{
+    auto attempt = [&] {
+        return !take_one(g_full_skip) && take_one(g_full_count) ? cudaErrorMemoryAllocation : alloc();
+    };
+    cudaError_t e = attempt();
     if (e == cudaErrorMemoryAllocation && ws_trim()) {
         cudaGetLastError();
-        e = cudaMalloc(p, bytes);
+        e = attempt();
     }
     return e;
+}
+
+cudaError_t trim_malloc(void** p, size_t bytes)
+{
+    *p = nullptr;
+    return malloc_or_trim([&] { return cudaMalloc(p, bytes); });
+}
+
+cudaError_t dev_malloc(void** p, size_t bytes)
+{
+    if (take_one(g_fail_allocs)) {
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
+    return trim_malloc(p, bytes);
 }
 
 cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st)
@@ -122,7 +143,7 @@ cudaError_t ws_malloc_async(void** p, size_t bytes, cudaStream_t st)
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
     cudaMemPool_t pool = cap == cudaStreamCaptureStatusNone ? ws_pool(true) : nullptr;
     if (!pool) return cudaMallocAsync(p, bytes, st);
-    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+    return malloc_or_trim([&] { return cudaMallocFromPoolAsync(p, bytes, pool, st); });
 }
 
 void set_error(const char* fmt, ...)
@@ -588,6 +609,17 @@ nl_status nl_debug_fail_allocs(int count)
         return NL_EINVAL;
     }
     g_fail_allocs.store(count);
+    return NL_OK;
+}
+
+nl_status nl_debug_device_full(int skip, int count)
+{
+    if (skip < 0 || count < 0) {
+        set_error("nl_debug_device_full: skip < 0 or count < 0");
+        return NL_EINVAL;
+    }
+    g_full_skip.store(skip);
+    g_full_count.store(count);
     return NL_OK;
 }
 

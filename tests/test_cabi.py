@@ -147,3 +147,9 @@ def test_test_hooks_and_scaled_jacobian_validate_arguments():
     assert L.nl_k_jacobian_scaled(0, 0.5, 8, 8, 64, 8, 64, 8, None) == nl.NL_EINVAL
     c = nl.config()
     assert c.wait_limit == 0 and c.scale_fp16 == 0 and c.fft_f == 0
+
+
+def test_device_full_hook_rejects_negative_counts():
+    L = nl.lib()
+    assert L.nl_debug_device_full(-1, 0) == nl.NL_EINVAL and L.nl_debug_device_full(0, -1) == nl.NL_EINVAL
+    assert L.nl_debug_device_full(0, 0) == nl.NL_OK

@@ -162,3 +162,50 @@ def test_cluster_solve_waits_run_out_in_part(N, cluster, limit):
     with nl.Solver(N, c, trsv_cluster=cluster) as s:
         x, st = s.solve(tol=1e-10, mode="IR16")
         assert st == nl.NL_OK and np.array_equal(x, xr)
+
+
+@pytest.mark.parametrize("call", ["lu_grouped", "lu_grouped_persistent", "batch", "solver", "gemv"])
+def test_full_device_gives_kept_workspaces_back(call):
+    """An allocation that finds the device full is tried again after the library
+    has given its kept workspace memory back: each of a call's allocations in
+    turn fails once and the call succeeds; when the second attempt fails too the
+    call returns an error, and the next one succeeds."""
+    L, d, N, ld = nl.lib(), torch.device("cuda:0"), 300, 320
+    A32 = torch.eye(N, ld, device=d, dtype=torch.float32)
+    b, u, r = (torch.ones(ld, device=d, dtype=torch.float32) for _ in range(3))
+    fn = torch.zeros(1, device=d, dtype=torch.float64)
+    A = torch.zeros((N, ld), device=d, dtype=torch.float16)
+    ip = torch.empty(N, device=d, dtype=torch.int32)
+
+    def keep():  # a workspace, released and kept
+        nl.k_gemv_residual(N, A32, ld, b, u, r, fn)
+        torch.cuda.synchronize()
+
+    def run():
+        if call.startswith("lu_grouped"):
+            A[:, :N] = torch.eye(N, device=d, dtype=torch.float16)
+            flags = nl.lu_grouped([N], [A], [ld], [ip], nb=64, gemm=5 if "persistent" in call else 2)
+            assert not flags.any()
+        elif call == "batch":
+            with nl.Batch([64, N], [0.5, 0.9], lu_nb=64) as B:
+                assert B.solve(tol=1e-10)[1] == nl.NL_OK
+        elif call == "solver":
+            with nl.Solver(N, 0.9) as s:
+                assert s.solve(mode="FP64LU")[1] == nl.NL_OK
+        else:
+            nl.k_gemv_residual(N, A32, ld, b, u, r, fn)
+            torch.cuda.synchronize()
+
+    run()
+    try:
+        for skip in range(4):
+            keep()
+            assert L.nl_debug_device_full(skip, 1) == nl.NL_OK
+            run()
+        keep()
+        assert L.nl_debug_device_full(0, 2) == nl.NL_OK
+        with pytest.raises(nl.NLError):
+            run()
+    finally:
+        assert L.nl_debug_device_full(0, 0) == nl.NL_OK
+    run()
