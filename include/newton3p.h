@@ -494,6 +494,21 @@ nl_status nl_lusolve_grouped(int count, const int64_t* N, const void* const* LU,
 /* the hot path on its own, for tests and for callers with their own loop.  */
 /* ----------------------------------------------------------------------- */
 
+/* Workspaces.  Entry points that need one take it, in stream order, from a
+ * memory pool of the library's own on the current device (inside a stream
+ * capture: from the device's current pool, as cudaMallocAsync does).  Of what
+ * they release, the pool keeps up to 256 MB per device context across
+ * synchronisations, and nl_linsolve16 keeps up to 16 blocks of 64 bytes of pinned
+ * host memory, until the process ends or the device is reset: a call would
+ * otherwise spend longer on getting and returning memory than on a small
+ * solve.  An allocation of the library that finds the device full gives the
+ * kept memory back and tries again; an allocation made elsewhere in the
+ * process cannot, so a program that is short of device memory calls
+ * nl_release_workspaces: it gives back what the current context's pool keeps and no
+ * unfinished work uses (synchronise first to give back everything), and the
+ * pinned blocks.  Thread-safe; later calls take new memory.  Always NL_OK. */
+nl_status nl_release_workspaces(void);
+
 /* C <- C - A B on the tensor cores (tcgen05 kind::f16, binary32 accumulation
  * in tensor memory, one binary32 rounding per entry of C), the two-level
  * factorisation's inner update on its single-precision shadow (Section 2:
@@ -524,7 +539,7 @@ nl_status nl_k_residual(int64_t N, double c, const double* x, const void* u, int
  * passes of radix-2 Stockham transforms in shared memory, twiddles from
  * sincospi).  Results differ from nl_k_residual by rounding only (about
  * 1e-14 relative to max|x| at N = 4096).  Allocates its workspace (16 L
- * doubles) with cudaMallocAsync; the transform of h is recomputed per call
+ * doubles, stream-ordered); the transform of h is recomputed per call
  * (a solver handle keeps it). */
 nl_status nl_k_residual_fft(int64_t N, double c, const double* x, const void* u, int u_is_double,
                             double fnorm_scale, double* x_out, double* F, double* r, double* fnorm_dev,
@@ -577,8 +592,8 @@ nl_status nl_k_jacobian64(int64_t N, double c, const double* r, double* J64, int
  * With the tcgen05 update the entries of a row in columns N ..
  * round_up(N, 8) - 1 (inside ld) may be overwritten (the tensor-memory copies
  * store whole 16-byte units at the matrix's right edge).
- * Allocates its workspace (and the copy) with cudaMallocAsync on
- * `stream`.  Synchronises the stream. */
+ * Allocates its workspace (and the copy) on `stream`.  Synchronises the
+ * stream. */
 nl_status nl_lu16(int64_t N, void* A16, int64_t ld, int32_t* ipiv, int nb, int gemm, int path, int32_t* info_host,
                   void* stream);
 
@@ -590,8 +605,8 @@ nl_status nl_lu64(int64_t N, double* A, int64_t ld, int32_t* ipiv, int nb, int p
 
 /* b <- U^{-1} L^{-1} P b with the binary16 factors of nl_lu16 promoted to
  * single on the fly (eq. (2.16)), b single precision (device, N floats).
- * Allocates its workspace with cudaMallocAsync.  Returns NL_ETIMEOUT if a
- * bounded wait gave up. Synchronises the stream. */
+ * Allocates its workspace on `stream`.  Returns NL_ETIMEOUT if a bounded wait
+ * gave up.  Synchronises the stream. */
 nl_status nl_lusolve16(int64_t N, const void* LU16, int64_t ld, const int32_t* ipiv, float* b, void* stream);
 
 /* b <- U^{-1} L^{-1} P b in double with the factors of nl_lu64. */
@@ -601,8 +616,8 @@ nl_status nl_lusolve64(int64_t N, const double* LU, int64_t ld, const int32_t* i
  * the F32 column of Section 1.3): binary32 storage and arithmetic (the
  * updates as fused multiply-adds), always the interchanging path.  Layout,
  * ipiv and info as nl_lu16.  nb: 0 = 128, else a multiple of 16 in
- * [16, 128].  Allocates its workspace with cudaMallocAsync; synchronises
- * the stream. */
+ * [16, 128].  Allocates its workspace on `stream`; synchronises the
+ * stream. */
 nl_status nl_lu32(int64_t N, float* A, int64_t ld, int32_t* ipiv, int nb, int32_t* info_host, void* stream);
 
 /* b <- U^{-1} L^{-1} P b in single with the factors of nl_lu32 (device, N

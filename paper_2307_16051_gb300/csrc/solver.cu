@@ -1581,6 +1581,19 @@ struct PinnedWords {
 };
 }  // namespace
 
+nl_status nl_release_workspaces(void)
+{
+    const unsigned long long ctx = context_id();
+    ws_trim();
+    std::lock_guard<std::mutex> lock(PinnedWords::mu);
+    for (auto& k : PinnedWords::kept)
+        if (ctx && k.p && k.ctx == ctx) {
+            cudaFreeHost(k.p);
+            k.p = nullptr;
+        }
+    return NL_OK;
+}
+
 nl_status nl_linsolve16(int64_t N, const float* J32, int64_t ld32, const void* LU16, int64_t ld16, const int32_t* ipiv,
                         const float* b, float* u, double eta, int maxit, int solver, int m, double gtol, int gcycles,
                         int32_t* stats_host, double* relres_host, void* stream)

@@ -108,6 +108,7 @@ SIGNATURES = {
     "nl_last_error": (ctypes.c_char_p, []),
     "nl_version": (ctypes.c_char_p, []),
     "nl_kernel_timing": (_int, [ctypes.c_char_p, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_double)]),
+    "nl_release_workspaces": (_int, []),
     "nl_debug_fail_allocs": (_int, [_int]),
     "nl_debug_device_full": (_int, [_int, _int]),
     "nl_k_residual": (_int, [_i64, _dbl, _P, _P, _int, _dbl, _P, _P, _P, _P, _P]),
@@ -219,6 +220,11 @@ def kernel_timing(kernel_class=None):
     ms = ctypes.c_double(0.0)
     check(lib().nl_kernel_timing(kernel_class.encode() if kernel_class else None, ctypes.byref(cnt), ctypes.byref(ms)))
     return cnt.value, ms.value
+
+
+def release_workspaces():
+    """Give back the workspace memory that the library keeps between calls (nl_release_workspaces)."""
+    check(lib().nl_release_workspaces())
 
 
 class Solver:

@@ -209,3 +209,35 @@ def test_full_device_gives_kept_workspaces_back(call):
     finally:
         assert L.nl_debug_device_full(0, 0) == nl.NL_OK
     run()
+
+
+@pytest.mark.parametrize("N", [4096, 14000])
+def test_released_workspaces_leave_the_device(N):
+    """What a call's workspace leaves in the library's pool is at most 256 MB (N = 14000
+    takes 784 MB) and goes back to the device on request; the call gives the same
+    result after it."""
+    d, ld = torch.device("cuda:0"), (N + 63) // 64 * 64
+    J, A = (torch.empty((N, ld), device=d, dtype=t) for t in (torch.float32, torch.float16))
+    r, ip = torch.ones(N, device=d, dtype=torch.float64), torch.empty(N, device=d, dtype=torch.int32)
+
+    def run():
+        nl.k_jacobian(N, 0.9, r, J, ld, A, ld)
+        nl.lu16(N, A, ld, ip)
+        torch.cuda.synchronize()
+        return A.clone()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    first = run()
+    nl.release_workspaces()
+    before = free()
+    second = run()
+    del second
+    torch.cuda.empty_cache()
+    kept = before - free()
+    nl.release_workspaces()
+    assert 0 < kept <= (256 << 20) + (64 << 20) and free() >= before  # (64 MB: the pool's granularity)
+    third = run()
+    assert torch.equal(first.view(torch.int16), third.view(torch.int16))
