@@ -267,6 +267,10 @@ nl_status nl_debug_fail_allocs(int count);
  * been kept.  (0, 0) turns it off.  NL_EINVAL for negative arguments. */
 nl_status nl_debug_device_full(int skip, int count);
 
+/* Test hook: the next `count` creations of a look-ahead's second stream
+ * (nl_config.lu_lookahead, nl_lu16) fail.  0 turns it off.  NL_EINVAL for count < 0. */
+nl_status nl_debug_fail_streams(int count);
+
 /* ----------------------------------------------------------------------- */
 /* Batched solves: many independent instances of eq. (3.2), each with its   */
 /* own N and c, advanced together on the device.                            */
@@ -588,7 +592,8 @@ nl_status nl_k_jacobian64(int64_t N, double c, const double* r, double* J64, int
  * gemm are ignored, and *info_host is also set (to -1) after a binary16
  * overflow, returned as NL_ENUMERIC; 4 = as 0 with look-ahead
  * (nl_config.lu_lookahead; same result; the call creates and destroys a
- * second stream; path 0 does so too from N = 1024 with the tcgen05 update).
+ * second stream; path 0 does so too from N = 1024, and goes without if that
+ * fails).  With nb > 128 or the SIMT update there is no look-ahead.
  * With the tcgen05 update the entries of a row in columns N ..
  * round_up(N, 8) - 1 (inside ld) may be overwritten (the tensor-memory copies
  * store whole 16-byte units at the matrix's right edge).

@@ -44,6 +44,9 @@ cudaError_t trim_malloc(void** p, size_t bytes);
 // hook nl_debug_fail_allocs has allocations left to fail.
 cudaError_t dev_malloc(void** p, size_t bytes);
 
+// Whether the next stream creation fails on purpose (the test hook nl_debug_fail_streams).
+bool debug_fail_stream();
+
 // Stream-ordered workspace of a kernel-level entry point, released with
 // cudaFreeAsync: from the library's own memory pool on the current device,
 // which keeps up to kWsKeep bytes of released memory across synchronisations

@@ -69,6 +69,8 @@ struct LuWork {
 // The look-ahead's side stream and events for w (created at st's priority, or
 // re-created when the priority differs); lu_side_release destroys them.
 nl_status lu_side_prepare(LuWork* w, cudaStream_t st);
+// Whether the binary16 fast path uses them (its one-level form with the tensor-core update).
+inline bool lu_looks_ahead(int nb, int gemm) { return gemm == 2 && nb <= 128; }
 void lu_side_release(LuWork* w);
 size_t lu_work_bytes(int N, int nb, bool fp64);
 void lu_work_carve(void* base, int N, int nb, bool fp64, LuWork* w);

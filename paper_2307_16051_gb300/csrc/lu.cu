@@ -1884,6 +1884,10 @@ nl_status lu_side_prepare(LuWork* w, cudaStream_t st)
         NL_CUDA_OK(cudaStreamDestroy(w->side));
         w->side = nullptr;
     }
+    if (debug_fail_stream()) {
+        set_error("LU look-ahead: stream creation failed (test hook)");
+        return NL_ECUDA;
+    }
     NL_CUDA_OK(cudaStreamCreateWithPriority(&w->side, cudaStreamNonBlocking, prio));
     if (!w->ev_fork) NL_CUDA_OK(cudaEventCreateWithFlags(&w->ev_fork, cudaEventDisableTiming));
     for (auto& e : w->ev_join)
@@ -2142,7 +2146,7 @@ static nl_status lu_factor_impl(int N, S* A, int64_t ld, int* ipiv, int nb, int 
     // tiles are the same tcgen05 tiles as in one update, so the factors are bitwise the same.
     // Panels alternate U12^T buffers.
     constexpr int kLaTile = 128;  // the tcgen05 update's tile (M = N = 128)
-    const bool la = kHalf && fast && gemm == 2 && nb <= kLaTile && w.side && w.ut2 && w.ev_fork && w.ev_join[0] &&
+    const bool la = kHalf && fast && lu_looks_ahead(nb, gemm) && w.side && w.ut2 && w.ev_fork && w.ev_join[0] &&
                     w.ev_join[1];
     struct Join {
         const LuWork& w;

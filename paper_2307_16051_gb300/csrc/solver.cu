@@ -106,6 +106,9 @@ static bool take_one(std::atomic<int>& left)
         if (left.compare_exchange_weak(n, n - 1)) return true;
     return false;
 }
+// Test hook (nl_debug_fail_streams).
+static std::atomic<int> g_fail_streams{0};
+bool debug_fail_stream() { return take_one(g_fail_streams); }
 template <typename Alloc>
 static cudaError_t malloc_or_trim(Alloc alloc)
 {
@@ -609,6 +612,16 @@ nl_status nl_debug_fail_allocs(int count)
         return NL_EINVAL;
     }
     g_fail_allocs.store(count);
+    return NL_OK;
+}
+
+nl_status nl_debug_fail_streams(int count)
+{
+    if (count < 0) {
+        set_error("nl_debug_fail_streams: count < 0");
+        return NL_EINVAL;
+    }
+    g_fail_streams.store(count);
     return NL_OK;
 }
 
@@ -1282,8 +1295,8 @@ nl_status nl_k_jacobian64(int64_t N, double c, const double* r, double* J64, int
 
 // Factor with the no-interchange fast path, falling back to the interchanging
 // path (from a saved copy of A) when partial pivoting would swap rows.
-// Measured whole calls without / with look-ahead: N = 768 390 / 394 us, 1024 463 / 456,
-// 1536 611 / 581, 4096 1509 / 1330, 8192 3667 / 3340.
+// Measured whole calls without / with look-ahead: N = 512 162 / 176 us, 768 232 / 236,
+// 1024 300 / 295, 1536 448 / 416, 4096 1290 / 1045, 8192 3200 / 2820.
 constexpr int kLuSideMinN = 1024;
 template <typename S>
 static nl_status lu_entry(int64_t N, S* A, int64_t ld, int32_t* ipiv, int nb, int gemm, int path, int32_t* info_host,
@@ -1305,15 +1318,20 @@ static nl_status lu_entry(int64_t N, S* A, int64_t ld, int32_t* ipiv, int nb, in
         ~SideGuard() { lu_side_release(w); }
     } side_guard{&w};
     // the fast path with look-ahead (a side stream for the trailing updates): asked for, or where the
-    // updates it hides take longer than making the stream and its events (kLuSideMinN)
-    if (path == 4 || (path == 0 && w.stream == 0 && !fp64 && gemm == 2 && n >= kLuSideMinN)) {
+    // updates it hides take longer than making the stream and its events (kLuSideMinN); if it was not
+    // asked for, a failure to make them is no failure of the call
+    if (!fp64 && lu_looks_ahead(nb, gemm) && (path == 4 || (path == 0 && w.stream == 0 && n >= kLuSideMinN))) {
         const nl_status ps = lu_side_prepare(&w, st);
-        if (ps != NL_OK) {
+        if (ps != NL_OK && path == 4) {
             cudaFreeAsync(wk, st);
             return ps;
         }
-        path = 0;
+        if (ps != NL_OK) {
+            lu_side_release(&w);
+            cudaGetLastError();
+        }
     }
+    if (path == 4) path = 0;
     S* backup = (S*)((char*)wk + round_up(lw, 256));
     int iflag[2] = {0, 0};
     nl_status s = NL_OK;

@@ -111,6 +111,7 @@ SIGNATURES = {
     "nl_release_workspaces": (_int, []),
     "nl_debug_fail_allocs": (_int, [_int]),
     "nl_debug_device_full": (_int, [_int, _int]),
+    "nl_debug_fail_streams": (_int, [_int]),
     "nl_k_residual": (_int, [_i64, _dbl, _P, _P, _int, _dbl, _P, _P, _P, _P, _P]),
     "nl_k_jacobian": (_int, [_i64, _dbl, _P, _P, _i64, _P, _i64, _P]),
     "nl_k_residual_fft": (_int, [_i64, _dbl, _P, _P, _int, _dbl, _P, _P, _P, _P, _P]),

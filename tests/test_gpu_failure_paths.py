@@ -241,3 +241,38 @@ def test_released_workspaces_leave_the_device(N):
     assert 0 < kept <= (256 << 20) + (64 << 20) and free() >= before  # (64 MB: the pool's granularity)
     third = run()
     assert torch.equal(first.view(torch.int16), third.view(torch.int16))
+
+
+@pytest.mark.parametrize("N,nb,gemm,path,used", [(1100, 128, 2, 0, True), (1100, 64, 2, 0, True), (1000, 128, 2, 0, False),
+                                                 (1100, 256, 2, 0, False), (1100, 512, 2, 4, False),
+                                                 (1100, 96, 2, 0, False), (1100, 128, 1, 4, False),
+                                                 (300, 128, 2, 4, True)])
+def test_lu16_second_stream(N, nb, gemm, path, used):
+    """nl_lu16 makes a second stream only where its look-ahead runs (outer block
+    at most 128, tensor-core update, asked for or N >= 1024), and a failure to
+    make it fails the call only if the look-ahead was asked for (path 4)."""
+    d, ld, L = torch.device("cuda:0"), (N + 63) // 64 * 64, nl.lib()
+    J32, A = (torch.empty((N, ld), device=d, dtype=t) for t in (torch.float32, torch.float16))
+    r, ip = torch.ones(N, device=d, dtype=torch.float64), torch.empty(N, device=d, dtype=torch.int32)
+
+    def run(p):
+        nl.k_jacobian(N, 0.99, r, J32, ld, A, ld)
+        st = L.nl_lu16(N, A.data_ptr(), ld, ip.data_ptr(), nb, gemm, p, None, None)
+        torch.cuda.synchronize()
+        return st, A.clone()
+
+    st, ref = run(2)
+    assert st == nl.NL_OK
+    try:
+        assert L.nl_debug_fail_streams(1) == nl.NL_OK
+        st, got = run(path)
+        assert st == (nl.NL_ECUDA if used and path == 4 else nl.NL_OK)
+        if st == nl.NL_OK:
+            assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+        # was the hook used up?  path 4 with a one-level tensor-core update always asks for a stream
+        st = L.nl_lu16(128, A.data_ptr(), ld, ip.data_ptr(), 128, 2, 4, None, None)
+        assert (st == nl.NL_ECUDA) == (not used)
+    finally:
+        assert L.nl_debug_fail_streams(0) == nl.NL_OK
+    st, got = run(path)
+    assert st == nl.NL_OK and torch.equal(got.view(torch.int16), ref.view(torch.int16))
