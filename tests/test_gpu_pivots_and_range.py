@@ -8,7 +8,7 @@ from oracle import oracle as O
 from paper_2307_16051_gb300 import nl
 from paper_2307_16051_gb300 import workloads as W
 from tests.test_gpu_batch import lu_grouped
-from tests.test_gpu_kernels import T, dev
+from tests.test_gpu_kernels import T, _lu16_gpu, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -111,3 +111,54 @@ def test_div64_equals_ieee_division():
     got = out.cpu().numpy()
     bad = ~((got.view(np.uint64) == ref.view(np.uint64)) | (np.isnan(got) & np.isnan(ref)))
     assert not bad.any(), (bad.sum(), a[bad][:5], b[bad][:5], got[bad][:5], ref[bad][:5])
+
+
+@pytest.mark.parametrize("to", ["zero", "infinity"])
+@pytest.mark.parametrize("gemm", [1, 2])
+@pytest.mark.parametrize("N,k", [(300, 1), (300, 7), (300, 8), (300, 127), (300, 299), (1200, 200), (1200, 1199)])
+def test_lu16_pivot_leaves_binary16_by_rounding(N, k, gemm, to):
+    """A pivot that single precision holds and its rounding to binary16 does not:
+    -2^-34 (fl16(l u) - l u) becomes zero, 70000 becomes infinity, with only zeros
+    below it, so that every check of the unrounded value passes.  Every path
+    agrees bit for bit with the interchanging one, which names the zero pivot in
+    info and, with the SIMT update, is the oracle's.  In the first and later
+    columns of a block of eight and of a panel, in a ragged last panel, and in the
+    matrix's last pivot."""
+    nb = 128
+    k0 = k // nb * nb  # the first column of k's panel: no rounding to storage in between
+    A = 2.0 * np.eye(N) + W.random_matrix(N, 31) / (8.0 * N)
+    A[[k0, k], :] = A[:, [k0, k]] = 0.0
+    if to == "zero":
+        l, u, a = 2.0 ** -1 * (1 + 2.0 ** -10), 2.0 ** -13 * (1 + 2.0 ** -10), 2.0 ** -14 * (1 + 2.0 ** -9)
+        assert a - l * u == -(2.0 ** -34)
+        A[k0, k0], A[k, k0], A[k0, k], A[k, k] = 1.0, l, u, a
+    else:
+        A[k0, k0], A[k, k0], A[k0, k], A[k, k] = 2.0, 1.0, -20000.0, 60000.0
+    A16 = O.fl16(A)
+    assert all(A16[i, j] == A[i, j] for i in (k0, k) for j in (k0, k))
+    ref = _lu16_gpu(A16, nb, gemm, 1)
+    assert ref[2] == (k + 1 if to == "zero" else 0) and abs(ref[0][k, k]) == (0.0 if to == "zero" else np.inf)
+    for path in (0, 2, 4):
+        got = _lu16_gpu(A16, nb, gemm, path)
+        assert ref[2] == got[2] and np.array_equal(ref[1], got[1]), path
+        assert np.array_equal(ref[0].view(np.uint64), got[0].view(np.uint64)), path
+    if to == "zero" and gemm == 1 and N <= 300:
+        LUo, ipivo, infoo, _ = O.lu16_dev(A16, nb)
+        assert infoo == k + 1 and np.array_equal(ipivo, ref[1]) and np.array_equal(LUo, ref[0])
+
+
+@pytest.mark.parametrize("kind", [1, 2, 3, 5])
+def test_lu_grouped_pivot_leaves_binary16_by_rounding(kind):
+    """The same in the grouped factorisations: such a matrix is flagged, its
+    neighbours are not."""
+    mats = []
+    for N, k in ((200, 70), (200, 199), (64, 63), (130, 5), (96, -1)):
+        A = 2.0 * np.eye(N) + W.random_matrix(N, 31) / (8.0 * N)
+        if k >= 0:
+            k0 = k // 64 * 64
+            A[[k0, k], :] = A[:, [k0, k]] = 0.0
+            A[k0, k0], A[k, k0], A[k0, k] = 1.0, 2.0 ** -1 * (1 + 2.0 ** -10), 2.0 ** -13 * (1 + 2.0 ** -10)
+            A[k, k] = 2.0 ** -14 * (1 + 2.0 ** -9)
+        mats.append(O.fl16(A))
+    _, flags = lu_grouped(mats, 64, kind)
+    assert list(flags) == [1, 1, 1, 1, 0]
