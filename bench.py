@@ -21,6 +21,9 @@ large     : GMRES-IR16 at N = 32768, c = .99, autotuned panel width (median of
             three solves; LU TFLOP/s, residual / triangular-solve GB/s), the
             scaled variant, and FP64-LU Newton on the same GPU.
 
+The details are printed as lines "# key {...}"; the last line is one short JSON line
+with the metric (report).
+
 python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 """
 from __future__ import annotations
@@ -357,6 +360,39 @@ def bench_serving(nl, W, seconds, mode="IR16_GMRES", drain_s=120.0, max_inflight
            "admission": f"device-memory footprint (budget 96 GiB), {max_inflight} slots, smallest N first with a "
                         "250 ms starvation bound, high-priority streams for N <= 1024"}
     return out
+
+
+LINE_LIMIT = 1400  # characters: what keeps only the end of a run's output still has the whole last line
+
+
+def report(full):
+    """The lines to print for a run's results: every detail as "# key {...}", then one
+    short JSON line with the metric, its configuration, the end-to-end figure, clocks
+    and the summary of each further workload."""
+    def rounded(v):
+        if isinstance(v, float):
+            return float(f"{v:.7g}")
+        if isinstance(v, dict):
+            return {k: rounded(x) for k, x in v.items()}
+        return [rounded(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+    short = {k: full[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                  "higher_is_better", "scaling", "vs_baseline", "dtype", "data")}
+    short["config"] = {k: full["config"][k] for k in ("workload", "N", "mode", "l2", "parallelism")}
+    for key, keep in (("e2e", ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")),
+                      ("clocks", ("sm_mhz", "sm_max_mhz", "reasons")),
+                      ("roofline", ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic")),
+                      ("cpu_baseline", ("value", "unit", "cores", "kind"))):
+        if key in full:
+            short[key] = {k: full[key][k] for k in keep}
+    short["gpu_launches"] = full["gpu_launches"]
+    also = {"speedup_vs_fp64lu": full.get("speedup_vs_fp64lu")}
+    for key, name, field in (("batched", "batched_solves_per_s", "solves_per_s"), ("large", "large_ms", "ms_to_solution"),
+                             ("serving", "serving_p50_ms", "p50_ms"), ("serving", "serving_p99_ms", "p99_ms")):
+        also[name] = full.get(key, {}).get(field)
+    short["also"] = {k: v for k, v in also.items() if v is not None}
+    details = [f"# {k} {json.dumps(v)}" for k, v in full.items() if isinstance(v, dict)]
+    return details + [json.dumps(rounded(short), separators=(",", ":"))]
 
 
 def golden_x():
@@ -717,7 +753,8 @@ def main():
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = oracle_sample()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        for text in report(line):
+            print(text, flush=True)
     for s in solvers.values():
         s.close()
     pool.shutdown()
