@@ -33,46 +33,6 @@ __device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
 
 // ---------------------------------------------------------------- prepare --
 
-// Inverses of the diagonal blocks: Linv (unit lower) and Uinv (upper).
-template <typename S, typename T>
-__global__ void __launch_bounds__(T_) k_invdiag(int N, const S* __restrict__ LU, int64_t ld, T* __restrict__ dinv,
-                                                int nblk)
-{
-    __shared__ T A[T_][T_ + 1];
-    __shared__ T X[T_][T_ + 1];
-    const int b = blockIdx.x, r0 = b * T_, nb_ = min(T_, N - r0);
-    const int col = threadIdx.x;
-    for (int i = 0; i < T_; ++i) A[i][col] = (i < nb_ && col < nb_) ? (T)ld_elem(LU + (int64_t)(r0 + i) * ld + r0 + col) : T(0);
-    __syncthreads();
-    // L^{-1} e_col by forward substitution (unit diagonal)
-    for (int i = 0; i < T_; ++i) {
-        T x = T(0);
-        if (col < nb_ && i < nb_) {
-            if (i == col) x = T(1);
-            else if (i > col) {
-                T s = T(0);
-                for (int t = col; t < i; ++t) s = fma(A[i][t], X[t][col], s);
-                x = -s;
-            }
-        }
-        X[i][col] = x;
-    }
-    T* Linv = dinv + (int64_t)b * T_ * T_;
-    for (int i = 0; i < T_; ++i) Linv[i * T_ + col] = X[i][col];
-    // U^{-1} e_col by back substitution
-    for (int i = T_ - 1; i >= 0; --i) {
-        T x = T(0);
-        if (col < nb_ && i < nb_ && i <= col) {
-            T s = (i == col) ? T(1) : T(0);
-            for (int t = i + 1; t <= col; ++t) s = fma(-A[i][t], X[t][col], s);
-            x = s / A[i][i];
-        }
-        X[i][col] = x;
-    }
-    T* Uinv = dinv + (int64_t)(nblk + b) * T_ * T_;
-    for (int i = 0; i < T_; ++i) Uinv[i * T_ + col] = X[i][col];
-}
-
 // Final row permutation from the LAPACK-style interchanges:
 // perm[i] = original index of the entry that ends up at position i.
 __global__ void __launch_bounds__(1024) k_perm(int N, const int* __restrict__ ipiv, int* __restrict__ perm,
@@ -873,15 +833,15 @@ template <typename S, typename T>
 static nl_status prepare_impl(int N, const S* LU, int64_t ld, const int* ipiv, const TrsvWork& w, cudaStream_t st,
                               int* launches)
 {
-    constexpr bool fp64 = std::is_same<T, double>::value;
-    constexpr int TB = std::is_same<S, __half>::value ? T2 : T_;  // the block size of the solve that follows
+    constexpr bool half = std::is_same<S, __half>::value;
+    constexpr int TB = half ? T2 : T_;  // the block size of the solve that follows
     const int nblk = (int)cdiv(N, TB);
     static bool attr = false;
     if (!attr) {
-        if (set_max_dynamic_smem((const void*)k_perm) != NL_OK ||
-            set_max_dynamic_smem((const void*)k_invdiag_t<S, T, TB>) != NL_OK ||
-            set_max_dynamic_smem((const void*)k_invdiag16) != NL_OK)
-            return NL_ECUDA;
+        const void* inv;
+        if constexpr (half) inv = (const void*)k_invdiag16;
+        else inv = (const void*)k_invdiag_t<S, T, TB>;
+        if (set_max_dynamic_smem((const void*)k_perm) != NL_OK || set_max_dynamic_smem(inv) != NL_OK) return NL_ECUDA;
         attr = true;
     }
     if ((size_t)N * 4 > 200 * 1024) {
@@ -890,7 +850,7 @@ static nl_status prepare_impl(int N, const S* LU, int64_t ld, const int* ipiv, c
     }
     k_perm<<<1, 1024, (size_t)N * 4, st>>>(N, ipiv, w.perm, w.scan);
     prof_begin("k_invdiag", st);
-    if constexpr (std::is_same<S, __half>::value && !fp64)
+    if constexpr (half)
         k_invdiag16<<<2 * nblk, kInvThreads, kInvSmem, st>>>(N, LU, ld, (float*)w.dinv, nblk);
     else
         k_invdiag_t<S, T, TB><<<2 * nblk * (TB / kInvC), kInvC * kInvG, (size_t)TB * (TB + 1) * sizeof(T), st>>>(
