@@ -322,7 +322,9 @@ __global__ void __launch_bounds__(kTvThreads, 1) k_trsv_mb(int N, int nblk, cons
         }
         float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         const int cnt = LOWER ? b : nblk - 1 - b;
-        // tile (b, c): its entries are loaded two tiles ahead of their use, streamed once (not kept in the caches)
+        // tile (b, c): its entries are loaded one tile ahead of their use, streamed once (not kept in the caches).
+        // Two ahead needs more than the 128 registers (44 bytes spilled) and takes 96 us a pair of triangles
+        // at N = 4096 and 283 at 12000, one ahead 86 and 261.
         auto fetch = [&](int s, uint4 (&t)[4]) {
             const int c = LOWER ? s : nblk - 1 - s;
             tv_load_tile<true>(LU, ld, N, r0 + row4, c * T2 + 8 * cg, vecld, t);
@@ -335,21 +337,17 @@ __global__ void __launch_bounds__(kTvThreads, 1) k_trsv_mb(int N, int nblk, cons
             ys[s & 1][tv_pos(tid)] = y;
             return okp;
         };
-        uint4 t0[4], t1[4], t2[4];
+        uint4 t0[4], t1[4];
         if (cnt > 0) fetch(0, t0);
-        if (cnt > 1) fetch(1, t1);
         for (int s = 0; s < cnt; ++s) {
-            if (s + 2 < cnt) fetch(s + 2, t2);
+            if (s + 1 < cnt) fetch(s + 1, t1);
             if (__syncthreads_or(!poll(s))) {  // (the other buffer's readers are at most one tile behind)
                 if (tid == 0) atomicOr(err, (unsigned)ERR_TIMEOUT_TRSV);
                 return;
             }
             tv_dot_tile(t0, ys[s & 1] + tv_pos(8 * cg), p);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                t0[q] = t1[q];
-                t1[q] = t2[q];
-            }
+            for (int q = 0; q < 4; ++q) t0[q] = t1[q];
         }
         const float part = tv_reduce(p, lane);
         if (cnt == 0) __syncthreads();  // (acc was written by other threads; with tiles the loop's barriers passed)
@@ -980,9 +978,11 @@ static bool trsv_cluster_ok(int C)
 // -1 = none, else the largest available <= req); 0 = use the mailbox solve.
 // Automatic choice: the cluster's 16 SMs stream the whole factor, so beyond
 // 24 blocks (N > 3072) the mailbox solve over all SMs is faster (measured on
-// GB300 per solve pair: 49 vs 54 us at N = 2048, 102 vs 96 us at 4096, 297 vs
-// 192 us at 8192; mailbox alone 282 us at 12000, 377 us at 16384, where a row
-// half per thread with its inverse in shared memory took 600 and 980).
+// GB300 per solve pair, cluster / mailbox: 26 / 29 us at N = 1024, 49 / 49 at 2048, 77 / 69 at
+// 3072, 90 / 79 at 3584, 103 / 90 at 4096, 299 / 173 at 8192; mailbox alone 261 us at
+// 12000, 347 at 16384, where a row half per thread with its inverse in shared memory took
+// 600 and 980).  The line lies between the sizes where a mailbox that loaded two tiles
+// ahead lost and won (54 us at 2048, 96 at 4096); with one ahead it is level at 2048.
 constexpr int kClAutoMaxBlocks = 24;
 static int trsv_cluster_size(int nblk, int req)
 {
