@@ -232,6 +232,7 @@ def test_released_workspaces_leave_the_device(N):
 
     first = run()
     nl.release_workspaces()
+    torch.cuda.empty_cache()  # (what earlier tests left with torch's allocator)
     before = free()
     second = run()
     del second
