@@ -103,9 +103,10 @@ typedef struct {
                             the cluster size (any N); -1 = always the global-memory hand-off */
     int lu_stream;       /* [0 = auto] half-precision fast path: the diagonal block and the off-diagonal
                             solves of a panel in one launch, the solves streaming one block of eight
-                            columns behind the diagonal block, 64 rows per CTA while all CTAs fit on
-                            the GPU at once, else 128; 256 = the same with 256 rows per CTA (fewer
-                            SMs, for solves that share the GPU); -1 = two launches per panel.
+                            columns behind the diagonal block, 64 rows per CTA while the CTAs take at
+                            most half of the SMs, 96 while all fit on the GPU at once, else 128; 256 =
+                            the same with 256 rows per CTA (fewer SMs, for solves that share the GPU);
+                            -1 = two launches per panel.
                             Bitwise the same factors in every case */
     int ir_variant;      /* [0] IR correction (NL_IR16, and the IR part of NL_IR16_GMRES): 0 = on the
                             fly, d = U^{-1} L^{-1} r with the binary16 factors promoted to single
@@ -142,14 +143,15 @@ typedef struct {
                             convolution in double (nl_k_residual_fft: four launches, rounding-level
                             differences from the direct sum); -1 = the direct double sum over the Hankel
                             table (N^2 products); 0 = the FFT for N >= 4096, where it is the faster one
-                            (45 against 61 us at N = 4096, 70 us against 2.1 ms at N = 32768), the direct
+                            (31 against 52 us at N = 4096, 48 us against 2.1 ms at N = 32768), the direct
                             sum below */
     int lu_lookahead;    /* [0 = on] half-precision fast path with the tensor-core update (lu_nb <= 128):
                             after each panel only the trailing matrix's first 128-row and 128-column
                             tile strips (which hold the next panel) are updated on the solve's
                             stream (with lu_nb = 128 by the next panel's own launch), and the rest of
-                            the update runs on a second stream one priority step lower while the
-                            next panel is factored; the two are joined before the next update.
+                            the update runs on a second stream while the next panel is factored (one
+                            priority step lower where there is one: a stream of the lowest priority,
+                            the default, gets one of its own); the two are joined before the next update.
                             -1 = one update per panel.  Bitwise the same factors */
 } nl_config;
 
@@ -646,9 +648,9 @@ nl_status nl_k_gemv_residual(int64_t N, const float* A, int64_t ld, const float*
 
 /* out[i] = fl16(fl32(a[i] / b[i])) (device, n floats each): the multiplier
  * rounding l = fl16(a / u) of the half-precision LU (Section 2), as the LU
- * kernels compute it (a correctly rounded reciprocal, a product, and the IEEE
- * division wherever the product lies within a few single-precision units of a
- * binary16 rounding boundary).  For tests of that arithmetic. */
+ * kernels compute it (the product with an approximate reciprocal corrected by
+ * its exact remainder, which is the IEEE single quotient for a binary16 u; no
+ * division).  For tests of that arithmetic. */
 nl_status nl_k_div_round16(int64_t n, const float* a, const float* b, float* out, void* stream);
 
 /* out[i] = a[i] / b[i] (device, n doubles each), bit for bit the IEEE quotient,

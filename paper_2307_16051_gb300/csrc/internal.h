@@ -50,7 +50,8 @@ struct LuWork {
                               // barrier (+4, +5) and the streaming panel's two role counters (+8, +9)
     int* flag = nullptr;      // device int (info + 1): set when the no-interchange fast path failed
     void* stage = nullptr;    // diagonal-block factors staged for the off-diagonal solves (<= 256 KB)
-    unsigned long long* pub = nullptr;  // 128 x 128 {epoch, value} words: columns published by k_panel16
+    unsigned long long* pub = nullptr;  // 2 x 128 x 64 + 128 words {epoch, value}: U's rows and L's columns (two
+                                        // binary16 entries a word) and the pivots, published by k_panel16
     int stream = 0;           // binary16 fast path: 0 = one streaming launch per panel (64, 96 or 128 rows per
                               // CTA), 256 = the same with 256 rows per CTA, -1 = two launches
     float* p32 = nullptr;     // two-level LU (outer block > 128): single-precision shadow of the matrix, N x ldp32,
@@ -66,8 +67,8 @@ struct LuWork {
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};  // ev_join[q % 2]: the rest of update q
 };
-// The look-ahead's side stream and events for w (created at st's priority, or
-// re-created when the priority differs); lu_side_release destroys them.
+// The look-ahead's side stream and events for w (created one priority step below st's where there
+// is one, or re-created when that priority differs); lu_side_release destroys them.
 nl_status lu_side_prepare(LuWork* w, cudaStream_t st);
 // Whether the binary16 fast path uses them (its one-level form with the tensor-core update).
 inline bool lu_looks_ahead(int nb, int gemm) { return gemm == 2 && nb <= 128; }
